@@ -161,6 +161,14 @@ __device__ __forceinline__ void pdl_enter() {
   pdl_trigger();
 }
 
+// --------------------------------------------------------------------------- node scatter
+// One node's contribution of the atomic forms (plain form, allocation-free step) as one 16-byte
+// reduction instead of a scalar one per channel: the scatter is bound by the number of reductions L2
+// takes, not by their bytes.  Each component is added as its own float atomic.
+__device__ __forceinline__ void node_add(float4* node, float x, float y, float z, float w) {
+  atomicAdd(node, make_float4(x, y, z, w));
+}
+
 // --------------------------------------------------------------------------- scalar functions
 // One name per function for both precisions (the float overloads are the FP32 library calls).
 __device__ __forceinline__ float s_log(float a) { return logf(a); }

@@ -2096,24 +2096,26 @@ __global__ void k_plain_scatter(const ScenePar* __restrict__ dsp) {
           dp[a] = (float(k[a]) - stn.f[a]) * sp.dx;
         }
         const int nl = lin3<D>(nd, sp.n);
-        float* gp = reinterpret_cast<float*>(sp.grid + nl);
+        float q4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int a = 0; a < D; ++a) {
           float s = pm.mass * q.v[a];
 #pragma unroll
           for (int c = 0; c < D; ++c) s += G[a][c] * dp[c];
-          atomicAdd(gp + a, N * s);
+          q4[a] = N * s;
         }
-        atomicAdd(gp + (D == 2 ? 2 : 3), N * pm.mass);
+        q4[D] = N * pm.mass;
+        node_add(sp.grid + nl, q4[0], q4[1], q4[2], q4[3]);
         if constexpr (ADJ) {
-          float* gb = reinterpret_cast<float*>(sp.grid_b + nl);
+          float b4[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
           for (int a = 0; a < D; ++a) {
             float s = vb[a];
 #pragma unroll
             for (int c = 0; c < D; ++c) s += Dinv * Cb[a][c] * dp[c];
-            atomicAdd(gb + a, N * s);
+            b4[a] = N * s;
           }
+          node_add(sp.grid_b + nl, b4[0], b4[1], b4[2], 0.0f);
         }
       }
 }
