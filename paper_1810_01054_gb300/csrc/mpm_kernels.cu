@@ -2289,52 +2289,96 @@ template cudaError_t launch_plain_adjoint<2>(const ScenePar*, const ScenePar&, f
 template cudaError_t launch_plain_adjoint<3>(const ScenePar*, const ScenePar&, float*, cudaStream_t);
 
 // ============================================================================ pack / unpack
-// Storage slot p takes caller particle q = order[p] (q = p without an order).
-__global__ void k_pack(int dim, int N, int npad, const float* x, const float* v, const float* C, const float* F,
-                       float4* planes, int* status, const int* __restrict__ order) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+// Storage slot p takes caller particle q = order[p] (q = p without an order).  The caller's rows
+// ([N][W] floats, W = D or D * D) cross shared memory, where consecutive threads move consecutive
+// words of a row: with a thread moving its own rows every warp instruction touched 32 separate
+// sectors.  A block covers PACK_THREADS slots; rows are padded to an odd stride (no bank conflicts).
+constexpr int PACK_THREADS = 128;
+template <int W>
+struct PackRows {
+  static constexpr int STRIDE = W | 1;
+  float a[PACK_THREADS * STRIDE];
+  __device__ __forceinline__ void load(const float* src, const int* q, int n) {
+    for (int i = threadIdx.x; i < n * W; i += PACK_THREADS) a[(i / W) * STRIDE + i % W] = src[size_t(q[i / W]) * W + i % W];
+  }
+  __device__ __forceinline__ void store(float* dst, const int* q, int n) const {
+    for (int i = threadIdx.x; i < n * W; i += PACK_THREADS) dst[size_t(q[i / W]) * W + i % W] = a[(i / W) * STRIDE + i % W];
+  }
+  __device__ __forceinline__ float* row() { return a + threadIdx.x * STRIDE; }
+};
+template <int D>
+struct PackBlock {
+  PackRows<D> x, v;
+  PackRows<D * D> F, C;
+  int q[PACK_THREADS];
+};
+
+template <int D>
+__global__ void __launch_bounds__(PACK_THREADS) k_pack(int N, int npad, const float* x, const float* v, const float* C,
+                                                       const float* F, float4* planes, int* status,
+                                                       const int* __restrict__ order) {
+  __shared__ PackBlock<D> sm;
+  constexpr int S = Cfg<D>::S, DD = D * D;
+  const int base = blockIdx.x * PACK_THREADS, p = base + threadIdx.x;
+  const int n = N - base < PACK_THREADS ? N - base : PACK_THREADS;  // rows of this block (<= 0: padding only)
+  if (p < N) sm.q[threadIdx.x] = order ? order[p] : p;
+  __syncthreads();
+  sm.x.load(x, sm.q, n);
+  if (F) sm.F.load(F, sm.q, n);
+  if (v) sm.v.load(v, sm.q, n);
+  if (C) sm.C.load(C, sm.q, n);
+  __syncthreads();
   if (p >= npad) return;
-  const int S = dim == 2 ? 12 : 24, d2 = dim * dim;
-  float r[24];
+  float r[S];
   if (p < N) {
-    const size_t q = order ? size_t(order[p]) : size_t(p);
-    int o = 0;
-    for (int a = 0; a < dim; ++a) r[o++] = x[q * dim + a];
-    for (int a = 0; a < d2; ++a) r[o++] = F ? F[q * d2 + a] : ((a % (dim + 1)) == 0 ? 1.0f : 0.0f);
-    for (int a = 0; a < dim; ++a) r[o++] = v ? v[q * dim + a] : 0.0f;
-    for (int a = 0; a < d2; ++a) r[o++] = C ? C[q * d2 + a] : 0.0f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      r[a] = sm.x.row()[a];
+      r[D + DD + a] = v ? sm.v.row()[a] : 0.0f;
+    }
+#pragma unroll
+    for (int a = 0; a < DD; ++a) {
+      r[D + a] = F ? sm.F.row()[a] : ((a % (D + 1)) == 0 ? 1.0f : 0.0f);
+      r[2 * D + DD + a] = C ? sm.C.row()[a] : 0.0f;
+    }
+#pragma unroll
     for (int a = 0; a < S; ++a)
       if (!(r[a] == r[a]) || fabsf(r[a]) > 3.0e38f) set_status(status, -1);
   } else {
+#pragma unroll
     for (int a = 0; a < S; ++a) r[a] = 0.0f;
   }
-  for (int j = 0; j < S / 4; ++j) planes[size_t(j) * npad + p] = make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+  store_planes<D, Cfg<D>::PLANES>(planes, npad, p, r);
 }
 
 // Storage slot p goes to caller particle q = order[p] (q = p without an order).
-__global__ void k_unpack(int dim, int N, int npad, const float4* planes, float* x, float* v, float* C, float* F,
-                         const int* __restrict__ order) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= N) return;
-  const size_t qo = order ? size_t(order[p]) : size_t(p);
-  const int S = dim == 2 ? 12 : 24, d2 = dim * dim;
-  float r[24];
-  for (int j = 0; j < S / 4; ++j) {
-    float4 q = planes[size_t(j) * npad + p];
-    r[4 * j] = q.x;
-    r[4 * j + 1] = q.y;
-    r[4 * j + 2] = q.z;
-    r[4 * j + 3] = q.w;
+template <int D>
+__global__ void __launch_bounds__(PACK_THREADS) k_unpack(int N, int npad, const float4* planes, float* x, float* v,
+                                                         float* C, float* F, const int* __restrict__ order) {
+  __shared__ PackBlock<D> sm;
+  constexpr int S = Cfg<D>::S, DD = D * D;
+  const int base = blockIdx.x * PACK_THREADS, p = base + threadIdx.x;
+  const int n = N - base < PACK_THREADS ? N - base : PACK_THREADS;
+  if (p < N) {
+    sm.q[threadIdx.x] = order ? order[p] : p;
+    float r[S];
+    load_planes<D, Cfg<D>::PLANES>(planes, npad, p, r);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      sm.x.row()[a] = r[a];
+      sm.v.row()[a] = r[D + DD + a];
+    }
+#pragma unroll
+    for (int a = 0; a < DD; ++a) {
+      sm.F.row()[a] = r[D + a];
+      sm.C.row()[a] = r[2 * D + DD + a];
+    }
   }
-  int o = 0;
-  for (int a = 0; a < dim; ++a, ++o)
-    if (x) x[qo * dim + a] = r[o];
-  for (int a = 0; a < d2; ++a, ++o)
-    if (F) F[qo * d2 + a] = r[o];
-  for (int a = 0; a < dim; ++a, ++o)
-    if (v) v[qo * dim + a] = r[o];
-  for (int a = 0; a < d2; ++a, ++o)
-    if (C) C[qo * d2 + a] = r[o];
+  __syncthreads();
+  if (x) sm.x.store(x, sm.q, n);
+  if (F) sm.F.store(F, sm.q, n);
+  if (v) sm.v.store(v, sm.q, n);
+  if (C) sm.C.store(C, sm.q, n);
 }
 
 // Device-side choice of this step's scene records: scene s of the launch uses
@@ -2408,7 +2452,11 @@ cudaError_t launch_set_int(int* p, int v, cudaStream_t s) {
 cudaError_t launch_pack(int dim, int N, int npad, const float* x, const float* v, const float* C, const float* F,
                         float4* planes, int* status, const int* order, cudaStream_t s) {
   if (npad == 0) return cudaSuccess;
-  k_pack<<<(npad + 255) / 256, 256, 0, s>>>(dim, N, npad, x, v, C, F, planes, status, order);
+  const int blocks = (npad + PACK_THREADS - 1) / PACK_THREADS;
+  if (dim == 2)
+    k_pack<2><<<blocks, PACK_THREADS, 0, s>>>(N, npad, x, v, C, F, planes, status, order);
+  else
+    k_pack<3><<<blocks, PACK_THREADS, 0, s>>>(N, npad, x, v, C, F, planes, status, order);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -2416,7 +2464,11 @@ cudaError_t launch_pack(int dim, int N, int npad, const float* x, const float* v
 cudaError_t launch_unpack(int dim, int N, int npad, const float4* planes, float* x, float* v, float* C, float* F,
                           const int* order, cudaStream_t s) {
   if (N == 0) return cudaSuccess;
-  k_unpack<<<(N + 255) / 256, 256, 0, s>>>(dim, N, npad, planes, x, v, C, F, order);
+  const int blocks = (N + PACK_THREADS - 1) / PACK_THREADS;
+  if (dim == 2)
+    k_unpack<2><<<blocks, PACK_THREADS, 0, s>>>(N, npad, planes, x, v, C, F, order);
+  else
+    k_unpack<3><<<blocks, PACK_THREADS, 0, s>>>(N, npad, planes, x, v, C, F, order);
   count_launches(1);
   return cudaGetLastError();
 }
