@@ -67,6 +67,16 @@ mpm_status dalloc(T** p, size_t count, std::vector<void*>& list) {
   return MPM_OK;
 }
 
+// Tile bins of a batch of `tiles` tiles (at most BIN_TILES): control words and the appended lists;
+// the canonical lists take the place of `sorted`.
+mpm_status alloc_bins(BatchDev& b, int dim, int edge, int tiles, std::vector<void*>& list) {
+  const size_t room = size_t(tiles) * bin_cap(dim, edge), ctl = (bin_ctl_words(tiles) + 63) / 64 * 64;
+  CKS(dalloc(&b.bin_ctl, ctl + 2 * room, list));
+  b.bin_raw = b.bin_ctl + ctl;
+  b.sorted = b.bin_raw + room;
+  return MPM_OK;
+}
+
 int planes_of(int dim) { return dim == 2 ? Cfg<2>::PLANES : Cfg<3>::PLANES; }
 // Nodes of a tile's node block ((edge + 2)^dim).
 int block_nodes(int dim, int edge) {
@@ -287,8 +297,9 @@ mpm_status upload_map(mpm_scene* s, int which, const std::vector<int>& m, int ba
   const int phs[3][2] = {{PH_ROLL, -1}, {PH_RCM, PH_PREP}, {PH_REV, -1}};
   bool sel_changed = false;
   for (int ph : phs[which])
-    if (ph >= 0 && s->hsel[ph].base != base) {
+    if (ph >= 0 && (s->hsel[ph].base != base || s->hsel[ph].len != int(m.size()))) {
       s->hsel[ph].base = base;
+      s->hsel[ph].len = int(m.size());
       sel_changed = true;
     }
   if (!same) {
@@ -393,7 +404,7 @@ mpm_status enqueue_forward(mpm_scene* s, int ph, cudaStream_t st) {
   }
   const bool two = s->dim == 2;
   BatchDev& b = workspace(s, ph);
-  {
+  if (!b.bin_ctl) {  // with bins the step before (or the keys) left the tile lists and the record
     ProfScope p(c, st, MPM_K_SORT);
     CK(two ? launch_sort<2>(b, st, s->dsel + ph) : launch_sort<3>(b, st, s->dsel + ph));
     // keep the sort of this state for its reverse step (before P2G rewrites the tile lists in
@@ -403,7 +414,7 @@ mpm_status enqueue_forward(mpm_scene* s, int ph, cudaStream_t st) {
   }
   {
     ProfScope p(c, st, MPM_K_CTRL);
-    CK(ctrl_step_forward(s->hp, b.scenes, &b == &s->b2 ? s->ctrl2 : s->ctrl, st));
+    CK(ctrl_step_forward(s->hp, b.scenes, &b == &s->b2 ? s->ctrl2 : s->ctrl, st, b.bin_ctl));
   }
   {
     ProfScope p(c, st, MPM_K_P2G);
@@ -413,7 +424,8 @@ mpm_status enqueue_forward(mpm_scene* s, int ph, cudaStream_t st) {
   {
     ProfScope p(c, st, MPM_K_G2P);
     TuneScope t(s->tune, TK_G2P, st);
-    CK(two ? launch_g2p<2>(b, st) : launch_g2p<3>(b, st));
+    const SelectPar* next = b.bin_ctl ? s->dsel + ph : nullptr;
+    CK(two ? launch_g2p<2>(b, st, next) : launch_g2p<3>(b, st, next));
   }
   return MPM_OK;
 }
@@ -452,7 +464,7 @@ mpm_status enqueue_adjoint(mpm_scene* s, BatchDev& b, cudaStream_t st) {
     }
   } else {
     ProfScope p(c, st, MPM_K_CTRL);
-    CK(ctrl_step_backward(s->hp, s->cur, s->ctrl, st));
+    CK(ctrl_step_backward(s->hp, s->cur, s->ctrl, st, b.bin_ctl ? b.bin_ctl + 1 : nullptr));
   }
   return MPM_OK;
 }
@@ -461,19 +473,21 @@ mpm_status enqueue_adjoint(mpm_scene* s, BatchDev& b, cudaStream_t st) {
 mpm_status enqueue_reverse(mpm_scene* s, cudaStream_t st) {
   mpm_ctx* c = s->ctx;
   const bool two = s->dim == 2;
-  const bool stored = s->impl != MPM_IMPL_PLAIN && s->rcm_ws2;  // the recompute kept this state's sort
+  const bool bins = s->b.bin_ctl != nullptr;
+  const bool kept = s->impl != MPM_IMPL_PLAIN && s->rcm_ws2;
+  const bool stored = kept && !bins;  // the recompute kept this state's sort
   if (stored) {
     ProfScope p(c, st, MPM_K_SORT);
     CK(two ? launch_load_sort<2>(s->b, s->dsel + PH_REV, st) : launch_load_sort<3>(s->b, s->dsel + PH_REV, st));
   } else if (s->impl != MPM_IMPL_PLAIN) {
     ProfScope p(c, st, MPM_K_SORT);
-    CK(two ? launch_keys<2>(s->b, st, s->dsel + PH_REV) : launch_keys<3>(s->b, st, s->dsel + PH_REV));
+    CK(two ? launch_keys<2>(s->b, st, s->dsel + PH_REV, false) : launch_keys<3>(s->b, st, s->dsel + PH_REV, false));
   } else {
     CK(launch_select(s->dsel + PH_REV, 1, s->cur, st));
   }
-  if (!(stored && s->ctrl_store)) {  // else the recompute kept this state's controller input
+  if (!(kept && s->ctrl_store)) {  // else the recompute kept this state's controller input
     ProfScope p(c, st, MPM_K_CTRL);
-    CK(ctrl_step_forward(s->hp, s->cur, s->ctrl, st));
+    CK(ctrl_step_forward(s->hp, s->cur, s->ctrl, st, s->b.bin_ctl));
   }
   if (s->impl == MPM_IMPL_PLAIN) {
     {
@@ -485,7 +499,7 @@ mpm_status enqueue_reverse(mpm_scene* s, cudaStream_t st) {
     CK(ctrl_step_backward(s->hp, s->cur, s->ctrl, st));
     return MPM_OK;
   }
-  if (!stored) {
+  if (!stored && !bins) {
     ProfScope p(c, st, MPM_K_SORT);
     CK(two ? launch_sort<2>(s->b, st) : launch_sort<3>(s->b, st));
   }
@@ -513,12 +527,17 @@ mpm_status capture_reverse_branched(mpm_scene* s, int steps) {
   sets[1].active = bb.active;
   sets[1].n_active = bb.n_active;
   sets[1].sorted = bb.sorted;
+  sets[1].bin_ctl = bb.bin_ctl;
+  sets[1].bin_raw = bb.bin_raw;
   auto set = [&](int j) -> BatchDev& { return sets[j & 1]; };
   auto load = [&](int j, cudaStream_t on) -> mpm_status {
     const SelectPar* q = s->dsel + (j == 0 ? int(PH_REV) : (j & 1) ? int(SEL_LOAD_B) : int(SEL_LOAD_A));
     int* snap = j == 0 ? s->d_gstep : nullptr;  // the branch's selections step back j from there
     BatchDev& b = set(j);
-    CK(two ? launch_load_sort<2>(b, q, on, j, snap) : launch_load_sort<3>(b, q, on, j, snap));
+    if (b.bin_ctl)  // binned from the state itself
+      CK(two ? launch_keys<2>(b, on, q, false, j, snap) : launch_keys<3>(b, on, q, false, j, snap));
+    else
+      CK(two ? launch_load_sort<2>(b, q, on, j, snap) : launch_load_sort<3>(b, q, on, j, snap));
     return MPM_OK;
   };
   CKS(load(0, st));
@@ -545,7 +564,29 @@ mpm_status capture_reverse_branched(mpm_scene* s, int steps) {
 mpm_status enqueue_keys(mpm_scene* s, int ph, cudaStream_t st) {
   if (s->impl == MPM_IMPL_PLAIN) return MPM_OK;
   BatchDev& b = workspace(s, ph);
+  if (ph == PH_STEP) s->keys_stale = false;
   CK(s->dim == 2 ? launch_keys<2>(b, st, s->dsel + ph) : launch_keys<3>(b, st, s->dsel + ph));
+  return MPM_OK;
+}
+
+// What phase ph needs before its first step: the current state's keys, if a batch advanced the scene
+// since they were made; with bins a forward phase's first record (each step publishes its
+// successor's), and a reverse phase's empty lists.
+mpm_status begin_phase(mpm_scene* s, int ph, cudaStream_t st) {
+  if (s->impl == MPM_IMPL_PLAIN) return MPM_OK;
+  if (s->keys_stale && (ph == PH_STEP || ph == PH_ROLL)) CKS(enqueue_keys(s, PH_STEP, st));
+  BatchDev& b = workspace(s, ph);
+  if (!b.bin_ctl) return MPM_OK;
+  if (ph == PH_STEP || ph == PH_ROLL) {  // (a recompute's first record comes with its keys)
+    CK(launch_select(s->dsel + ph, 1, b.scenes, st, b.bin_ctl));
+  } else if (ph == PH_REV) {
+    CK(reset_bins(b, st));
+    if (load_branch(s)) {
+      BatchDev set_b = s->b;
+      set_b.bin_ctl = s->bB.bin_ctl;
+      CK(reset_bins(set_b, st));
+    }
+  }
   return MPM_OK;
 }
 
@@ -601,6 +642,7 @@ mpm_status capture(mpm_scene* s, int ph, int steps, Graph* g) {
 mpm_status run_phase(mpm_scene* s, int ph, int count, cudaStream_t graph_stream = nullptr) {
   mpm_ctx* c = s->ctx;
   cudaStream_t gs = graph_stream ? graph_stream : c->stream;
+  if (count > 0) CKS(begin_phase(s, ph, gs));
   // steps that still try launch shapes run one at a time, launched directly and timed; graphs are
   // captured only once the shapes of the phase's kernels are settled
   for (; count > 0 && tune_wants(s, ph); --count) CKS(tune_step(s, ph));
@@ -672,7 +714,7 @@ mpm_status ensure_ws2_parts(mpm_scene* s) {
   b = s->b;  // scene tables, offsets and launch shapes; the tile arrays below are its own
   const int nt = s->hp.n_tiles, NB = block_nodes(s->dim, s->b.tile_edge);
   std::vector<void*>& L = s->ws2_allocs;
-  CKS(dalloc(&s->cur2, 1, L));
+  CKS(dalloc(&s->cur2, 2, L));
   CKS(dalloc(&s->key2, s->npad, L));
   CKS(dalloc(&s->act2, std::max(1, s->G), L));
   CKS(dalloc(&s->grid2, s->n_nodes, L));
@@ -685,7 +727,11 @@ mpm_status ensure_ws2_parts(mpm_scene* s) {
   CKS(dalloc(&b.block_sums, 2 * ((nt + 2047) / 2048) + 2, L));
   CKS(dalloc(&b.work, 4, L));
   CK(cudaMemsetAsync(b.work, 0, sizeof(uint32_t) * 4, s->ctx->stream));
-  CKS(dalloc(&b.sorted, s->npad, L));
+  const bool bins = s->b.bin_ctl != nullptr;
+  if (bins)
+    CKS(alloc_bins(b, s->dim, s->b.tile_edge, nt, L));
+  else
+    CKS(dalloc(&b.sorted, s->npad, L));
   CKS(dalloc(&b.partial, size_t(nt) * NB, L));
   CKS(dalloc(&b.partial_b, size_t(nt) * NB, L));
   b.scenes = s->cur2;
@@ -705,7 +751,7 @@ mpm_status ensure_ws2_parts(mpm_scene* s) {
   if (s->ctrl_branch) {  // buffer set B of the reverse steps whose sorts load on a branch
     BatchDev& bb = s->bB;  // only its sort arrays and record are used
     bb = BatchDev{};
-    CKS(dalloc(&s->curB, 1, L));
+    CKS(dalloc(&s->curB, 2, L));
     CKS(dalloc(&s->keyB, s->npad, L));
     CKS(dalloc(&s->actB, std::max(1, s->G), L));
     CKS(dalloc(&s->d_gstep, 1, L));
@@ -713,7 +759,10 @@ mpm_status ensure_ws2_parts(mpm_scene* s) {
     CKS(dalloc(&bb.tile_slot, nt, L));
     CKS(dalloc(&bb.active, nt, L));
     CKS(dalloc(&bb.n_active, 1, L));
-    CKS(dalloc(&bb.sorted, s->npad, L));
+    if (bins)
+      CKS(alloc_bins(bb, s->dim, s->b.tile_edge, nt, L));
+    else
+      CKS(dalloc(&bb.sorted, s->npad, L));
     bb.scenes = s->curB;
     CK(cudaMemsetAsync(s->actB, 0, sizeof(float) * std::max(1, s->G), st));
     for (cudaEvent_t& e : s->ev_load) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -802,6 +851,7 @@ mpm_status rollout_records(mpm_scene* s, int T, int k, size_t budget, bool copy_
 // read the state, their inputs.
 size_t overlap_store_bytes(const mpm_scene* s, int k) {
   const size_t ctrl = ctrl_reads_state(s->ctrl) ? 2 * size_t(k) * CTRL_SLOT_FLOATS * sizeof(float) : 0;
+  if (s->b.bin_ctl) return ctrl;  // the reverse steps bin their states again
   return 2 * size_t(k) * sort_slot_words(s->npad, s->hp.n_tiles) * sizeof(uint32_t) + ctrl;
 }
 
@@ -960,7 +1010,7 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
       s->seg2 = segs;
     }
     // the sorts of every recomputed state, by segment parity (each reverse step loads its own)
-    if (!s->sort_store)
+    if (!s->sort_store && !s->b.bin_ctl)
       CKS(dalloc(&s->sort_store, (store_bytes - ctrl_bytes) / sizeof(uint32_t), s->roll_allocs));
     if (keep_ctrl && !s->ctrl_store) CKS(dalloc(&s->ctrl_store, ctrl_bytes / sizeof(float), s->roll_allocs));
   }
@@ -1083,7 +1133,7 @@ mpm_status recompute_segment(mpm_scene* s, int sg, cudaStream_t st) {
   CK(launch_set_int(s->d_step, n0 + sg * k, st));
   CKS(run_phase(s, PH_PREP, 1, st));  // bin keys of the checkpoint the recompute starts from
   if (L > 1) CKS(run_phase(s, PH_RCM, L - 1, st));
-  if (s->rcm_ws2) {
+  if (s->rcm_ws2 && !s->b.bin_ctl) {
     // the segment's last state has its keys (from the last recompute step, or the checkpoint's
     // own for L = 1) but no scatter yet: sort it into its slot and leave the counters clear
     BatchDev& b2 = workspace(s, PH_RCM);
@@ -1093,10 +1143,11 @@ mpm_status recompute_segment(mpm_scene* s, int sg, cudaStream_t st) {
     CK(two ? launch_store_sort<2>(b2, slot, st) : launch_store_sort<3>(b2, slot, st));
     CK(cudaMemsetAsync(b2.tile_count, 0, sizeof(uint32_t) * size_t(b2.total_tiles), st));
     CK(cudaMemsetAsync(b2.tile_fill, 0, sizeof(uint32_t) * size_t(b2.total_tiles), st));
-    if (s->ctrl_store) {  // the last state's controller input and actuation into its slot
-      CK(launch_select(s->dsel + PH_RCM, 1, s->cur2, st));
-      CK(ctrl_step_forward(s->hp, s->cur2, s->ctrl2, st));
-    }
+  }
+  if (s->rcm_ws2 && s->ctrl_store) {  // the last state's controller input and actuation into its slot
+    const uint32_t* flip = workspace(s, PH_RCM).bin_ctl;
+    CK(launch_select(s->dsel + PH_RCM, 1, s->cur2, st, flip));
+    CK(ctrl_step_forward(s->hp, s->cur2, s->ctrl2, st, flip));
   }
   return MPM_OK;
 }
@@ -1580,7 +1631,7 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   ALLOC(s->d_step, 1);
   ALLOC(s->d_bstep, 1);
   ALLOC(s->d_status, 1);
-  ALLOC(s->cur, 1);
+  ALLOC(s->cur, 2);
   ALLOC(s->dsel, SEL_COUNT);
   p.planes = p.planes_out = s->state;
   p.key = key;
@@ -1638,7 +1689,12 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   ALLOC(b.n_active, 1);
   ALLOC(b.block_sums, 2 * ((p.n_tiles + 2047) / 2048) + 2);
   ALLOC(b.work, 4);
-  ALLOC(b.sorted, s->npad);
+  if (s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES) {
+    TRY(alloc_bins(b, dim, edge, p.n_tiles, s->allocs));
+    b.rec_flip = 1;
+  } else {
+    ALLOC(b.sorted, s->npad);
+  }
   if (s->impl == MPM_IMPL_TILED) {
     ALLOC(b.partial, size_t(p.n_tiles) * NB);
     ALLOC(b.partial_b, size_t(p.n_tiles) * NB);

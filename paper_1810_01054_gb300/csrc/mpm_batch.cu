@@ -48,6 +48,7 @@ struct SubBatch {
   TuneState tune;
   long long key_particles = -1, key_tiles = -1;
   int trial_wait = 0;  // steps of this key left before its trials start (0: none pending)
+  uint32_t *bin_ctl = nullptr, *bin_raw = nullptr;  // tile bins, for compositions of at most BIN_TILES tiles
   float4 *partial = nullptr, *partial_b = nullptr;  // node blocks (each half its own: they run at once)
   int cap_edge = 0;  // tile edge the node-block arrays are sized for
 };
@@ -90,6 +91,8 @@ void free_sub(SubBatch& sb) {
   dfree(sb.b.block_sums);
   dfree(sb.b.work);
   dfree(sb.b.sorted);
+  dfree(sb.bin_ctl);
+  dfree(sb.bin_raw);
   dfree(sb.b.gpartial);
   dfree(sb.partial);
   dfree(sb.partial_b);
@@ -143,7 +146,11 @@ mpm_status grow(mpm_batch* B, SubBatch& sb, int n_scenes, int tiles, int particl
   CK(cudaMalloc(&sb.b.block_sums, sizeof(uint32_t) * (2 * ((tl + 2047) / 2048) + 2)));
   CK(cudaMalloc(&sb.b.work, sizeof(uint32_t) * 4));
   CK(cudaMemsetAsync(sb.b.work, 0, sizeof(uint32_t) * 4, B->ctx->stream));
-  CK(cudaMalloc(&sb.b.sorted, sizeof(uint32_t) * pc));
+  const int bt = std::min(tl, BIN_TILES);
+  const size_t room = size_t(bt) * bin_cap(B->dim, B->edge);
+  CK(cudaMalloc(&sb.bin_ctl, sizeof(uint32_t) * bin_ctl_words(bt)));
+  CK(cudaMalloc(&sb.bin_raw, sizeof(uint32_t) * room));
+  CK(cudaMalloc(&sb.b.sorted, sizeof(uint32_t) * std::max(size_t(pc), room)));
   CK(cudaMalloc(&sb.b.gpartial, sizeof(float) * size_t(tl) * MAX_GROUPS));
   CK(cudaMemsetAsync(sb.b.tile_count, 0, sizeof(uint32_t) * tl, B->ctx->stream));
   CK(cudaMemsetAsync(sb.b.tile_fill, 0, sizeof(uint32_t) * tl, B->ctx->stream));
@@ -204,6 +211,8 @@ mpm_status compose(mpm_batch* B, SubBatch& sb) {
   }
   CK(cudaMemcpy(sb.pbase, pb.data(), sizeof(int) * pb.size(), cudaMemcpyHostToDevice));
   if (tiles > 0) CK(cudaMemcpy(sb.b.tile_scene, tscene.data(), sizeof(int) * tiles, cudaMemcpyHostToDevice));
+  sb.b.bin_ctl = tiles <= BIN_TILES ? sb.bin_ctl : nullptr;
+  sb.b.bin_raw = sb.bin_raw;
   sb.b.scenes = sb.cur;
   sb.b.tile_edge = B->edge;
   sb.b.n_scenes = int(sb.members.size());
@@ -279,7 +288,8 @@ mpm_status reverse_step(mpm_batch* B, cudaStream_t st) {
   const int n = int(sb.members.size());
   if (n == 0) return MPM_OK;
   CK(launch_select(sb.dsel, n, sb.cur, st));
-  CK(launch_keys<D>(sb.b, st));
+  CK(launch_keys<D>(sb.b, st, nullptr, sb.need_keys));
+  sb.need_keys = false;
   for (int m = 0; m < n; ++m) {
     mpm_scene* s = B->slots[sb.members[m]].s;
     if (ctrl_reads_state(s->ctrl)) CK(ctrl_step_forward(s->hp, sb.cur + m, s->ctrl, st));
@@ -497,6 +507,7 @@ mpm_status mpm_batch_admit(mpm_batch* B, mpm_scene* s, int n_steps, int want_gra
   B->used += need;
   B->dirty = true;
   s->batch_refs += 1;
+  s->keys_stale = true;
   *slot = idx;
   return MPM_OK;
 }

@@ -27,9 +27,9 @@ int reduction_rows(int N) { return (N + RED_ROW - 1) / RED_ROW; }
 template <int CH>
 __global__ void __launch_bounds__(256) k_group_rows(const ScenePar* __restrict__ dsp, float* __restrict__ rows,
                                                     int mode, const int* __restrict__ perm,
-                                                    const int* __restrict__ pgroup) {
+                                                    const int* __restrict__ pgroup, const uint32_t* flip) {
   pdl_enter();
-  const ScenePar& sp = *dsp;
+  const ScenePar& sp = dsp[flip ? *flip : 0u];
   __shared__ float wacc[RED_WARPS][MAX_GROUPS][CH];
   __shared__ float wbody[RED_WARPS][CH];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -205,9 +205,9 @@ __device__ __forceinline__ void mlp_layers(const CtrlPar& c, const float* P, con
 // MLP controller of step n = *step_ctr (the sinusoid forms are evaluated by the record
 // selection): group centroids from the partial rows, then the three tanh layers -> sp.act.
 __global__ void __launch_bounds__(1024) k_ctrl_forward(const ScenePar* __restrict__ dsp, CtrlPar c, const float* rows,
-                                                       int n_rows) {
+                                                       int n_rows, const uint32_t* flip) {
   pdl_enter();
-  const ScenePar& sp = *dsp;
+  const ScenePar& sp = dsp[flip ? *flip : 0u];
   __shared__ float red[MAX_GROUPS * 3 + 3];
   __shared__ float z[MAX_GROUPS * 3], h1[MAX_HIDDEN], h2[MAX_HIDDEN];
   const int G = c.G, tid = threadIdx.x;
@@ -230,9 +230,9 @@ __global__ void __launch_bounds__(1024) k_ctrl_forward(const ScenePar* __restric
 // group means of x and v (partial rows of x, then of v), a = scale * tanh(W z + b) -> sp.act; z is
 // kept for the reverse step (in the record's controller slot, else in c.centroid).
 __global__ void __launch_bounds__(1024) k_ctrl_forward_com(const ScenePar* __restrict__ dsp, CtrlPar c,
-                                                           const float* rows, int n_rows) {
+                                                           const float* rows, int n_rows, const uint32_t* flip) {
   pdl_enter();
-  const ScenePar& sp = *dsp;
+  const ScenePar& sp = dsp[flip ? *flip : 0u];
   __shared__ float rx[MAX_GROUPS * 3 + 3], rv[MAX_GROUPS * 3 + 3];
   __shared__ float z[3 * (1 + 2 * MAX_GROUPS)];
   const int G = c.G, dim = c.dim, tid = threadIdx.x, Z = dim * (1 + 2 * G);
@@ -415,9 +415,10 @@ __device__ void ctrl_backward_body(const ScenePar& sp, const CtrlPar& c) {
 }
 
 template <bool STATE>
-__global__ void __launch_bounds__(1024) k_ctrl_backward(const ScenePar* __restrict__ dsp, CtrlPar c) {
+__global__ void __launch_bounds__(1024) k_ctrl_backward(const ScenePar* __restrict__ dsp, CtrlPar c,
+                                                        const uint32_t* flip) {
   pdl_enter();
-  ctrl_backward_body<STATE>(*dsp, c);
+  ctrl_backward_body<STATE>(dsp[flip ? *flip : 0u], c);
 }
 
 // Reverse of a form that reads no state for one step of a scene alone: the adjoint gather of the
@@ -443,9 +444,9 @@ __global__ void __launch_bounds__(1024) k_ctrl_backward_multi(const ScenePar* __
 // x (and, for the closed-loop form, v) adjoint of the controller input: the MLP's centroids
 // (z_g = c_g - c_body, so the body term), or the closed-loop form's group means of x and v.
 template <int D>
-__global__ void k_ctrl_scatter_x(const ScenePar* __restrict__ dsp, CtrlPar c) {
+__global__ void k_ctrl_scatter_x(const ScenePar* __restrict__ dsp, CtrlPar c, const uint32_t* flip) {
   pdl_enter();
-  const ScenePar& sp = *dsp;
+  const ScenePar& sp = dsp[flip ? *flip : 0u];
   __shared__ float coef[MAX_GROUPS * 3], coefv[MAX_GROUPS * 3], body[3];
   const int G = c.G;
   const bool com = c.type == 4;
@@ -485,7 +486,8 @@ __global__ void k_ctrl_scatter_x(const ScenePar* __restrict__ dsp, CtrlPar c) {
 
 // Controller forward for one step: the forms that read the state (MLP on centroids, closed loop on
 // group means of x and v): group rows, then the controller.
-cudaError_t ctrl_step_forward(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s) {
+cudaError_t ctrl_step_forward(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s,
+                              const uint32_t* flip) {
   if (!ctrl_reads_state(c)) return cudaSuccess;
   const int rows = reduction_rows(sp.N);
   const bool com = c.type == 4;
@@ -493,18 +495,18 @@ cudaError_t ctrl_step_forward(const ScenePar& sp, const ScenePar* dsp, const Ctr
   if (rows > 0) {
     float* vrows = c.partials + size_t(rows) * RED_STRIDE;
     if (sp.dim == 2) {
-      launch_pdl(k_group_rows<2>, dim3(rows), dim3(256), 0, s, dsp, c.partials, 0, c.perm, c.pgroup);
-      if (com) launch_pdl(k_group_rows<2>, dim3(rows), dim3(256), 0, s, dsp, vrows, 2, c.perm, c.pgroup);
+      launch_pdl(k_group_rows<2>, dim3(rows), dim3(256), 0, s, dsp, c.partials, 0, c.perm, c.pgroup, flip);
+      if (com) launch_pdl(k_group_rows<2>, dim3(rows), dim3(256), 0, s, dsp, vrows, 2, c.perm, c.pgroup, flip);
     } else {
-      launch_pdl(k_group_rows<3>, dim3(rows), dim3(256), 0, s, dsp, c.partials, 0, c.perm, c.pgroup);
-      if (com) launch_pdl(k_group_rows<3>, dim3(rows), dim3(256), 0, s, dsp, vrows, 2, c.perm, c.pgroup);
+      launch_pdl(k_group_rows<3>, dim3(rows), dim3(256), 0, s, dsp, c.partials, 0, c.perm, c.pgroup, flip);
+      if (com) launch_pdl(k_group_rows<3>, dim3(rows), dim3(256), 0, s, dsp, vrows, 2, c.perm, c.pgroup, flip);
     }
     n += com ? 2 : 1;
   }
   if (com)
-    launch_pdl(k_ctrl_forward_com, dim3(1), dim3(1024), 0, s, dsp, c, c.partials, rows);
+    launch_pdl(k_ctrl_forward_com, dim3(1), dim3(1024), 0, s, dsp, c, c.partials, rows, flip);
   else
-    launch_pdl(k_ctrl_forward, dim3(1), dim3(1024), 0, s, dsp, c, c.partials, rows);
+    launch_pdl(k_ctrl_forward, dim3(1), dim3(1024), 0, s, dsp, c, c.partials, rows, flip);
   count_launches(n + 1);
   return cudaGetLastError();
 }
@@ -528,25 +530,28 @@ cudaError_t ctrl_backward_batched(const ScenePar* cur, const CtrlPar* cs, int n,
 cudaError_t ctrl_scatter_x(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s) {
   if (!ctrl_reads_state(c) || sp.N == 0) return cudaSuccess;
   if (sp.dim == 2)
-    launch_pdl(k_ctrl_scatter_x<2>, dim3((sp.N + 255) / 256), dim3(256), 0, s, dsp, c);
+    launch_pdl(k_ctrl_scatter_x<2>, dim3((sp.N + 255) / 256), dim3(256), 0, s, dsp, c,
+               static_cast<const uint32_t*>(nullptr));
   else
-    launch_pdl(k_ctrl_scatter_x<3>, dim3((sp.N + 255) / 256), dim3(256), 0, s, dsp, c);
+    launch_pdl(k_ctrl_scatter_x<3>, dim3((sp.N + 255) / 256), dim3(256), 0, s, dsp, c,
+               static_cast<const uint32_t*>(nullptr));
   count_launches(1);
   return cudaGetLastError();
 }
 
 // Controller backward for one reverse step: group sums of (K), parameter adjoint, and (MLP) the
 // centroid adjoint added to dL/dx of state n.  Rewinds the scene's step counter.
-cudaError_t ctrl_step_backward(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s) {
+cudaError_t ctrl_step_backward(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s,
+                               const uint32_t* flip) {
   if (ctrl_reads_state(c))
-    launch_pdl(k_ctrl_backward<true>, dim3(1), dim3(1024), 0, s, dsp, c);
+    launch_pdl(k_ctrl_backward<true>, dim3(1), dim3(1024), 0, s, dsp, c, flip);
   else
-    launch_pdl(k_ctrl_backward<false>, dim3(1), dim3(1024), 0, s, dsp, c);
+    launch_pdl(k_ctrl_backward<false>, dim3(1), dim3(1024), 0, s, dsp, c, flip);
   if (ctrl_reads_state(c) && sp.N > 0) {
     if (sp.dim == 2)
-      launch_pdl(k_ctrl_scatter_x<2>, dim3((sp.N + 255) / 256), dim3(256), 0, s, dsp, c);
+      launch_pdl(k_ctrl_scatter_x<2>, dim3((sp.N + 255) / 256), dim3(256), 0, s, dsp, c, flip);
     else
-      launch_pdl(k_ctrl_scatter_x<3>, dim3((sp.N + 255) / 256), dim3(256), 0, s, dsp, c);
+      launch_pdl(k_ctrl_scatter_x<3>, dim3((sp.N + 255) / 256), dim3(256), 0, s, dsp, c, flip);
   }
   count_launches(1 + ((ctrl_reads_state(c) && sp.N > 0) ? 1 : 0));
   return cudaGetLastError();

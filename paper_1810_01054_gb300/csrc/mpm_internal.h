@@ -105,7 +105,7 @@ inline size_t sort_slot_words(int npad, int nt) { return 2 * size_t(npad) + 3 * 
 struct SelectPar {
   const ScenePar* table;  // the scene's record table for the running phase
   const int* map;         // record index of step n at map[n - base]; NULL = record 0
-  int base;
+  int base, len;          // steps base .. base + len - 1 are mapped (a selection beyond publishes nothing)
   const int* ctr;         // step counter n
   int tile_base, pbase;   // batch offsets of the scene
   int ctrl_type, G;       // sinusoid and table controllers are evaluated by the selection
@@ -146,7 +146,25 @@ struct BatchDev {
   uint32_t* block_sums; // scan scratch
   uint32_t* work;       // [4] tile counters of the dynamically scheduled P2G and adjoint gather and
                         // their CTAs-done tickets; zero between launches
-  uint32_t* sorted;     // [total_particles] scene-local particle ids, tile-major, canonical
+  uint32_t* sorted;     // [total_particles] scene-local particle ids, tile-major, canonical;
+                        // with tile bins [total_tiles * cap], tile t's list at t * cap
+  // Tile bins (batches of at most BIN_TILES tiles; NULL: the sort's arrays above): every tile owns
+  // room for as many entries as its kernels stage, and the kernel that moves a particle (G2P; the
+  // keys kernel) appends it to its tile's list, so a step has no sort: P2G starts from the lists.
+  // bin_raw holds the appended entries (cell in tile << 26 | id), which P2G puts in canonical order
+  // into `sorted`.  bin_ctl holds the counts and the mask of non-empty tiles twice, by parity: the
+  // kernels of a step read one while the next step's lists are counted in the other.
+  //   word 0  parity P2G reads (written by the appending kernel)
+  //   word 1  parity the gathers read (written by P2G); the appending kernel fills the other one
+  //   words BIN_MASK .., two masks of BIN_WORDS; then two counts of total_tiles
+  // P2G clears the other parity's mask and counts; a phase starts from all zeros (launch_keys).
+  // The line at BIN_TILES: the lists take 8 or 16 KB a tile and set (their room cannot overflow before
+  // the tile's kernels refuse it), 64 MB at most, and a tile mask of 64 words is read by every CTA;
+  // beyond it a step is long enough that the sort's launches (19 of 143 us at one million particles)
+  // matter less.  Steps with bins against the sort: 1,024 particles (2D) 13.3 -> 10.9 us, the 31k
+  // walker 16.9 -> 13.9 us.
+  uint32_t *bin_ctl, *bin_raw;
+  int rec_flip;         // scenes[] holds one scene's records by parity (a scene alone, with bins)
   float4* partial;      // [total_tiles * BLOCK_NODES] node blocks of P2G
   float4* partial_b;    // [total_tiles * BLOCK_NODES] node blocks of the adjoint scatter
   float* gpartial;      // [total_tiles * MAX_GROUPS] per active tile group sums of dL/da
@@ -161,6 +179,15 @@ struct BatchDev {
   int* rewind_rows;
 };
 
+constexpr int BIN_TILES = 2048;                 // most tiles a batch with bins holds
+constexpr int BIN_WORDS = BIN_TILES / 32;       // words of a tile mask
+constexpr int BIN_MASK = 4;                     // first mask word in bin_ctl
+constexpr int BIN_COUNT = BIN_MASK + 2 * BIN_WORDS;  // first count word
+inline size_t bin_ctl_words(int tiles) { return BIN_COUNT + 2 * size_t(tiles); }
+// Most entries of a tile's list: what its kernels stage (Tile<D, TB>::SORT_CAP).
+inline int bin_cap(int dim, int edge) { return dim == 2 && edge != 8 ? Tile<2, 4>::SORT_CAP : Tile<2, 8>::SORT_CAP; }
+static_assert(Tile<2, 8>::SORT_CAP == Tile<3, 4>::SORT_CAP, "bin_cap");
+
 // Sets every tile kernel of b to the default launch shape.
 inline void default_launch(BatchDev& b, int sm_count) {
   b.sm_count = sm_count;
@@ -173,15 +200,23 @@ cudaError_t configure_kernels();
 // Tiled (sorted, deterministic) form.
 // sel non-null (a single scene): the first kernel also makes the step's record selection (what
 // launch_select does), publishing it to b.scenes[0].
+// With bins the keys kernel appends the particles to their tiles' lists; `reset` first empties the
+// lists (the start of a phase: in a chain of reverse steps P2G has cleared the other parity).  It
+// selects step *sel->ctr - back and with `snap` also writes that step number there.
 template <int D>
-cudaError_t launch_keys(const BatchDev& b, cudaStream_t s, const SelectPar* sel = nullptr);
+cudaError_t launch_keys(const BatchDev& b, cudaStream_t s, const SelectPar* sel = nullptr, bool reset = true,
+                        int back = 0, int* snap = nullptr);
+// Empties the tile bins (nothing without them).
+cudaError_t reset_bins(const BatchDev& b, cudaStream_t s);
 template <int D>
 cudaError_t launch_sort(const BatchDev& b, cudaStream_t s, const SelectPar* sel = nullptr);
 template <int D>
 cudaError_t launch_p2g(const BatchDev& b, bool with_adjoint, cudaStream_t s);
-// G2P (Eqs. 7-10) including the grid update of its node block (Eq. 6, gravity, boundary).
+// G2P (Eqs. 7-10) including the grid update of its node block (Eq. 6, gravity, boundary).  With sel
+// (a scene alone, with bins) an extra CTA makes the next step's record selection and advances the
+// step counter.
 template <int D>
-cudaError_t launch_g2p(const BatchDev& b, cudaStream_t s);
+cudaError_t launch_g2p(const BatchDev& b, cudaStream_t s, const SelectPar* sel = nullptr);
 // Adjoint gather (S4 (F)-(K), (J)) including the grid adjoint of its node block (S3, S5) and
 // the per-tile group sums of dL/da into gpartial.
 template <int D>
@@ -226,8 +261,11 @@ int reduction_rows(int N);                  // partial rows of the group reducti
 constexpr int RED_ROW_FLOATS = MAX_GROUPS * 3 + 3;  // floats per partial row
 // Controller forward (MLP form; the sinusoid forms are evaluated by k_select) and the reverse of
 // the step *sp.step_ctr, which it then decrements.
-cudaError_t ctrl_step_forward(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s);
-cudaError_t ctrl_step_backward(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s);
+// The record is dsp[*flip] (dsp[0] without flip): the parity word of the batch's bins.
+cudaError_t ctrl_step_forward(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s,
+                              const uint32_t* flip = nullptr);
+cudaError_t ctrl_step_backward(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s,
+                               const uint32_t* flip = nullptr);
 // Reverse of a controller that reads no state (sinusoid and table forms) for the step after the
 // one *ctr names, whose group sums are rows [0, *rows) of c.gpart: the counter was already rewound
 // by the adjoint gather (BatchDev::rewind_ctr), so the launch depends on nothing but that kernel.
@@ -237,8 +275,10 @@ cudaError_t ctrl_backward_open(const CtrlPar& c, const int* ctr, const int* rows
 cudaError_t ctrl_backward_batched(const ScenePar* cur, const CtrlPar* cs, int n, cudaStream_t s);
 cudaError_t ctrl_scatter_x(const ScenePar& sp, const ScenePar* dsp, const CtrlPar& c, cudaStream_t s);
 
-// Copies every scene's record for the current step into cur[] (one block per scene).
-cudaError_t launch_select(const SelectPar* sel, int n_scenes, ScenePar* cur, cudaStream_t s);
+// Copies every scene's record for the current step into cur[] (one block per scene); with flip (one
+// scene) into cur[*flip].
+cudaError_t launch_select(const SelectPar* sel, int n_scenes, ScenePar* cur, cudaStream_t s,
+                          const uint32_t* flip = nullptr);
 // Sort store of a single scene: the sort just made in b (raw tile lists, tile arrays, keys) into
 // slot `dst` (NULL: the slot named by the published record b.scenes[0]), and the sort of the
 // state the reverse selection `sel` names back into b (publishing the record, like launch_keys).

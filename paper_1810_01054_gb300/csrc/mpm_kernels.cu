@@ -105,11 +105,11 @@ __device__ __forceinline__ uint32_t bin_key(const float* x, const ScenePar& sp) 
   return (uint32_t(lin3<D>(t, sp.nt)) << 6) | uint32_t(cell_lin<D, TB>(c));
 }
 
-// Actuation group of particle id (-1: none).
-__device__ __forceinline__ int group_of(const ScenePar& sp, int id) {
-  const int g = sp.group ? __ldg(sp.group + id) : -1;
-  return g < sp.G ? g : -1;
-}
+// Actuation group of particle id as given, and the one it acts in (-1: none).  Apart, so that a
+// caller that requests the group early does not wait for it there.
+__device__ __forceinline__ int group_raw(const ScenePar& sp, int id) { return sp.group ? __ldg(sp.group + id) : -1; }
+__device__ __forceinline__ int group_in(const ScenePar& sp, int g) { return g < sp.G ? g : -1; }
+__device__ __forceinline__ int group_of(const ScenePar& sp, int id) { return group_in(sp, group_raw(sp, id)); }
 
 // Actuations [G] and directions [G][dim] of the step: the scene's arrays, or a tile kernel's copies.
 struct ActSrc {
@@ -127,28 +127,34 @@ __device__ __forceinline__ void actuation(const ActSrc& as, int g, float* sig) {
 
 // A tile kernel's copy of the scene record it works under (and, with ACT, of the actuations and
 // directions), in shared memory.  Read from global memory every field costs its first user a trip to
-// L2, at several places of a tile's dependent chain, and the actuation one more after the particle's
-// group; here all of it arrives in two trips beside the tile list's (1M-particle 3D scene, 16 steps
-// 2298 -> 2268 us; 1,024-particle 2D scene, 64 steps 871 -> 850 us).  Every thread calls it; the
-// record is readable on return, the actuations after the caller's next barrier.
+// L2 (about 900 cycles for what another SM has just written), at several places of a tile's dependent
+// chain, and the actuation one more after the particle's group.
 struct SceneShared {
   __align__(16) ScenePar sp;
   float act[MAX_GROUPS], dir[MAX_GROUPS * 3];
 };
+constexpr int SCENE_WORDS = int(sizeof(ScenePar) / sizeof(int));
+static_assert(SCENE_WORDS <= 128, "one word per thread of the smallest tile kernel");
+
+// Requests the actuations of the staged record: asynchronous copies, so nobody waits for them here.
+// The caller waits for its own copies (cp_async_wait_all) before the barrier that precedes their use.
+template <int D>
+__device__ __forceinline__ void stage_actuation(SceneShared& sh) {
+  const int G = sh.sp.G;
+  for (int i = threadIdx.x; i < G * D; i += blockDim.x) {
+    cp_async4(&sh.dir[i], sh.sp.act_dir + i);
+    if (i < G) cp_async4(&sh.act[i], sh.sp.act + i);
+  }
+  cp_async_commit();
+}
+
+// The record src; every thread calls it, readable on return.
 template <int D, bool ACT>
 __device__ __forceinline__ void stage_scene(const ScenePar* src, SceneShared& sh) {
-  constexpr int W = int(sizeof(ScenePar) / sizeof(int));
-  const int* s = reinterpret_cast<const int*>(src);
-  int* d = reinterpret_cast<int*>(&sh.sp);
-  for (int i = threadIdx.x; i < W; i += blockDim.x) d[i] = s[i];
+  if (threadIdx.x < SCENE_WORDS)
+    reinterpret_cast<int*>(&sh.sp)[threadIdx.x] = reinterpret_cast<const int*>(src)[threadIdx.x];
   __syncthreads();
-  if constexpr (ACT) {
-    const int G = sh.sp.G;
-    for (int i = threadIdx.x; i < G * D; i += blockDim.x) {
-      sh.dir[i] = sh.sp.act_dir[i];
-      if (i < G) sh.act[i] = sh.sp.act[i];
-    }
-  }
+  if constexpr (ACT) stage_actuation<D>(sh);
 }
 
 // Material of particle id: the scene's, or its own Young's modulus and mass when the scene has
@@ -213,6 +219,7 @@ __device__ __forceinline__ void select_copy(const SelectPar& q, int n, ScenePar*
 // The selection of step n for one scene: its record into cur, and the sinusoid and table
 // controllers' actuation a_g(t_n) into q.act.
 __device__ __forceinline__ void select_publish_at(const SelectPar& q, int n, ScenePar* cur) {
+  if (q.map && n - q.base >= q.len) return;  // past the phase: its successor makes its own selection
   select_copy(q, n, cur);
   const float tt = float(n) * q.dt;
   const int g = threadIdx.x;
@@ -231,29 +238,106 @@ __device__ __forceinline__ void select_publish_at(const SelectPar& q, int n, Sce
 __device__ __forceinline__ void select_publish(const SelectPar& q, ScenePar* cur) { select_publish_at(q, *q.ctr, cur); }
 
 // ============================================================================ keys / sort
-// Bin keys of the state being read, and the tile histogram (tile_count must be zero on entry).
-// With SEL (a single scene) the kernel also makes the step's selection: every CTA copies the
-// selected record to shared memory for its own use and CTA 0 publishes it (and the actuation) for
-// the kernels that follow, which replaces the selection launch.
+// ============================================================================ tile bins
+// Appends particle entry e to tile t's list (t < 0: nothing) under parity q: one atomic per distinct
+// tile of the warp gives the places, the first entry of a tile sets its mask bit.  An entry beyond
+// the tile's room is dropped; its count still shows the tile over capacity.
+template <int D, int TB>
+__device__ __forceinline__ void bin_append(const BatchDev& b, uint32_t q, int t, uint32_t e) {
+  const uint32_t rank = warp_aggregated_inc(b.bin_ctl + BIN_COUNT + size_t(q) * b.total_tiles, t);
+  if (t < 0) return;
+  if (rank < uint32_t(Tile<D, TB>::SORT_CAP)) b.bin_raw[size_t(t) * Tile<D, TB>::SORT_CAP + rank] = e;
+  if (rank == 0) atomicOr(b.bin_ctl + BIN_MASK + q * BIN_WORDS + (t >> 5), 1u << (t & 31));
+}
+
+// The non-empty tiles as a tile kernel sees them with bins: their mask and its running counts in
+// shared memory.  Every CTA reads it once, together with its scene record, and finds the tile of any
+// active slot (the slot-th set bit), and whether a neighbouring tile is active, without another trip
+// to memory.
+struct BinView {
+  uint32_t mask[BIN_WORDS], before[BIN_WORDS];
+  int n;
+};
+
+// Fills v from parity p = bin_ctl[which], and sh with the scene record of that parity (record 0
+// unless the batch keeps them by parity): both parities are requested with the parity word, so all
+// of it takes one trip to memory.  Every thread calls it; readable on return.  Returns p.
+__device__ __forceinline__ uint32_t bin_view(const BatchDev& b, int which, BinView& v, SceneShared& sh) {
+  const int tid = threadIdx.x;
+  const uint32_t m0 = tid < BIN_WORDS ? b.bin_ctl[BIN_MASK + tid] : 0u;
+  const uint32_t m1 = tid < BIN_WORDS ? b.bin_ctl[BIN_MASK + BIN_WORDS + tid] : 0u;
+  const int* rec = reinterpret_cast<const int*>(b.scenes);
+  const int r0 = tid < SCENE_WORDS ? rec[tid] : 0;
+  const int r1 = tid < SCENE_WORDS && b.rec_flip ? rec[SCENE_WORDS + tid] : r0;
+  const uint32_t p = b.bin_ctl[which] & 1u;
+  if (tid < BIN_WORDS) v.mask[tid] = p ? m1 : m0;
+  if (tid < SCENE_WORDS) reinterpret_cast<int*>(&sh.sp)[tid] = p ? r1 : r0;
+  __syncthreads();
+  if (tid < 32) {
+    const int c0 = __popc(v.mask[tid]), c1 = __popc(v.mask[tid + 32]);
+    int i0 = c0, i1 = c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int a0 = __shfl_up_sync(0xffffffffu, i0, o), a1 = __shfl_up_sync(0xffffffffu, i1, o);
+      if (tid >= o) {
+        i0 += a0;
+        i1 += a1;
+      }
+    }
+    const int tot0 = __shfl_sync(0xffffffffu, i0, 31);
+    v.before[tid] = uint32_t(i0 - c0);
+    v.before[tid + 32] = uint32_t(tot0 + i1 - c1);
+    if (tid == 31) v.n = tot0 + i1;
+  }
+  __syncthreads();
+  return p;
+}
+
+// Tile of active slot `slot` < v.n (all 32 lanes of a warp call it).
+__device__ __forceinline__ int bin_tile(const BinView& v, int slot) {
+  const int lane = threadIdx.x & 31;
+  const unsigned b0 = __ballot_sync(0xffffffffu, int(v.before[lane]) <= slot);
+  const unsigned b1 = __ballot_sync(0xffffffffu, int(v.before[lane + 32]) <= slot);
+  const int w = __popc(b0) + __popc(b1) - 1;  // the last word that starts at or before it
+  const uint32_t word = v.mask[w];
+  const int r = slot - int(v.before[w]);
+  const unsigned hit = __ballot_sync(0xffffffffu, ((word >> lane) & 1u) && __popc(word & ((1u << lane) - 1u)) == r);
+  return w * 32 + __ffs(hit) - 1;
+}
+
+// Bin keys of the state being read, and the tile histogram (tile_count must be zero on entry), or
+// with bins the tile lists of the parity the gathers do not read.  With SEL (a single scene) the
+// kernel also makes the step's selection (step *ctr - back): every CTA copies the selected record to
+// shared memory for its own use and CTA 0 publishes it (and the actuation) for the kernels that
+// follow, which replaces the selection launch.
 template <int D, int TB, bool SEL>
-__global__ void k_keys(BatchDev b, const SelectPar* __restrict__ sel) {
+__global__ void k_keys(BatchDev b, const SelectPar* __restrict__ sel, int back, int* snap) {
   pdl_enter();
   __shared__ __align__(16) ScenePar srec[1];
+  const uint32_t q = b.bin_ctl ? (b.bin_ctl[1] & 1u) ^ 1u : 0u;
   if constexpr (SEL) {
-    const int n = *sel->ctr;
+    const int n = *sel->ctr - back;
     select_copy(*sel, n, srec);
-    if (blockIdx.x == 0) select_publish(*sel, b.scenes);
+    if (blockIdx.x == 0) {
+      select_publish_at(*sel, n, b.scenes + (b.rec_flip ? q : 0u));
+      if (snap && threadIdx.x == 0) *snap = n;
+    }
     __syncthreads();
   }
+  if (b.bin_ctl && blockIdx.x == 0 && threadIdx.x == 0) b.bin_ctl[0] = q;
   int gp = blockIdx.x * blockDim.x + threadIdx.x;
   if (gp >= b.total_particles) return;
   const ScenePar& sp = SEL ? srec[0] : b.scenes[find_scene(b.scene_pbase, b.n_scenes, gp)];
   int p = gp - sp.pbase;
-  float4 q = sp.planes[p];
-  float x[3] = {q.x, q.y, q.z};
+  float4 xq = sp.planes[p];
+  float x[3] = {xq.x, xq.y, xq.z};
   const uint32_t k = bin_key<D, TB>(x, sp);
   sp.key[p] = k;
-  warp_aggregated_inc(b.tile_count, k != KEY_INVALID ? int(sp.tile_base + (k >> 6)) : -1);
+  const int t = k != KEY_INVALID ? int(sp.tile_base + (k >> 6)) : -1;
+  if (b.bin_ctl)
+    bin_append<D, TB>(b, q, t, ((k & 63u) << 26) | uint32_t(p));
+  else
+    warp_aggregated_inc(b.tile_count, t);
 }
 
 // Exclusive block scan of (sum, count) pairs over blockDim.x <= 1024 threads.
@@ -299,10 +383,6 @@ __device__ __forceinline__ void block_scan2(uint32_t& a, uint32_t& c, uint32_t& 
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_PER_THREAD = 2;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_PER_THREAD;
-// Small batches scan the tile histogram inside the scatter kernel (k_scatter<D, true>); the P2G
-// that follows every scatter clears the counters.
-__host__ __device__ __forceinline__ bool fused_scan(const BatchDev& b) { return b.total_tiles <= SCAN_TILE; }
-
 // Phase 1 of the tile scan: per-block totals of particle counts and of active tiles.
 template <bool SEL>
 __global__ void k_scan_reduce(BatchDev b, const SelectPar* __restrict__ sel) {
@@ -389,73 +469,20 @@ __global__ void k_scan_down(BatchDev b) {
   }
 }
 
-// Scatter of the particles into their tiles' ranges of `sorted`.  With FUSED (total_tiles <=
-// SCAN_TILE) the tile scan is done here instead of by the scan kernels: every CTA scans the whole
-// histogram in shared memory (it is small), CTA 0 publishes tile_start, tile_slot, the active list
-// and n_active; the P2G that follows clears the per-step counters.
-// With SEL (a single scene, fused scan) one extra CTA, launched after the scatter's own, makes the
-// step's selection (see k_keys) alongside them; the scatter reads only the record's step-invariant
-// fields (keys, offsets, status), which it takes from the phase's first record instead of the
-// one being published.
-template <int D, bool FUSED, bool SEL>
-__global__ void __launch_bounds__(256) k_scatter(BatchDev b, const SelectPar* __restrict__ sel) {
+// Scatter of the particles into their tiles' ranges of `sorted`.
+template <int D>
+__global__ void __launch_bounds__(256) k_scatter(BatchDev b) {
   pdl_enter();
-  if (SEL && blockIdx.x == gridDim.x - 1) {
-    select_publish(*sel, b.scenes);
-    return;
-  }
-  constexpr int PER = FUSED ? SCAN_TILE / 256 : 1;
-  __shared__ uint32_t sstart[FUSED ? SCAN_TILE + 1 : 1];
-  if constexpr (FUSED) {
-    const int nt = b.total_tiles, t0 = threadIdx.x * PER;
-    uint32_t cnt[PER], s = 0, c = 0;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      cnt[i] = t0 + i < nt ? b.tile_count[t0 + i] : 0u;
-      s += cnt[i];
-      c += cnt[i] > 0;
-    }
-    uint32_t ts, tc;
-    block_scan2(s, c, ts, tc);
-    const bool pub = blockIdx.x == 0;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int t = t0 + i;
-      if (t < nt) {
-        sstart[t] = s;
-        if (pub) {
-          b.tile_start[t] = s;
-          if (cnt[i] > 0) {
-            b.tile_slot[t] = int(c);
-            b.active[c] = t;
-          } else {
-            b.tile_slot[t] = -1;
-          }
-        }
-        s += cnt[i];
-        c += cnt[i] > 0;
-      }
-    }
-    if (threadIdx.x == 0) {
-      sstart[nt] = ts;
-      if (pub) {
-        b.tile_start[nt] = ts;
-        *b.n_active = int(tc);
-      }
-    }
-    __syncthreads();
-  }
   int gp = blockIdx.x * blockDim.x + threadIdx.x;
   if (gp >= b.total_particles) return;
-  const ScenePar& sp = SEL ? sel->table[0] : b.scenes[find_scene(b.scene_pbase, b.n_scenes, gp)];
-  const int pbase = SEL ? sel->pbase : sp.pbase, tbase = SEL ? sel->tile_base : sp.tile_base;
-  int p = gp - pbase;
+  const ScenePar& sp = b.scenes[find_scene(b.scene_pbase, b.n_scenes, gp)];
+  int p = gp - sp.pbase;
   const uint32_t k = sp.key[p];
-  const int t = k != KEY_INVALID ? int(tbase + (k >> 6)) : -1;
+  const int t = k != KEY_INVALID ? int(sp.tile_base + (k >> 6)) : -1;
   const uint32_t rank = warp_aggregated_inc(b.tile_fill, t);
   if (t < 0) return;
-  const uint32_t start = FUSED ? sstart[t] : b.tile_start[t];
-  const uint32_t end = FUSED ? sstart[t + 1] : b.tile_start[t + 1];
+  const uint32_t start = b.tile_start[t];
+  const uint32_t end = b.tile_start[t + 1];
   if (start + rank >= end) {  // a key the histogram did not count: record it, write nothing
     set_status(sp.status, ST_BINNING);
     return;
@@ -620,7 +647,8 @@ struct P2GCfg {
 // Resident CTAs: the 3D forward P2G keeps 3 of 256 threads per SM (85 registers, a few spills in
 // its record phase; 4 % faster on the 1M-particle cluster than 2 at 126 registers); the adjoint
 // scatter holds 63 accumulators and keeps 2.
-template <int D, int TB, bool ADJ, int T>
+// BINS: the tile lists are bins (BatchDev::bin_ctl), else the sort's.
+template <int D, int TB, bool ADJ, int T, bool BINS>
 __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_p2g(BatchDev b) {
   pdl_enter();
   using K = P2GCfg<D, TB, ADJ, T>;
@@ -634,19 +662,37 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
   const int tid = threadIdx.x;
   // the CTA's first active tile is requested together with the count (the entry is in bounds
   // whatever the count; it is used only when the slot is below it)
-  const int first_gt = b.total_tiles > 0 ? b.active[int(blockIdx.x) < b.total_tiles ? blockIdx.x : 0] : 0;
-  const int n_active = *b.n_active;
   __shared__ SceneShared sh;
+  __shared__ BinView bv;  // (unused without BINS)
   const ScenePar& sp = sh.sp;
   const ActSrc as{sh.act, sh.dir};
-  int scene = 0;
-  stage_scene<D, true>(b.scenes, sh);
-  // the per-step counters are cleared here whichever scan ran (the fused one leaves them set, the
-  // separate one leaves the scatter's fill counts): every step then starts from zero, also when a
-  // batch's composition moves it between the two scans
-  for (int i = blockIdx.x * blockDim.x + tid; i < b.total_tiles; i += gridDim.x * blockDim.x) {
-    b.tile_count[i] = 0u;
-    b.tile_fill[i] = 0u;
+  int scene = 0, first_gt = 0, n_active;
+  uint32_t par = 0;
+  if constexpr (BINS) {
+    par = bin_view(b, 0, bv, sh);
+    n_active = bv.n;
+    // the other parity is cleared for the lists of the next state
+    uint32_t* om = b.bin_ctl + BIN_MASK + (par ^ 1u) * BIN_WORDS;
+    uint32_t* oc = b.bin_ctl + BIN_COUNT + size_t(par ^ 1u) * b.total_tiles;
+    for (int i = blockIdx.x * blockDim.x + tid; i < b.total_tiles; i += gridDim.x * blockDim.x) oc[i] = 0u;
+    if (blockIdx.x == 0) {
+      if (tid < BIN_WORDS) om[tid] = 0u;
+      if (tid == 0) {
+        b.bin_ctl[1] = par;
+        *b.n_active = n_active;
+      }
+    }
+    if (int(blockIdx.x) >= n_active) return;
+    stage_actuation<D>(sh);
+  } else {
+    if (b.total_tiles > 0) first_gt = b.active[int(blockIdx.x) < b.total_tiles ? blockIdx.x : 0];
+    n_active = *b.n_active;
+    stage_scene<D, true>(b.scenes, sh);
+    // the scatter's counts are cleared here: every step starts from zero
+    for (int i = blockIdx.x * blockDim.x + tid; i < b.total_tiles; i += gridDim.x * blockDim.x) {
+      b.tile_count[i] = 0u;
+      b.tile_fill[i] = 0u;
+    }
   }
 
   __shared__ int s_next[2];
@@ -657,19 +703,38 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
   int it = 0;
   for (int slot = blockIdx.x; slot < n_active; slot = dyn ? take_next(s_next, it++) : slot + int(gridDim.x)) {
     if (dyn) claim_next(b, 0, s_next, it);
-    const int gt = slot == int(blockIdx.x) ? first_gt : b.active[slot];
-    const uint32_t st = b.tile_start[gt];
-    const int cnt = int(b.tile_start[gt + 1] - st);
+    // the tile, its list as binned (raw) and its place for the canonical one, the row of its node block
+    int gt, cnt, row;
+    const uint32_t* raw;
+    uint32_t* canon;
+    uint32_t e0 = 0u, e1 = 0u;
+    if constexpr (BINS) {
+      gt = row = bin_tile(bv, slot);
+      raw = b.bin_raw + size_t(gt) * K::CAP;
+      canon = b.sorted + size_t(gt) * K::CAP;
+      // the thread's entries are requested with the count (in bounds whatever the count)
+      e0 = raw[tid];
+      e1 = raw[tid + K::THREADS];
+      cnt = int(b.bin_ctl[BIN_COUNT + size_t(par) * b.total_tiles + gt]);
+      if (tid == 0) b.active[slot] = gt;  // for the controller reverse
+    } else {
+      gt = slot == int(blockIdx.x) ? first_gt : b.active[slot];
+      const uint32_t st = b.tile_start[gt];
+      cnt = int(b.tile_start[gt + 1] - st);
+      raw = canon = b.sorted + st;
+      row = slot;
+    }
     if (b.n_scenes > 1 && b.tile_scene[gt] != scene) {  // uniform across the CTA
       scene = b.tile_scene[gt];
-      __syncthreads();  // a skipped tile ends without a barrier
+      cp_async_wait_all();  // the copies of the record before it
+      __syncthreads();      // (a skipped tile ends without a barrier)
       stage_scene<D, true>(b.scenes + scene, sh);
     }
     if (cnt > K::CAP) {  // the step fails (status); the tile adds nothing to the grid
       if (tid == 0) set_status(sp.status, ST_DENSITY);
       for (int i = tid; i < NB; i += blockDim.x) {
-        b.partial[size_t(slot) * NB + i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if constexpr (ADJ) b.partial_b[size_t(slot) * NB + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        b.partial[size_t(row) * NB + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (ADJ) b.partial_b[size_t(row) * NB + i] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
       continue;  // uniform across the CTA
     }
@@ -910,15 +975,15 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
       // Its first particle's state is requested at once and arrives while the tile is being
       // bucketed; its canonical position is the cell start plus the number of smaller ids in its
       // cell (order: cell, then particle id), and its record is written straight there.
-      const uint32_t r0 = tid < cnt ? b.sorted[st + tid] : 0xffffffffu;
-      const uint32_t r1 = tid + K::THREADS < cnt ? b.sorted[st + tid + K::THREADS] : 0xffffffffu;
+      const uint32_t r0 = tid < cnt ? (BINS ? e0 : raw[tid]) : 0xffffffffu;
+      const uint32_t r1 = tid + K::THREADS < cnt ? (BINS ? e1 : raw[tid + K::THREADS]) : 0xffffffffu;
       float pre[Cfg<D>::S];
       int g0 = -1, g1 = -1;
       if (r0 != 0xffffffffu) {
         load_planes<D, Cfg<D>::PLANES>(sp.planes, sp.npad, int(r0 & 0x3ffffffu), pre);
-        g0 = group_of(sp, int(r0 & 0x3ffffffu));
+        g0 = group_raw(sp, int(r0 & 0x3ffffffu));
       }
-      if (r1 != 0xffffffffu) g1 = group_of(sp, int(r1 & 0x3ffffffu));
+      if (r1 != 0xffffffffu) g1 = group_raw(sp, int(r1 & 0x3ffffffu));
       // the counting atomics also give each entry its place among its cell's entries
       const int k0 = r0 != 0xffffffffu ? atomicAdd(&cfill[r0 >> 26], 1) : 0;
       const int k1 = r1 != 0xffffffffu ? atomicAdd(&cfill[r1 >> 26], 1) : 0;
@@ -933,6 +998,7 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
         if (r0 != 0xffffffffu) ids[s0 + k0] = r0 & 0x3ffffffu;
         if (r1 != 0xffffffffu) ids[s1 + k1] = r1 & 0x3ffffffu;
       }
+      cp_async_wait_all();  // the actuations (readable by all after the barrier)
       __syncthreads();
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -941,13 +1007,13 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
         const uint32_t id = rr & 0x3ffffffu, c = rr >> 26;
         int pos = cstart[c];
         for (int j = cstart[c]; j < cstart[c + 1]; ++j) pos += ids[j] < id;
-        b.sorted[st + pos] = id;  // canonical order for the gathers of this step
+        canon[pos] = id;  // canonical order for the gathers of this step
         if (h == 0) {
-          make_record(int(id), c, g0, pre, pos);
+          make_record(int(id), c, group_in(sp, g0), pre, pos);
         } else {
           float r[Cfg<D>::S];
           load_planes<D, Cfg<D>::PLANES>(sp.planes, sp.npad, int(id), r);
-          make_record(int(id), c, g1, r, pos);
+          make_record(int(id), c, group_in(sp, g1), r, pos);
         }
       }
       __syncthreads();
@@ -956,12 +1022,13 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
         if (item_thread[j]) accumulate(j, cstart[my_cell[j]], cstart[my_cell[j] + 1], 0);
     } else {
       // ---- general path: bucket, insertion-sort each cell's ids, stage records in chunks
-      uint32_t* raw = reinterpret_cast<uint32_t*>(U);
+      uint32_t* ent = reinterpret_cast<uint32_t*>(U);
       if (tid < CELLS) cfill[tid] = 0;
+      cp_async_wait_all();  // the actuations
       __syncthreads();
       for (int i = tid; i < cnt; i += blockDim.x) {
-        const uint32_t r = b.sorted[st + i];  // (cell << 26) | id, written by the scatter
-        raw[i] = r;
+        const uint32_t r = raw[i];  // (cell << 26) | id, as binned
+        ent[i] = r;
         atomicAdd(&cfill[r >> 26], 1);
       }
       __syncthreads();
@@ -970,7 +1037,7 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
       if (tid < CELLS) cfill[tid] = 0;
       __syncthreads();
       for (int i = tid; i < cnt; i += blockDim.x) {
-        const uint32_t r = raw[i];
+        const uint32_t r = ent[i];
         const uint32_t c = r >> 26;
         ids[cstart[c] + atomicAdd(&cfill[c], 1)] = r & 0x3ffffffu;
       }
@@ -988,7 +1055,7 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
         }
       }
       __syncthreads();
-      for (int i = tid; i < cnt; i += blockDim.x) b.sorted[st + i] = ids[i];
+      for (int i = tid; i < cnt; i += blockDim.x) canon[i] = ids[i];
       int cs[K::IPT], ce[K::IPT];
 #pragma unroll
       for (int j = 0; j < K::IPT; ++j) {
@@ -1083,14 +1150,14 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
         o = make_float4(s[0], s[1], s[2], 0.0f);
       else
         o = make_float4(s01.x, s01.y, s23.x, s23.y);
-      b.partial[size_t(slot) * NB + tid] = o;
+      b.partial[size_t(row) * NB + tid] = o;
       if constexpr (ADJ) {
         float4 oa;
         if constexpr (D == 2)
           oa = make_float4(s[K::CHF], s[K::CHF + 1], 0.0f, 0.0f);
         else
           oa = make_float4(s45.x, s45.y, s6, 0.0f);
-        b.partial_b[size_t(slot) * NB + tid] = oa;
+        b.partial_b[size_t(row) * NB + tid] = oa;
       }
     }
     if (tid < CELLS) cfill[tid] = 0;  // for the next tile (nothing reads the counts after placement)
@@ -1106,8 +1173,8 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
 // vbar*, and (L), (D), (E) give pbar and mbar.  Nodes a tile owns (its B^D corner) are also
 // written to the dense grid for inspection.
 template <int D, int TB, bool ADJ>
-__device__ __forceinline__ void build_node_block(const BatchDev& b, const ScenePar& sp, const int* t, float4* sv,
-                                                 float4* sb) {
+__device__ __forceinline__ void build_node_block(const BatchDev& b, const ScenePar& sp, const BinView* bv,
+                                                 const int* t, float4* sv, float4* sb) {
   constexpr int B = Tile<D, TB>::B, NB = Tile<D, TB>::BLOCK_NODES, BN = Tile<D, TB>::BN;
   constexpr int NN = D == 2 ? 9 : 27;  // tiles t + o, o in {-1, 0, 1}^D
   __shared__ int nslot[NN];
@@ -1121,7 +1188,12 @@ __device__ __forceinline__ void build_node_block(const BatchDev& b, const SceneP
       u[a] = t[a] + o[a];
       ok = ok && u[a] >= 0 && u[a] < sp.nt[a];
     }
-    nslot[threadIdx.x] = ok ? b.tile_slot[sp.tile_base + lin3<D>(u, sp.nt)] : -1;
+    int row = -1;  // row of the tile's node block: the tile itself with bins, else its active slot
+    if (ok) {
+      const int g = sp.tile_base + lin3<D>(u, sp.nt);
+      row = bv ? ((bv->mask[g >> 5] >> (g & 31)) & 1u ? g : -1) : b.tile_slot[g];
+    }
+    nslot[threadIdx.x] = row;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < NB; i += blockDim.x) {
@@ -1344,29 +1416,61 @@ struct G2PCfg {
   static constexpr int NP = Cfg<D>::XF_PLANES;
 };
 
-template <int D, int TB, int T>
-__global__ void __launch_bounds__(T, 768 / T) k_g2p(BatchDev b) {
+template <int D, int TB, int T, bool BINS>
+__global__ void __launch_bounds__(T, 768 / T) k_g2p(BatchDev b, const SelectPar* __restrict__ sel) {
   pdl_enter();
   using K = G2PCfg<D>;
   constexpr int B = Tile<D, TB>::B, NB = Tile<D, TB>::BLOCK_NODES, BN = Tile<D, TB>::BN;
   __shared__ float4 sv[NB];
   __shared__ float4 stage[K::NP][K::STAGE];
   const int tid = threadIdx.x;
-  // the CTA's first active tile is requested together with the count (the entry is in bounds
-  // whatever the count; it is used only when the slot is below it)
-  const int first_gt = b.total_tiles > 0 ? b.active[int(blockIdx.x) < b.total_tiles ? blockIdx.x : 0] : 0;
-  const int n_active = *b.n_active;
+  // with sel CTA 0 only makes the next step's selection (into the other parity's record, which no
+  // kernel of this step reads) and moves the counter on
+  const int own = BINS && sel ? 1 : 0, cta = int(blockIdx.x) - own, ctas = int(gridDim.x) - own;
+  if (BINS && cta < 0) {
+    const int n = *sel->ctr;
+    const uint32_t q = (b.bin_ctl[1] & 1u) ^ 1u;
+    select_publish_at(*sel, n + 1, b.scenes + q);
+    __syncthreads();
+    if (tid == 0) *const_cast<int*>(sel->ctr) = n + 1;
+    return;
+  }
   __shared__ SceneShared sh;
+  __shared__ BinView bv;
   const ScenePar& sp = sh.sp;
-  int scene = 0;
-  stage_scene<D, false>(b.scenes, sh);
-  if (blockIdx.x == 0)  // this step's counters move on (every reader of them ran before)
+  int scene = 0, first_gt = 0, n_active;
+  uint32_t par = 0;
+  if constexpr (BINS) {
+    par = bin_view(b, 1, bv, sh);
+    n_active = bv.n;
+    if (cta == 0 && tid == 0) b.bin_ctl[0] = par ^ 1u;  // the lists appended below come next
+  } else {
+    // the CTA's first active tile is requested together with the count (the entry is in bounds
+    // whatever the count; it is used only when the slot is below it)
+    if (b.total_tiles > 0) first_gt = b.active[cta < b.total_tiles ? cta : 0];
+    n_active = *b.n_active;
+    stage_scene<D, false>(b.scenes, sh);
+  }
+  if (cta == 0 && !own)  // this step's counters move on (every reader of them ran before)
     for (int s = tid; s < b.n_scenes; s += blockDim.x)
       if (b.scenes[s].step_ctr) *b.scenes[s].step_ctr += 1;
-  for (int slot = blockIdx.x; slot < n_active; slot += gridDim.x) {
-    const int gt = slot == int(blockIdx.x) ? first_gt : b.active[slot];
-    const uint32_t st = b.tile_start[gt];
-    const int cnt = int(b.tile_start[gt + 1] - st);
+  for (int slot = cta; slot < n_active; slot += ctas) {
+    int gt, cnt;
+    const uint32_t* list;
+    constexpr int SPT = (K::STAGE + T - 1) / T;
+    uint32_t ent[SPT];  // the thread's entries of the staged particles
+    if constexpr (BINS) {
+      gt = bin_tile(bv, slot);
+      list = b.sorted + size_t(gt) * Tile<D, TB>::SORT_CAP;
+#pragma unroll
+      for (int u = 0; u < SPT; ++u) ent[u] = list[tid + u * T];  // with the count (in bounds whatever it is)
+      cnt = int(b.bin_ctl[BIN_COUNT + size_t(par) * b.total_tiles + gt]);
+    } else {
+      gt = slot == cta ? first_gt : b.active[slot];
+      const uint32_t st = b.tile_start[gt];
+      cnt = int(b.tile_start[gt + 1] - st);
+      list = b.sorted + st;
+    }
     if (b.n_scenes > 1 && b.tile_scene[gt] != scene) {  // uniform across the CTA
       scene = b.tile_scene[gt];
       __syncthreads();  // a skipped tile ends without a barrier
@@ -1379,17 +1483,19 @@ __global__ void __launch_bounds__(T, 768 / T) k_g2p(BatchDev b) {
     if (cnt > Tile<D, TB>::SORT_CAP) {  // uniform across the CTA
       // its particles are not advanced: their keys go invalid so the next step's histogram and
       // scatter (which count keys) stay consistent; the step has already reported the error
-      for (int e = tid; e < cnt; e += blockDim.x) sp.key[b.sorted[st + e] & 0x3ffffffu] = KEY_INVALID;
+      // (with bins they are simply not appended again)
+      if constexpr (!BINS)
+        for (int e = tid; e < cnt; e += blockDim.x) sp.key[list[e] & 0x3ffffffu] = KEY_INVALID;
       continue;
     }
     const int staged = cnt < K::STAGE ? cnt : K::STAGE;
     // request the x, F planes of the tile's particles; they arrive while the node block is built
     // (the thread's list entries are read first, all at once, then the copies are issued)
     {
-      constexpr int SPT = (K::STAGE + T - 1) / T;
-      uint32_t ent[SPT];
+      if constexpr (!BINS) {
 #pragma unroll
-      for (int u = 0; u < SPT; ++u) ent[u] = tid + u * T < staged ? b.sorted[st + tid + u * T] : 0u;
+        for (int u = 0; u < SPT; ++u) ent[u] = tid + u * T < staged ? list[tid + u * T] : 0u;
+      }
 #pragma unroll
       for (int u = 0; u < SPT; ++u) {
         const int e = tid + u * T;
@@ -1400,11 +1506,11 @@ __global__ void __launch_bounds__(T, 768 / T) k_g2p(BatchDev b) {
       }
     }
     cp_async_commit();
-    build_node_block<D, TB, false>(b, sp, t, sv, nullptr);
+    build_node_block<D, TB, false>(b, sp, BINS ? &bv : nullptr, t, sv, nullptr);
     cp_async_wait_all();
     __syncthreads();
     for (int e = tid; e < cnt; e += blockDim.x) {
-      const int id = int(b.sorted[st + e] & 0x3ffffffu);
+      const int id = int(list[e] & 0x3ffffffu);
       float r[Cfg<D>::S];
       if (e < K::STAGE) {
 #pragma unroll
@@ -1443,9 +1549,13 @@ __global__ void __launch_bounds__(T, 768 / T) k_g2p(BatchDev b) {
       float ro[Cfg<D>::S];
       pack<D>(q, ro);
       store_planes<D, Cfg<D>::PLANES>(sp.planes_out, sp.npad, id, ro);
-      const uint32_t nk = bin_key<D, TB>(q.x, sp);  // bin of state n+1 and its histogram
+      const uint32_t nk = bin_key<D, TB>(q.x, sp);  // bin of state n+1 and its list or histogram
       sp.key[id] = nk;
-      warp_aggregated_inc(b.tile_count, nk != KEY_INVALID ? int(sp.tile_base + (nk >> 6)) : -1);
+      const int ntile = nk != KEY_INVALID ? int(sp.tile_base + (nk >> 6)) : -1;
+      if constexpr (BINS)
+        bin_append<D, TB>(b, par ^ 1u, ntile, ((nk & 63u) << 26) | uint32_t(id));
+      else
+        warp_aggregated_inc(b.tile_count, ntile);
     }
     __syncthreads();
   }
@@ -1809,22 +1919,30 @@ __device__ __forceinline__ float adj_core(Part<D>& q, Part<D>& g1, const float* 
 template <int D>
 constexpr int kAdjThreads = D == 3 ? 128 : 256;
 
-template <int D, int TB, bool MAT>
+template <int D, int TB, bool MAT, bool BINS>
 __global__ void __launch_bounds__(kAdjThreads<D>, 512 / kAdjThreads<D>) k_adj_gather(BatchDev b) {
   pdl_enter();
   constexpr int B = Tile<D, TB>::B, NB = Tile<D, TB>::BLOCK_NODES, BN = Tile<D, TB>::BN;
   __shared__ float4 sv[NB], sb[NB];
   __shared__ float wpart[8][MAX_GROUPS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // the CTA's first active tile is requested together with the count (the entry is in bounds
-  // whatever the count; it is used only when the slot is below it)
-  const int first_gt = b.total_tiles > 0 ? b.active[int(blockIdx.x) < b.total_tiles ? blockIdx.x : 0] : 0;
-  const int n_active = *b.n_active;
   __shared__ SceneShared sh;
+  __shared__ BinView bv;
   const ScenePar& sp = sh.sp;
   const ActSrc as{sh.act, sh.dir};
-  int scene = 0;
-  stage_scene<D, true>(b.scenes, sh);
+  int scene = 0, first_gt = 0, n_active;
+  uint32_t par = 0;
+  if constexpr (BINS) {
+    par = bin_view(b, 1, bv, sh);
+    n_active = bv.n;
+    stage_actuation<D>(sh);
+  } else {
+    // the CTA's first active tile is requested together with the count (the entry is in bounds
+    // whatever the count; it is used only when the slot is below it)
+    if (b.total_tiles > 0) first_gt = b.active[int(blockIdx.x) < b.total_tiles ? blockIdx.x : 0];
+    n_active = *b.n_active;
+    stage_scene<D, true>(b.scenes, sh);
+  }
   if (b.rewind_ctr && blockIdx.x == 0 && tid == 0) {
     *b.rewind_rows = n_active;
     *b.rewind_ctr -= 1;
@@ -1834,12 +1952,24 @@ __global__ void __launch_bounds__(kAdjThreads<D>, 512 / kAdjThreads<D>) k_adj_ga
   int it = 0;
   for (int slot = blockIdx.x; slot < n_active; slot = dyn ? take_next(s_next, it++) : slot + int(gridDim.x)) {
     if (dyn) claim_next(b, 1, s_next, it);
-    const int gt = slot == int(blockIdx.x) ? first_gt : b.active[slot];
-    const uint32_t st = b.tile_start[gt];
-    const int cnt = int(b.tile_start[gt + 1] - st);
+    int gt, cnt;
+    const uint32_t* list;
+    uint32_t ent0 = 0u;  // the thread's first entry
+    if constexpr (BINS) {
+      gt = bin_tile(bv, slot);
+      list = b.sorted + size_t(gt) * Tile<D, TB>::SORT_CAP;
+      ent0 = list[tid];  // with the count (in bounds whatever it is)
+      cnt = int(b.bin_ctl[BIN_COUNT + size_t(par) * b.total_tiles + gt]);
+    } else {
+      gt = slot == int(blockIdx.x) ? first_gt : b.active[slot];
+      const uint32_t st = b.tile_start[gt];
+      cnt = int(b.tile_start[gt + 1] - st);
+      list = b.sorted + st;
+    }
     if (b.n_scenes > 1 && b.tile_scene[gt] != scene) {  // uniform across the CTA
       scene = b.tile_scene[gt];
-      __syncthreads();  // a skipped tile ends without a barrier
+      cp_async_wait_all();  // the copies of the record before it
+      __syncthreads();      // (a skipped tile ends without a barrier)
       stage_scene<D, true>(b.scenes + scene, sh);
     }
     int t[D];
@@ -1851,8 +1981,10 @@ __global__ void __launch_bounds__(kAdjThreads<D>, 512 / kAdjThreads<D>) k_adj_ga
     // the first particle's state is requested before the node block is built, so the two overlap
     // (requesting its adjoint too, or staging the second particle in shared memory, measured slower)
     float r[Cfg<D>::S];
-    if (tid < cnt) load_planes<D, Cfg<D>::PLANES>(sp.planes, sp.npad, int(b.sorted[st + tid] & 0x3ffffffu), r);
-    build_node_block<D, TB, true>(b, sp, t, sv, sb);
+    if (tid < cnt)
+      load_planes<D, Cfg<D>::PLANES>(sp.planes, sp.npad, int((BINS ? ent0 : list[tid]) & 0x3ffffffu), r);
+    build_node_block<D, TB, true>(b, sp, BINS ? &bv : nullptr, t, sv, sb);
+    cp_async_wait_all();  // the actuations (readable by all after the barrier)
     __syncthreads();
     float lo = 0.0f, hi = 0.0f;  // per-warp group sums of (K), lane-owned
     for (int e0 = 0; e0 < cnt; e0 += blockDim.x) {
@@ -1860,7 +1992,7 @@ __global__ void __launch_bounds__(kAdjThreads<D>, 512 / kAdjThreads<D>) k_adj_ga
       int g = -1;
       float contrib = 0.0f;
       if (e < cnt) {
-        const int id = int(b.sorted[st + e] & 0x3ffffffu);
+        const int id = int(list[e] & 0x3ffffffu);
         if (e0 > 0) load_planes<D, Cfg<D>::PLANES>(sp.planes, sp.npad, id, r);
         Part<D> q, g1, g0;
         unpack<D>(r, q);
@@ -1955,62 +2087,65 @@ static bool wide_tiles(const BatchDev& b) {
 }
 
 template <int D, int TB>
-static cudaError_t keys_impl(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
-  if (sel) {  // at least one CTA: the selection is published even without particles
-    const int nblk = b.total_particles > 0 ? (b.total_particles + 255) / 256 : 1;
-    launch_pdl(k_keys<D, TB, true>, dim3(nblk), dim3(256), 0, s, b, sel);
-    count_launches(1);
-    return cudaGetLastError();
-  }
-  if (b.total_particles == 0) return cudaSuccess;
-  launch_pdl(k_keys<D, TB, false>, dim3((b.total_particles + 255) / 256), dim3(256), 0, s, b, sel);
+static cudaError_t keys_impl(const BatchDev& b, cudaStream_t s, const SelectPar* sel, int back, int* snap) {
+  // at least one CTA with a selection or bins: what it publishes is there even without particles
+  const int nblk = b.total_particles > 0 ? (b.total_particles + 255) / 256 : (sel || b.bin_ctl) ? 1 : 0;
+  if (nblk == 0) return cudaSuccess;
+  if (sel)
+    launch_pdl(k_keys<D, TB, true>, dim3(nblk), dim3(256), 0, s, b, sel, back, snap);
+  else
+    launch_pdl(k_keys<D, TB, false>, dim3(nblk), dim3(256), 0, s, b, sel, back, snap);
   count_launches(1);
   return cudaGetLastError();
 }
 
+cudaError_t reset_bins(const BatchDev& b, cudaStream_t s) {
+  if (!b.bin_ctl) return cudaSuccess;
+  return cudaMemsetAsync(b.bin_ctl, 0, sizeof(uint32_t) * bin_ctl_words(b.total_tiles), s);
+}
+
 template <int D>
-cudaError_t launch_keys(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
-  cudaError_t e = cudaMemsetAsync(b.tile_count, 0, sizeof(uint32_t) * size_t(b.total_tiles), s);
+cudaError_t launch_keys(const BatchDev& b, cudaStream_t s, const SelectPar* sel, bool reset, int back, int* snap) {
+  cudaError_t e = cudaSuccess;
+  if (!b.bin_ctl)
+    e = cudaMemsetAsync(b.tile_count, 0, sizeof(uint32_t) * size_t(b.total_tiles), s);
+  else if (reset)
+    e = reset_bins(b, s);
   if (e != cudaSuccess) return e;
   if constexpr (D == 2)
-    if (wide_tiles<D>(b)) return keys_impl<D, 8>(b, s, sel);
-  return keys_impl<D, 4>(b, s, sel);
+    if (wide_tiles<D>(b)) return keys_impl<D, 8>(b, s, sel, back, snap);
+  return keys_impl<D, 4>(b, s, sel, back, snap);
 }
 
 template <int D>
 cudaError_t launch_sort(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
-  if (fused_scan(b)) {  // scan inside the scatter; at least one CTA so the scan results are written
-    const int nblk = b.total_particles > 0 ? (b.total_particles + 255) / 256 : 1;
-    if (sel)
-      launch_pdl(k_scatter<D, true, true>, dim3(nblk + 1), dim3(256), 0, s, b, sel);
-    else
-      launch_pdl(k_scatter<D, true, false>, dim3(nblk), dim3(256), 0, s, b, sel);
-    count_launches(1);
-    return cudaGetLastError();
-  }
+  if (b.bin_ctl) return cudaSuccess;  // the particles are in their tiles' lists already
   const int nblk = (b.total_tiles + SCAN_TILE - 1) / SCAN_TILE;
   if (sel)
     launch_pdl(k_scan_reduce<true>, dim3(nblk + 1), dim3(SCAN_THREADS), 0, s, b, sel);
   else
     launch_pdl(k_scan_reduce<false>, dim3(nblk), dim3(SCAN_THREADS), 0, s, b, sel);
   launch_pdl(k_scan_down, dim3(nblk), dim3(SCAN_THREADS), 0, s, b);
-  if (b.total_particles > 0)
-    launch_pdl(k_scatter<D, false, false>, dim3((b.total_particles + 255) / 256), dim3(256), 0, s, b,
-               static_cast<const SelectPar*>(nullptr));
+  if (b.total_particles > 0) launch_pdl(k_scatter<D>, dim3((b.total_particles + 255) / 256), dim3(256), 0, s, b);
   count_launches((b.total_particles > 0 ? 1 : 0) + 2);
   return cudaGetLastError();
 }
 
-template <int D, int TB, bool ADJ>
-static cudaError_t p2g_configure() {
-  cudaError_t e = cudaFuncSetAttribute(k_p2g<D, TB, ADJ, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+template <int D, int TB, bool ADJ, bool BINS>
+static cudaError_t p2g_configure_lists() {
+  cudaError_t e = cudaFuncSetAttribute(k_p2g<D, TB, ADJ, 256, BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        int(P2GCfg<D, TB, ADJ, 256>::SMEM));
   if constexpr (D == 2) {
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_p2g<D, TB, ADJ, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      e = cudaFuncSetAttribute(k_p2g<D, TB, ADJ, 128, BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                int(P2GCfg<D, TB, ADJ, 128>::SMEM));
   }
   return e;
+}
+template <int D, int TB, bool ADJ>
+static cudaError_t p2g_configure() {
+  const cudaError_t e = p2g_configure_lists<D, TB, ADJ, false>();
+  return e == cudaSuccess ? p2g_configure_lists<D, TB, ADJ, true>() : e;
 }
 
 cudaError_t configure_kernels() {
@@ -2030,19 +2165,23 @@ static int tile_grid(const BatchDev& b, int k) {
   return grid < 1 ? 1 : grid;
 }
 
-template <int D, int TB, bool ADJ>
-static cudaError_t p2g_impl(const BatchDev& b, cudaStream_t s) {
+template <int D, int TB, bool ADJ, bool BINS>
+static cudaError_t p2g_lists(const BatchDev& b, cudaStream_t s) {
   const int k = ADJ ? TK_P2G_ADJ : TK_P2G;
   const int grid = tile_grid(b, k);
   bool small = false;  // 128-thread CTAs (2D only)
   if constexpr (D == 2) small = b.launch[k].threads == 128;
   if constexpr (D == 2) {
     if (small)
-      launch_pdl(k_p2g<D, TB, ADJ, 128>, dim3(grid), dim3(128), P2GCfg<D, TB, ADJ, 128>::SMEM, s, b);
+      launch_pdl(k_p2g<D, TB, ADJ, 128, BINS>, dim3(grid), dim3(128), P2GCfg<D, TB, ADJ, 128>::SMEM, s, b);
   }
-  if (!small) launch_pdl(k_p2g<D, TB, ADJ, 256>, dim3(grid), dim3(256), P2GCfg<D, TB, ADJ, 256>::SMEM, s, b);
+  if (!small) launch_pdl(k_p2g<D, TB, ADJ, 256, BINS>, dim3(grid), dim3(256), P2GCfg<D, TB, ADJ, 256>::SMEM, s, b);
   count_launches(1);
   return cudaGetLastError();
+}
+template <int D, int TB, bool ADJ>
+static cudaError_t p2g_impl(const BatchDev& b, cudaStream_t s) {
+  return b.bin_ctl ? p2g_lists<D, TB, ADJ, true>(b, s) : p2g_lists<D, TB, ADJ, false>(b, s);
 }
 
 template <int D>
@@ -2052,33 +2191,41 @@ cudaError_t launch_p2g(const BatchDev& b, bool with_adjoint, cudaStream_t s) {
   return with_adjoint ? p2g_impl<D, 4, true>(b, s) : p2g_impl<D, 4, false>(b, s);
 }
 
-template <int D, int TB>
-static cudaError_t g2p_impl(const BatchDev& b, cudaStream_t s) {
-  const int grid = tile_grid(b, TK_G2P);
+template <int D, int TB, bool BINS>
+static cudaError_t g2p_lists(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
+  const int grid = tile_grid(b, TK_G2P) + (sel ? 1 : 0);
   if (b.launch[TK_G2P].threads == 128)
-    launch_pdl(k_g2p<D, TB, 128>, dim3(grid), dim3(128), 0, s, b);
+    launch_pdl(k_g2p<D, TB, 128, BINS>, dim3(grid), dim3(128), 0, s, b, sel);
   else
-    launch_pdl(k_g2p<D, TB, 256>, dim3(grid), dim3(256), 0, s, b);
+    launch_pdl(k_g2p<D, TB, 256, BINS>, dim3(grid), dim3(256), 0, s, b, sel);
   count_launches(1);
   return cudaGetLastError();
+}
+template <int D, int TB>
+static cudaError_t g2p_impl(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
+  return b.bin_ctl ? g2p_lists<D, TB, true>(b, s, sel) : g2p_lists<D, TB, false>(b, s, nullptr);
 }
 
 template <int D>
-cudaError_t launch_g2p(const BatchDev& b, cudaStream_t s) {
+cudaError_t launch_g2p(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
   if constexpr (D == 2)
-    if (wide_tiles<D>(b)) return g2p_impl<D, 8>(b, s);
-  return g2p_impl<D, 4>(b, s);
+    if (wide_tiles<D>(b)) return g2p_impl<D, 8>(b, s, sel);
+  return g2p_impl<D, 4>(b, s, sel);
 }
 
-template <int D, int TB>
-static cudaError_t adj_gather_impl(const BatchDev& b, cudaStream_t s) {
+template <int D, int TB, bool BINS>
+static cudaError_t adj_gather_lists(const BatchDev& b, cudaStream_t s) {
   const int grid = tile_grid(b, TK_ADJ_GATHER);
   if (b.has_material)
-    launch_pdl(k_adj_gather<D, TB, true>, dim3(grid), dim3(kAdjThreads<D>), 0, s, b);
+    launch_pdl(k_adj_gather<D, TB, true, BINS>, dim3(grid), dim3(kAdjThreads<D>), 0, s, b);
   else
-    launch_pdl(k_adj_gather<D, TB, false>, dim3(grid), dim3(kAdjThreads<D>), 0, s, b);
+    launch_pdl(k_adj_gather<D, TB, false, BINS>, dim3(grid), dim3(kAdjThreads<D>), 0, s, b);
   count_launches(1);
   return cudaGetLastError();
+}
+template <int D, int TB>
+static cudaError_t adj_gather_impl(const BatchDev& b, cudaStream_t s) {
+  return b.bin_ctl ? adj_gather_lists<D, TB, true>(b, s) : adj_gather_lists<D, TB, false>(b, s);
 }
 
 template <int D>
@@ -2088,14 +2235,14 @@ cudaError_t launch_adj_gather(const BatchDev& b, cudaStream_t s) {
   return adj_gather_impl<D, 4>(b, s);
 }
 
-template cudaError_t launch_keys<2>(const BatchDev&, cudaStream_t, const SelectPar*);
-template cudaError_t launch_keys<3>(const BatchDev&, cudaStream_t, const SelectPar*);
+template cudaError_t launch_keys<2>(const BatchDev&, cudaStream_t, const SelectPar*, bool, int, int*);
+template cudaError_t launch_keys<3>(const BatchDev&, cudaStream_t, const SelectPar*, bool, int, int*);
 template cudaError_t launch_sort<2>(const BatchDev&, cudaStream_t, const SelectPar*);
 template cudaError_t launch_sort<3>(const BatchDev&, cudaStream_t, const SelectPar*);
 template cudaError_t launch_p2g<2>(const BatchDev&, bool, cudaStream_t);
 template cudaError_t launch_p2g<3>(const BatchDev&, bool, cudaStream_t);
-template cudaError_t launch_g2p<2>(const BatchDev&, cudaStream_t);
-template cudaError_t launch_g2p<3>(const BatchDev&, cudaStream_t);
+template cudaError_t launch_g2p<2>(const BatchDev&, cudaStream_t, const SelectPar*);
+template cudaError_t launch_g2p<3>(const BatchDev&, cudaStream_t, const SelectPar*);
 template cudaError_t launch_adj_gather<2>(const BatchDev&, cudaStream_t);
 template cudaError_t launch_adj_gather<3>(const BatchDev&, cudaStream_t);
 
@@ -2445,14 +2592,14 @@ __global__ void __launch_bounds__(PACK_THREADS) k_unpack(int N, int npad, const 
 // sinusoid controllers' actuation a_g(t_n) is evaluated here too.  Every step of a rollout is
 // then the same launch sequence, which CUDA graphs replay.  (A single tiled scene makes this
 // selection inside the first kernel of its step instead: k_keys, k_scatter, k_scan_reduce.)
-__global__ void k_select(const SelectPar* __restrict__ sel, ScenePar* __restrict__ cur) {
+__global__ void k_select(const SelectPar* __restrict__ sel, ScenePar* __restrict__ cur, const uint32_t* flip) {
   pdl_enter();
-  select_publish(sel[blockIdx.x], cur + blockIdx.x);
+  select_publish(sel[blockIdx.x], cur + (flip ? *flip & 1u : blockIdx.x));
 }
 
-cudaError_t launch_select(const SelectPar* sel, int n_scenes, ScenePar* cur, cudaStream_t s) {
+cudaError_t launch_select(const SelectPar* sel, int n_scenes, ScenePar* cur, cudaStream_t s, const uint32_t* flip) {
   if (n_scenes <= 0) return cudaSuccess;
-  launch_pdl(k_select, dim3(n_scenes), dim3(64), 0, s, sel, cur);
+  launch_pdl(k_select, dim3(n_scenes), dim3(64), 0, s, sel, cur, flip);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -138,6 +138,7 @@ struct mpm_scene {
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
   TuneState tune;
+  bool keys_stale = false;  // a batch advanced the state since its bin keys were made
   int batch_refs = 0;  // batch slots holding the scene (admitted, not yet released)
   // The segment recompute's own workspace (tile arrays, selected record, bin keys, actuation,
   // grid), so that mpm_backward can run it on the context's second stream beside the reverse

@@ -1,0 +1,89 @@
+"""Tile bins against the sort: scenes of at most 2048 tiles keep a list per tile that the step itself
+appends to, larger ones sort their particles by tile every step.  The same particles in a grid on
+either side of that line give the same bits (the grids differ only at walls nothing is near), over
+forward steps, checkpointed rollouts and their reverse passes.
+"""
+import numpy as np
+import pytest
+
+from paper_1810_01054_gb300 import scenes as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def M():
+    from paper_1810_01054_gb300 import mpm
+    return mpm
+
+
+@pytest.fixture(scope="module")
+def ctx(M):
+    c = M.Context(0)
+    yield c
+    c.close()
+
+
+def _body(dim, edge, ctrl, n):
+    """A blob that spans several tiles, on a fine grid (dx = 1/64), moving so that particles change
+    tiles, far from the high wall of the first axis."""
+    s = S.blob(dim, 64, 2500 if dim == 2 else 3000, 61, radius_cells=9.0 if dim == 2 else 6.0, v_scale=1.0,
+               c_scale=1.0, f_scale=0.03, center=[0.4] * dim, ctrl_type=ctrl, hidden=8, n_groups=3, amp=2.0,
+               bc_width=3, dt=2e-3)
+    v = np.array(s.v0)
+    v[:, 0] += 3.0  # 0.4 cells a step
+    return s.copy(n_grid=n, v0=v, tile_edge=edge if dim == 2 else 0)
+
+
+# grids of 2048 tiles (or fewer) and just above, by dimension and tile edge
+GRIDS = {(2, 4): ((256, 128), (260, 128)), (2, 8): ((512, 256), (520, 256)), (3, 4): ((64, 64, 32), (68, 64, 32))}
+
+
+@pytest.mark.parametrize("ctrl", [S.CTRL_SIN, S.CTRL_TABLE, S.CTRL_MLP, S.CTRL_COM])
+@pytest.mark.parametrize("shape", list(GRIDS))
+def test_bins_give_the_bits_of_the_sort(M, ctx, shape, ctrl):
+    dim, edge = shape
+    res = []
+    for n in GRIDS[shape]:
+        spec = _body(dim, edge, ctrl, n)
+        if dim == 3:  # the blob sits lower than the short third axis
+            x = np.array(spec.x0)
+            x[:, 2] -= 0.15
+            spec = spec.copy(x0=x)
+        got = []
+        for steps, k in ((11, 1), (11, 4), (3, 2)):  # graph lengths 8 + 3 and 3; segments of 4, 4, 3
+            sc = M.Scene(ctx, spec)
+            sc.rollout(steps, k)
+            got += list(sc.get_state())
+            seed = np.zeros((sc.N, dim))
+            seed[:, 0] = 1.0 / sc.N
+            got += list(sc.backward(seed))
+            sc.step(2)  # goes on from the rollout's end after its reverse pass
+            got += list(sc.get_state())
+            sc.close()
+        res.append(got)
+    assert np.abs(res[0][1] - _body(dim, edge, ctrl, GRIDS[shape][0]).v0).max() > 0.01
+    for a, b in zip(*res):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_steps_after_a_forward_only_batch_request(M, ctx, dim):
+    """A batch advances the scene's particles with lists of its own; stepping the scene afterwards
+    starts from the state the batch left."""
+    spec = _body(dim, 4, S.CTRL_SIN, (128, 96) if dim == 2 else (48, 48, 48))
+    alone = M.Scene(ctx, spec)
+    alone.step(13)
+    want = alone.get_state()
+    alone.close()
+    sc = M.Scene(ctx, spec)
+    batch = M.Batch(ctx, dim)
+    slot = batch.admit(sc, 9, False)
+    while not batch.poll(slot):
+        batch.tick(4)
+    batch.release(slot)
+    sc.step(4)
+    for a, b in zip(want, sc.get_state()):
+        assert np.array_equal(a, b)
+    batch.close()
+    sc.close()
