@@ -29,6 +29,10 @@ namespace gbmpm {
 namespace {
 
 constexpr int F64_THREADS = 256;
+// Most particles per SM that get three lanes each.  Forward + reverse step, one thread and three lanes
+// a particle: 628 particles (2D) 50.7 and 39.0 us, 4,800 (2D, 32 an SM) 57.0 and 45.6, 4,800 (3D) 246
+// and 174; beyond it every SM's FP64 pipe has several warps of its own.
+constexpr int SPLIT_PER_SM = 32;
 
 // Everything one FP64 launch reads: scene constants and the buffers of the step being run.
 struct Par64 {
@@ -47,6 +51,7 @@ struct Par64 {
   double* adj_out;         // adjoint of state n (reverse)
   double* grid;            // [nodes][4]
   double* grid_b;          // [nodes][4]
+  double *grid_next, *grid_b_next;  // the next step's grids, cleared by this step's grid update
   double* g_act;           // [G] dL/da of this step (reverse), nullptr = not wanted
   int* status;
 };
@@ -69,20 +74,26 @@ __device__ __forceinline__ void load64(const double* __restrict__ st, int N, int
 }
 
 template <int D>
-__device__ __forceinline__ void store64(double* __restrict__ st, int N, int p, const Part<D, double>& q) {
+__device__ __forceinline__ void store64(double* __restrict__ st, int N, int p, const Part<D, double>& q, int sub = 0,
+                                        int lanes = 1) {
+  // of several lanes that hold the particle each stores every lanes-th component
   int c = 0;
+  auto put = [&](double v) {
+    if (c % lanes == sub) st[size_t(c) * N + p] = v;
+    ++c;
+  };
 #pragma unroll
-  for (int a = 0; a < D; ++a) st[size_t(c++) * N + p] = q.x[a];
-#pragma unroll
-  for (int a = 0; a < D; ++a)
-#pragma unroll
-    for (int b = 0; b < D; ++b) st[size_t(c++) * N + p] = q.F[a][b];
-#pragma unroll
-  for (int a = 0; a < D; ++a) st[size_t(c++) * N + p] = q.v[a];
+  for (int a = 0; a < D; ++a) put(q.x[a]);
 #pragma unroll
   for (int a = 0; a < D; ++a)
 #pragma unroll
-    for (int b = 0; b < D; ++b) st[size_t(c++) * N + p] = q.C[a][b];
+    for (int b = 0; b < D; ++b) put(q.F[a][b]);
+#pragma unroll
+  for (int a = 0; a < D; ++a) put(q.v[a]);
+#pragma unroll
+  for (int a = 0; a < D; ++a)
+#pragma unroll
+    for (int b = 0; b < D; ++b) put(q.C[a][b]);
 }
 
 template <int D>
@@ -109,42 +120,81 @@ __device__ __forceinline__ double stress_G64(const Par64& p, const Part<D, doubl
   return J;
 }
 
-// Visits the stencil nodes of a particle: f(node linear index, N, dN/dx_p, d = x_i - x_p).
-template <int D, class Fn>
-__device__ __forceinline__ void for_stencil(const Sten<D, double>& s, const int* n, double dx, Fn fn) {
+// The thread's particle.  With L = 3 three neighbouring lanes share a particle (ten particles a
+// warp, two lanes idle), each working one x-slab of its stencil: a small scene's launch is bound by
+// one thread's chain of FP64 operations, and the slabs are independent.
+template <int L>
+struct Lane {
+  int id, sub, first;  // particle, slab, the particle's first lane
+  bool mine;           // a particle's lane (id may still be past the end)
+  __device__ __forceinline__ Lane() {
+    if constexpr (L == 1) {
+      id = blockIdx.x * blockDim.x + threadIdx.x;
+      sub = first = 0;
+      mine = true;
+    } else {
+      const int lane = threadIdx.x & 31;
+      sub = lane % 3;
+      first = lane - sub;
+      mine = lane < 30;
+      id = int((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 10 + lane / 3;
+    }
+  }
+  // sum of v over the particle's lanes (the lanes of `mask` call it, whole particles)
+  __device__ __forceinline__ double total(double v, unsigned mask) const {
+    if constexpr (L == 1) return v;
+    const double a = __shfl_sync(mask, v, first), b = __shfl_sync(mask, v, first + 1),
+                 c = __shfl_sync(mask, v, (first + 2) & 31);
+    return a + b + c;
+  }
+};
+
+// Visits the stencil nodes of a particle (with L = 3 those of x-slab sub): f(node linear index, N,
+// dN/dx_p, d = x_i - x_p).
+template <int D, int L, class Fn>
+__device__ __forceinline__ void for_stencil(const Sten<D, double>& s, const int* n, double dx, int sub, Fn fn) {
 #pragma unroll
-  for (int kx = 0; kx < 3; ++kx)
+  for (int jx = 0; jx < 3 / L; ++jx) {
+    // the slab's weights by value (a runtime index would put the arrays in local memory)
+    const int kx = L == 1 ? jx : sub;
+    const double wx = kx == 0 ? s.w[0][0] : (kx == 1 ? s.w[0][1] : s.w[0][2]);
+    const double dwx = kx == 0 ? s.dw[0][0] : (kx == 1 ? s.dw[0][1] : s.dw[0][2]);
 #pragma unroll
     for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
       for (int kz = 0; kz < (D == 3 ? 3 : 1); ++kz) {
         const int k[3] = {kx, ky, kz};
         int nd[D];
-        double N = 1.0, dN[D], d[D];
+        double N = 1.0, dN[D], d[D], w[D], dw[D];
 #pragma unroll
         for (int a = 0; a < D; ++a) {
+          w[a] = a == 0 ? wx : s.w[a][a == 1 ? ky : kz];
+          dw[a] = a == 0 ? dwx : s.dw[a][a == 1 ? ky : kz];
           nd[a] = s.base[a] + k[a];
-          N *= s.w[a][k[a]];
+          N *= w[a];
           d[a] = (double(k[a]) - s.f[a]) * dx;
         }
 #pragma unroll
         for (int a = 0; a < D; ++a) {
           double t = 1.0;
 #pragma unroll
-          for (int b = 0; b < D; ++b) t *= (a == b) ? s.dw[b][k[b]] : s.w[b][k[b]];
+          for (int b = 0; b < D; ++b) t *= (a == b) ? dw[b] : w[b];
           dN[a] = t;
         }
         fn(node_lin<D>(nd, n), N, dN, d);
       }
+  }
 }
 
 // P2G (Eqs. 3-5): m_i += N m_p, p_i += N (m_p v_p + G_p d).  With ADJ also the reverse step's
 // (A)-(C) scatter of state n+1's adjoint: vbar_i += N (vbar_p + (4/dx^2) Cbar_p d) with
 // vbar_p = vbar' + dt xbar' (A) and Cbar_p = Cbar' + dt Fbar' F^T (B).
-template <int D, bool ADJ>
+template <int D, bool ADJ, int L>
 __global__ void __launch_bounds__(F64_THREADS) k64_p2g(Par64 p) {
-  const int id = blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= p.N) return;
+  pdl_enter();
+  const Lane<L> ln;
+  const int id = ln.id;
+  if (!ln.mine || id >= p.N) return;
   Part<D, double> q;
   load64<D>(p.st, p.N, id, q);
   Sten<D, double> stn;
@@ -172,7 +222,7 @@ __global__ void __launch_bounds__(F64_THREADS) k64_p2g(Par64 p) {
       }
     }
   }
-  for_stencil<D>(stn, p.n, p.dx, [&](int nl, double N, const double*, const double* d) {
+  for_stencil<D, L>(stn, p.n, p.dx, ln.sub, [&](int nl, double N, const double*, const double* d) {
     double* gp = p.grid + size_t(nl) * 4;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -199,8 +249,14 @@ __global__ void __launch_bounds__(F64_THREADS) k64_p2g(Par64 p) {
 // (L) through the boundary, then (D) pbar = vbar / m and (E) mbar = -v . vbar / m.
 template <int D, bool ADJ>
 __global__ void __launch_bounds__(F64_THREADS) k64_grid(Par64 p, int n_nodes) {
+  pdl_enter();
   const int nl = blockIdx.x * blockDim.x + threadIdx.x;
   if (nl >= n_nodes) return;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {  // the next step's sums start from zero
+    p.grid_next[size_t(nl) * 4 + a] = 0.0;
+    if constexpr (ADJ) p.grid_b_next[size_t(nl) * 4 + a] = 0.0;
+  }
   int node[D];
   {
     int r = nl;
@@ -255,19 +311,24 @@ __global__ void __launch_bounds__(F64_THREADS) k64_grid(Par64 p, int n_nodes) {
 }
 
 // G2P (Eqs. 7-10): v = sum N v*, C = (4/dx^2) sum N v* d^T, F <- (I + dt C) F, x <- x + dt v.
-template <int D>
+template <int D, int L>
 __global__ void __launch_bounds__(F64_THREADS) k64_g2p(Par64 p) {
-  const int id = blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= p.N) return;
+  pdl_enter();
+  const Lane<L> ln;
+  const int id = ln.id;
+  const bool mine = ln.mine && id < p.N;
+  if (L == 1 && !mine) return;
   Part<D, double> q;
-  load64<D>(p.st, p.N, id, q);
   Sten<D, double> stn;
-  if (!make_stencil<D>(q.x, p.inv_dx, p.n, stn)) {  // status already set by P2G: carry the particle over
-    store64<D>(p.st_out, p.N, id, q);
-    return;
+  bool live = false;
+  if (mine) {
+    load64<D>(p.st, p.N, id, q);
+    live = make_stencil<D>(q.x, p.inv_dx, p.n, stn);
+    if (!live) store64<D>(p.st_out, p.N, id, q, ln.sub, L);  // status already set by P2G: carry the particle over
   }
+  if (L == 1 && !live) return;
   double vn[D] = {}, Cn[D][D] = {};
-  for_stencil<D>(stn, p.n, p.dx, [&](int nl, double N, const double*, const double* d) {
+  if (live) for_stencil<D, L>(stn, p.n, p.dx, ln.sub, [&](int nl, double N, const double*, const double* d) {
     const double* gp = p.grid + size_t(nl) * 4;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -277,6 +338,13 @@ __global__ void __launch_bounds__(F64_THREADS) k64_g2p(Par64 p) {
       for (int c = 0; c < D; ++c) Cn[a][c] += Nv * d[c];
     }
   });
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    vn[a] = ln.total(vn[a], 0xffffffffu);
+#pragma unroll
+    for (int c = 0; c < D; ++c) Cn[a][c] = ln.total(Cn[a][c], 0xffffffffu);
+  }
+  if (!live) return;
   Part<D, double> o;
 #pragma unroll
   for (int a = 0; a < D; ++a)
@@ -294,7 +362,7 @@ __global__ void __launch_bounds__(F64_THREADS) k64_g2p(Par64 p) {
     o.v[a] = vn[a];
     o.x[a] = q.x[a] + p.dt * vn[a];
   }
-  store64<D>(p.st_out, p.N, id, o);
+  store64<D>(p.st_out, p.N, id, o, ln.sub, L);
 }
 
 // Reverse G2P per particle, Supplement S4 (F)-(K) in their direct form:
@@ -306,18 +374,21 @@ __global__ void __launch_bounds__(F64_THREADS) k64_g2p(Par64 p) {
 //   (K) dL/da_g += dir_g . diag(F^T Pbar)
 // with vbar_p, Cbar_p the (A), (B) totals of state n+1's adjoint.  Block-level group sums of (K)
 // go to g_act with one atomic per group and block.
-template <int D>
+template <int D, int L>
 __global__ void __launch_bounds__(F64_THREADS) k64_adjoint(Par64 p) {
+  pdl_enter();
   __shared__ double gsum[MAX_GROUPS];
   const bool want_act = p.g_act != nullptr && p.G > 0;
   if (want_act) {
     for (int g = threadIdx.x; g < p.G; g += blockDim.x) gsum[g] = 0.0;
     __syncthreads();
   }
-  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  const Lane<L> ln;
+  const int id = ln.id;
   Sten<D, double> stn;
   Part<D, double> q;
-  const bool live = id < p.N && (load64<D>(p.st, p.N, id, q), make_stencil<D>(q.x, p.inv_dx, p.n, stn));
+  const bool live = ln.mine && id < p.N && (load64<D>(p.st, p.N, id, q), make_stencil<D>(q.x, p.inv_dx, p.n, stn));
+  const unsigned some = L == 1 ? 0u : __ballot_sync(0xffffffffu, live);
   if (live) {
     Part<D, double> g1, g0;
     load64<D>(p.adj_in, p.N, id, g1);
@@ -338,7 +409,7 @@ __global__ void __launch_bounds__(F64_THREADS) k64_adjoint(Par64 p) {
       }
     }
     double gxs[D] = {}, sv[D] = {}, spb[D] = {}, Cn[D][D] = {}, Gb[D][D] = {};
-    for_stencil<D>(stn, p.n, p.dx, [&](int nl, double N, const double* dN, const double* d) {
+    for_stencil<D, L>(stn, p.n, p.dx, ln.sub, [&](int nl, double N, const double* dN, const double* d) {
       const double* gv = p.grid + size_t(nl) * 4;
       const double* gb = p.grid_b + size_t(nl) * 4;
       double si = p.mass * gb[3];
@@ -364,6 +435,17 @@ __global__ void __launch_bounds__(F64_THREADS) k64_adjoint(Par64 p) {
         }
       }
     });
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      gxs[a] = ln.total(gxs[a], some);
+      sv[a] = ln.total(sv[a], some);
+      spb[a] = ln.total(spb[a], some);
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        Cn[a][c] = ln.total(Cn[a][c], some);
+        Gb[a][c] = ln.total(Gb[a][c], some);
+      }
+    }
     double Pb[D][D];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -396,8 +478,8 @@ __global__ void __launch_bounds__(F64_THREADS) k64_adjoint(Par64 p) {
         }
         g0.F[a][c] = s + H[a][c] + Pb[a][c] * sig[c] + p.kG * t;  // (H)
       }
-    store64<D>(p.adj_out, p.N, id, g0);
-    if (want_act && grp >= 0) {  // (K)
+    store64<D>(p.adj_out, p.N, id, g0, ln.sub, L);
+    if (want_act && grp >= 0 && ln.sub == 0) {  // (K)
       double contrib = 0.0;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
@@ -428,24 +510,40 @@ Shape shape_for(int n, int sms) {
   return {std::max(1, (n + t - 1) / t), t};
 }
 
+// Three lanes a particle while the launch leaves the FP64 pipes idle: the particle's set-up runs on
+// every lane, so it costs pipe time that a larger scene has a use for.
+bool split_particles(int n, int sms) { return n <= SPLIT_PER_SM * sms; }
+
+// Launches a particle kernel: k1 with a thread, k3 with three lanes a particle.
+void launch_particles(void (*k1)(Par64), void (*k3)(Par64), const Par64& p, mpm_ctx* c, cudaStream_t s) {
+  if (split_particles(p.N, c->sm_count)) {
+    launch_pdl(k3, dim3((p.N + 9) / 10), dim3(32), 0, s, p);
+  } else {
+    const Shape sh = shape_for(p.N, c->sm_count);
+    launch_pdl(k1, dim3(sh.blocks), dim3(sh.threads), 0, s, p);
+  }
+}
+
+// The step's kernels are programmatic dependents of one another, and the grid update clears the next
+// step's grid, so a step has no launch of its own for that (the 628-particle discs, with the lanes:
+// 57.0 -> 41.3 us a forward and reverse step).
+template <int D, bool ADJ>
+void launch_grid64(const Par64& p, int n_nodes, mpm_ctx* c, cudaStream_t s) {
+  ProfScope ps(c, s, MPM_K_F64_GRID);
+  const Shape sh = shape_for(n_nodes, c->sm_count);
+  launch_pdl(k64_grid<D, ADJ>, dim3(sh.blocks), dim3(sh.threads), 0, s, p, n_nodes);
+}
+
 template <int D>
 cudaError_t launch_step64(const Par64& p, int n_nodes, mpm_ctx* c, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(p.grid, 0, sizeof(double) * 4 * size_t(n_nodes), s);
-  if (e != cudaSuccess) return e;
   if (p.N > 0) {
     ProfScope ps(c, s, MPM_K_F64_P2G);
-    const Shape sh = shape_for(p.N, c->sm_count);
-    k64_p2g<D, false><<<sh.blocks, sh.threads, 0, s>>>(p);
+    launch_particles(k64_p2g<D, false, 1>, k64_p2g<D, false, 3>, p, c, s);
   }
-  {
-    ProfScope ps(c, s, MPM_K_F64_GRID);
-    const Shape sh = shape_for(n_nodes, c->sm_count);
-    k64_grid<D, false><<<sh.blocks, sh.threads, 0, s>>>(p, n_nodes);
-  }
+  launch_grid64<D, false>(p, n_nodes, c, s);
   if (p.N > 0) {
     ProfScope ps(c, s, MPM_K_F64_G2P);
-    const Shape sh = shape_for(p.N, c->sm_count);
-    k64_g2p<D><<<sh.blocks, sh.threads, 0, s>>>(p);
+    launch_particles(k64_g2p<D, 1>, k64_g2p<D, 3>, p, c, s);
   }
   count_launches(p.N > 0 ? 3 : 1);
   return cudaGetLastError();
@@ -453,23 +551,14 @@ cudaError_t launch_step64(const Par64& p, int n_nodes, mpm_ctx* c, cudaStream_t 
 
 template <int D>
 cudaError_t launch_reverse64(const Par64& p, int n_nodes, mpm_ctx* c, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(p.grid, 0, sizeof(double) * 4 * size_t(n_nodes), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p.grid_b, 0, sizeof(double) * 4 * size_t(n_nodes), s);
-  if (e != cudaSuccess) return e;
   if (p.N > 0) {
     ProfScope ps(c, s, MPM_K_F64_P2G_ADJ);
-    const Shape sh = shape_for(p.N, c->sm_count);
-    k64_p2g<D, true><<<sh.blocks, sh.threads, 0, s>>>(p);
+    launch_particles(k64_p2g<D, true, 1>, k64_p2g<D, true, 3>, p, c, s);
   }
-  {
-    ProfScope ps(c, s, MPM_K_F64_GRID);
-    const Shape sh = shape_for(n_nodes, c->sm_count);
-    k64_grid<D, true><<<sh.blocks, sh.threads, 0, s>>>(p, n_nodes);
-  }
+  launch_grid64<D, true>(p, n_nodes, c, s);
   if (p.N > 0) {
     ProfScope ps(c, s, MPM_K_F64_ADJ);
-    const Shape sh = shape_for(p.N, c->sm_count);
-    k64_adjoint<D><<<sh.blocks, sh.threads, 0, s>>>(p);
+    launch_particles(k64_adjoint<D, 1>, k64_adjoint<D, 3>, p, c, s);
   }
   count_launches(p.N > 0 ? 3 : 1);
   return cudaGetLastError();
@@ -513,6 +602,12 @@ mpm_status cuda_status(cudaError_t e) {
   do {                                                \
     cudaError_t e_ = (expr);                          \
     if (e_ != cudaSuccess) return cuda_status(e_);    \
+  } while (0)
+
+#define CKS64(expr)              \
+  do {                           \
+    mpm_status s_ = (expr);      \
+    if (s_ != MPM_OK) return s_; \
   } while (0)
 
 template <class T>
@@ -593,13 +688,32 @@ void drop_graphs(mpm_scene64* s) {
   }
 }
 
+// The grids are held twice: the i-th step of a pass sums into one pair while its grid update clears
+// the other.  The first step's pair is cleared when the pass starts.
+mpm_status clear_grids(mpm_scene64* s, cudaStream_t str) {
+  CK64(cudaMemsetAsync(s->hp.grid, 0, sizeof(double) * 8 * size_t(s->n_nodes), str));
+  return MPM_OK;
+}
+
+// Scene constants and the grids of the i-th step of a pass.
+Par64 step_par(const mpm_scene64* s, int i) {
+  Par64 p = s->hp;
+  const size_t pair = size_t(8) * s->n_nodes, odd = size_t(i & 1) * pair;
+  p.grid = s->hp.grid + odd;
+  p.grid_b = p.grid + pair / 2;
+  p.grid_next = s->hp.grid + (pair - odd);
+  p.grid_b_next = p.grid_next + pair / 2;
+  return p;
+}
+
 // The T steps of a rollout from the initial state (status cleared first).
 mpm_status enqueue_rollout(mpm_scene64* s, int T, cudaStream_t str) {
+  CKS64(clear_grids(s, str));
   const size_t stride = size_t(s->S) * std::max(1, s->N);
   CK64(cudaMemsetAsync(s->hp.status, 0, sizeof(int), str));
   CK64(cudaMemcpyAsync(s->hist, s->init, sizeof(double) * stride, cudaMemcpyDeviceToDevice, str));
   for (int t = 0; t < T; ++t) {
-    Par64 p = s->hp;
+    Par64 p = step_par(s, t);
     p.st = s->hist + size_t(t) * stride;
     p.st_out = s->hist + size_t(t + 1) * stride;
     p.act = step_act(s, t);
@@ -611,11 +725,12 @@ mpm_status enqueue_rollout(mpm_scene64* s, int T, cudaStream_t str) {
 
 // The reverse steps T-1 .. 0 (adjoint of state T in adj[0]; that of state 0 ends in adj[T & 1]).
 mpm_status enqueue_reverse(mpm_scene64* s, int T, cudaStream_t str) {
+  CKS64(clear_grids(s, str));
   const size_t stride = size_t(s->S) * std::max(1, s->N);
   if (size_t(s->L) * s->G > 0) CK64(cudaMemsetAsync(s->g_act, 0, sizeof(double) * size_t(s->L) * s->G, str));
   int cur = 0;
   for (int t = T - 1; t >= 0; --t) {
-    Par64 p = s->hp;
+    Par64 p = step_par(s, T - 1 - t);
     p.st = s->hist + size_t(t) * stride;
     p.adj_in = s->adj[cur];
     p.adj_out = s->adj[cur ^ 1];
@@ -750,8 +865,7 @@ mpm_status mpm64_create(mpm_ctx* c, const mpm_scene64_desc* d, mpm_scene64** out
   if ((st = alloc64(s, &s->init, SN)) != MPM_OK) return fail(st);
   if ((st = alloc64(s, &s->adj[0], SN)) != MPM_OK) return fail(st);
   if ((st = alloc64(s, &s->adj[1], SN)) != MPM_OK) return fail(st);
-  if ((st = alloc64(s, &p.grid, size_t(4) * s->n_nodes)) != MPM_OK) return fail(st);
-  if ((st = alloc64(s, &p.grid_b, size_t(4) * s->n_nodes)) != MPM_OK) return fail(st);
+  if ((st = alloc64(s, &p.grid, size_t(16) * s->n_nodes)) != MPM_OK) return fail(st);  // two pairs (step_par)
   if ((st = alloc64(s, &group, std::max(1, s->N))) != MPM_OK) return fail(st);
   if ((st = alloc64(s, &act_dir, std::max(1, s->G * dim))) != MPM_OK) return fail(st);
   if ((st = alloc64(s, &p.status, 1)) != MPM_OK) return fail(st);
