@@ -2042,6 +2042,9 @@ mpm_status mpm_set_ctrl_params(mpm_scene* s, const float* params, int n, int mem
   CK(cudaStreamSynchronize(s->ctx->stream));
   CK(cudaMemcpy(const_cast<float*>(s->ctrl.params), params, sizeof(float) * n,
                 mem_space == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice));
+  // a device-to-device copy may still run when the call returns, and the controller kernels read the
+  // parameters ahead of their place in the stream
+  if (mem_space == 1) CK(cudaStreamSynchronize(cudaStreamLegacy));
   return MPM_OK;
 }
 

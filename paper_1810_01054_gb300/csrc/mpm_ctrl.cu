@@ -18,17 +18,18 @@ constexpr int RED_STRIDE = MAX_GROUPS * 3 + 3;    // floats per row: [64 groups]
 
 int reduction_rows(int N) { return (N + RED_ROW - 1) / RED_ROW; }
 
-// Group sums of x (mode 0) or v (mode 2), dim channels, and the body sum, over the particles in
-// group order: perm lists the particles by group (stable; ungrouped first) and pgroup[i] is the
+// Group sums of x (blockIdx.y 0) or v (1, the closed-loop form), dim channels, and the body sum, over
+// the particles in group order: perm lists the particles by group (stable; ungrouped first) and pgroup[i] is the
 // group of perm[i] (-1: none), both fixed at scene creation.  A warp takes 32 consecutive entries
 // at a time, where every group is one run of lanes: a segmented scan over the lanes gives each
 // run's sum at its last lane, which adds it to the warp's accumulator of that group (one writer
 // per group and chunk, chunks in order).  Warps then combine in warp order into the block's row.
 template <int CH>
 __global__ void __launch_bounds__(256) k_group_rows(const ScenePar* __restrict__ dsp, float* __restrict__ rows,
-                                                    int mode, const int* __restrict__ perm,
+                                                    const int* __restrict__ perm,
                                                     const int* __restrict__ pgroup, const uint32_t* flip) {
   pdl_enter();
+  const bool velocity = blockIdx.y > 0;
   const ScenePar& sp = dsp[flip ? *flip : 0u];
   __shared__ float wacc[RED_WARPS][MAX_GROUPS][CH];
   __shared__ float wbody[RED_WARPS][CH];
@@ -57,7 +58,7 @@ __global__ void __launch_bounds__(256) k_group_rows(const ScenePar* __restrict__
     if (i < sp.N) {
       const int p = perm[i];
       gk[k] = pgroup[i];
-      if (mode == 0) {
+      if (!velocity) {
         const float4 q = sp.planes[p];
         const float xv[3] = {q.x, q.y, q.z};
 #pragma unroll
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(256) k_group_rows(const ScenePar* __restrict__
     if (lane == 0) wbody[w][c] = b;
   }
   __syncthreads();
-  float* row = rows + size_t(blockIdx.x) * RED_STRIDE;
+  float* row = rows + (size_t(blockIdx.y) * gridDim.x + blockIdx.x) * RED_STRIDE;
   for (int i = threadIdx.x; i < MAX_GROUPS * CH; i += blockDim.x) {
     const int g = i / CH, c = i - g * CH;
     float s = 0.0f;
@@ -121,7 +122,9 @@ __global__ void __launch_bounds__(256) k_group_rows(const ScenePar* __restrict__
 
 // Sum rows in a fixed order into out[g*3+c] (groups) and out[192+c] (body); 1024-thread CTA.  Only
 // the U = (G + 1) CH outputs in use are summed, each by S = 1024 / U interleaved splits combined
-// in split order; the other outputs are set to zero.
+// in split order; the other outputs are set to zero.  The row loops here and in ctrl_group_sums are
+// unrolled so that eight loads are in flight: one at a time, a trip to L2 per row was most of these
+// kernels' time (1,024 particles, table controller, 48 steps with the reverse pass 1993 -> 1815 us).
 __device__ void reduce_rows(const float* __restrict__ rows, int n_rows, int G, int CH, float* out) {
   __shared__ float part[1024];
   const int O = MAX_GROUPS * 3 + 3;  // outputs
@@ -132,6 +135,7 @@ __device__ void reduce_rows(const float* __restrict__ rows, int n_rows, int G, i
   float acc = 0.0f;
   if (s < S) {
     const int o = out_index(u);
+#pragma unroll 8
     for (int r = s; r < n_rows; r += S) acc += rows[size_t(r) * RED_STRIDE + o];
   }
   part[threadIdx.x] = acc;
@@ -168,18 +172,19 @@ __device__ __forceinline__ void dot_rows(const float* A, int so, int sj, const f
 
 // The MLP's parameters (W1, b1, W2, b2, W3, b3, contiguous) copied to shared memory in one pass
 // when they fit (the soft body's 48-64-64-16 network: 8336 floats), so the layers read no global
-// memory; else the global copy.  Every thread calls it; it ends with a barrier either way.
+// memory; else the global copy.  Asynchronous copies, requested before pdl_enter() (parameters only
+// change between launches, behind a wait for the stream), so they arrive while the kernel before
+// still runs; mlp_params_ready() before the barrier that precedes their use.  Every thread calls both.
 constexpr int MLP_STAGE = 8704;
-__device__ const float* mlp_params(const CtrlPar& c) {
-  __shared__ float stage[MLP_STAGE];
+__device__ __forceinline__ const float* mlp_params(const CtrlPar& c, float* stage) {
   const int G = c.G, Z = G * c.dim, H = c.hidden;
   const int n = H * Z + H + H * H + H + G * H + G;
-  const bool fits = n <= MLP_STAGE;  // uniform
-  if (fits)
-    for (int i = threadIdx.x; i < n; i += blockDim.x) stage[i] = c.params[i];
-  __syncthreads();
-  return fits ? stage : c.params;
+  if (n > MLP_STAGE) return c.params;  // uniform
+  for (int i = threadIdx.x; i < n; i += blockDim.x) cp_async4(stage + i, c.params + i);
+  cp_async_commit();
+  return stage;
 }
+__device__ __forceinline__ void mlp_params_ready() { cp_async_wait_all(); }
 
 // The MLP's three layers from its input z (shared): h1, h2 (shared) and fin3(g, u3), u3 the last
 // layer's pre-activation, with parameters P (mlp_params).  The forward and the reverse step's
@@ -206,6 +211,8 @@ __device__ __forceinline__ void mlp_layers(const CtrlPar& c, const float* P, con
 // selection): group centroids from the partial rows, then the three tanh layers -> sp.act.
 __global__ void __launch_bounds__(1024) k_ctrl_forward(const ScenePar* __restrict__ dsp, CtrlPar c, const float* rows,
                                                        int n_rows, const uint32_t* flip) {
+  __shared__ float stage[MLP_STAGE];
+  const float* P = mlp_params(c, stage);
   pdl_enter();
   const ScenePar& sp = dsp[flip ? *flip : 0u];
   __shared__ float red[MAX_GROUPS * 3 + 3];
@@ -222,7 +229,8 @@ __global__ void __launch_bounds__(1024) k_ctrl_forward(const ScenePar* __restric
     cen[tid] = cg;
     if (tid < dim) cen[Z + tid] = cb;
   }
-  const float* P = mlp_params(c);  // its barrier also publishes z
+  mlp_params_ready();
+  __syncthreads();  // the parameters and z
   mlp_layers(c, P, z, h1, h2, [&](int g, float u) { sp.act[g] = c.scale * tanhf(u); });
 }
 
@@ -289,6 +297,7 @@ __device__ void ctrl_group_sums(const CtrlPar& c, int lo, int hi, float* ga, flo
   const int g = tid & (MAX_GROUPS - 1), split = tid >> 6;
   float acc = 0.0f;
   if (g < G)
+#pragma unroll 8
     for (int r = lo + split; r < hi; r += 16) acc += c.gpart[size_t(r) * MAX_GROUPS + g];
   part[split][g] = acc;
   __syncthreads();
@@ -321,8 +330,24 @@ __device__ void ctrl_open_params(const CtrlPar& c, int n, float t, const float* 
 
 // STATE: the forms that read the state (closed loop, MLP) are compiled in; without it the kernel
 // handles only the open-loop forms and needs no room for the MLP's parameters.
+// This step's parameter adjoint added to gp[0, n): gp[i] = f(i, gp[i]), eight loads in flight per
+// thread (one parameter at a time, each waiting for its own load, took a third of the MLP's kernel).
+template <class F>
+__device__ __forceinline__ void add_params(float* gp, int n, F f) {
+  constexpr int K = 8;
+  for (int i0 = threadIdx.x; i0 < n; i0 += K * blockDim.x) {
+    float v[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = i0 + k * int(blockDim.x) < n ? gp[i0 + k * blockDim.x] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (i0 + k * int(blockDim.x) < n) gp[i0 + k * blockDim.x] = f(i0 + k * int(blockDim.x), v[k]);
+  }
+}
+
+// P: the MLP's parameters as mlp_params returned them.
 template <bool STATE>
-__device__ void ctrl_backward_body(const ScenePar& sp, const CtrlPar& c) {
+__device__ void ctrl_backward_body(const ScenePar& sp, const CtrlPar& c, const float* P) {
   __shared__ float ga[MAX_GROUPS], z[MAX_GROUPS * 3], h1[MAX_HIDDEN], h2[MAX_HIDDEN], o3[MAX_GROUPS];
   __shared__ float gu3[MAX_GROUPS], gu2[MAX_HIDDEN], gu1[MAX_HIDDEN];
   int* step_ctr = sp.step_ctr;
@@ -355,60 +380,61 @@ __device__ void ctrl_backward_body(const ScenePar& sp, const CtrlPar& c) {
   } else if (c.type == 4) {  // closed loop: z of this step as its forward kept it
     const int dim = c.dim, Z = dim * (1 + 2 * G);
     const float* cen = sp.ctrl_z ? sp.ctrl_z : c.centroid;
-    __shared__ float gu4[MAX_GROUPS];
+    __shared__ float gu4[MAX_GROUPS], zc[3 * (1 + 2 * MAX_GROUPS)], gt[3];
     const float* b = c.params + dim + size_t(G) * Z;
-    dot_rows(c.params + dim, Z, 1, cen, Z, G, [&](int g, float u) {
+    if (tid < Z) zc[tid] = cen[tid];
+    __syncthreads();
+    dot_rows(c.params + dim, Z, 1, zc, Z, G, [&](int g, float u) {
       const float th = tanhf(u + b[g]);
       gu4[g] = ga[g] * c.scale * (1.0f - th * th);
-      c.gparams[dim + size_t(G) * Z + g] += gu4[g];  // b
     });
     __syncthreads();
-    for (int i = tid; i < G * Z; i += blockDim.x) c.gparams[dim + i] += gu4[i / Z] * cen[i % Z];  // W
     // dL/dz: the target's part goes to its parameters, the group means' to gz
     dot_rows(c.params + dim, 1, Z, gu4, G, Z, [&](int j, float u) {
       if (j < dim)
-        c.gparams[j] += u;
+        gt[j] = u;
       else
         c.gz[j - dim] = u;  // [c_g part (G*dim)][u_g part (G*dim)]
     });
+    __syncthreads();
+    add_params(c.gparams, dim + G * Z + G, [&](int i, float old) {
+      if (i < dim) return old + gt[i];
+      i -= dim;
+      if (i < G * Z) return fmaf(gu4[i / Z], zc[i % Z], old);
+      return old + gu4[i - G * Z];
+    });
   } else {
     const int dim = c.dim, Z = G * dim, H = c.hidden;
-    const float* P = mlp_params(c);
     const float* W1 = P;
-    const float* b1 = W1 + H * Z;
-    const float* W2 = b1 + H;
-    const float* b2 = W2 + H * H;
-    const float* W3 = b2 + H;
-    float* gW1 = c.gparams;
-    float* gb1 = gW1 + H * Z;
-    float* gW2 = gb1 + H;
-    float* gb2 = gW2 + H * H;
-    float* gW3 = gb2 + H;
-    float* gb3 = gW3 + G * H;
+    const float* W2 = W1 + H * Z + H;
+    const float* W3 = W2 + H * H + H;
     // forward replay from the centroids of this step (kept by k_ctrl_forward)
     const float* cen = sp.ctrl_z ? sp.ctrl_z : c.centroid;
     if (tid < Z) z[tid] = cen[tid] - cen[Z + tid % dim];
+    mlp_params_ready();
     __syncthreads();
     mlp_layers(c, P, z, h1, h2, [&](int g, float u) {
       o3[g] = tanhf(u);
       gu3[g] = ga[g] * c.scale * (1.0f - o3[g] * o3[g]);
-      gb3[g] += gu3[g];
     });
     __syncthreads();
-    for (int i = tid; i < G * H; i += blockDim.x) gW3[i] += gu3[i / H] * h2[i % H];
-    dot_rows(W3, 1, H, gu3, G, H, [&](int i, float u) {
-      gu2[i] = u * (1.0f - h2[i] * h2[i]);
-      gb2[i] += gu2[i];
-    });
+    dot_rows(W3, 1, H, gu3, G, H, [&](int i, float u) { gu2[i] = u * (1.0f - h2[i] * h2[i]); });
     __syncthreads();
-    for (int i = tid; i < H * H; i += blockDim.x) gW2[i] += gu2[i / H] * h1[i % H];
-    dot_rows(W2, 1, H, gu2, H, H, [&](int i, float u) {
-      gu1[i] = u * (1.0f - h1[i] * h1[i]);
-      gb1[i] += gu1[i];
-    });
+    dot_rows(W2, 1, H, gu2, H, H, [&](int i, float u) { gu1[i] = u * (1.0f - h1[i] * h1[i]); });
     __syncthreads();
-    for (int i = tid; i < H * Z; i += blockDim.x) gW1[i] += gu1[i / Z] * z[i % Z];
     dot_rows(W1, 1, Z, gu1, H, Z, [&](int j, float u) { c.gz[j] = u; });
+    add_params(c.gparams, H * Z + H + H * H + H + G * H + G, [&](int i, float old) {
+      if (i < H * Z) return fmaf(gu1[i / Z], z[i % Z], old);
+      i -= H * Z;
+      if (i < H) return old + gu1[i];
+      i -= H;
+      if (i < H * H) return fmaf(gu2[i / H], h1[i % H], old);
+      i -= H * H;
+      if (i < H) return old + gu2[i];
+      i -= H;
+      if (i < G * H) return fmaf(gu3[i / H], h2[i % H], old);
+      return old + gu3[i - G * H];
+    });
   }
   __syncthreads();
   if (tid == 0) *step_ctr = n - 1;
@@ -417,8 +443,13 @@ __device__ void ctrl_backward_body(const ScenePar& sp, const CtrlPar& c) {
 template <bool STATE>
 __global__ void __launch_bounds__(1024) k_ctrl_backward(const ScenePar* __restrict__ dsp, CtrlPar c,
                                                         const uint32_t* flip) {
+  const float* P = nullptr;
+  if constexpr (STATE) {
+    __shared__ float stage[MLP_STAGE];
+    if (c.type == 2) P = mlp_params(c, stage);
+  }
   pdl_enter();
-  ctrl_backward_body<STATE>(dsp[flip ? *flip : 0u], c);
+  ctrl_backward_body<STATE>(dsp[flip ? *flip : 0u], c, P);
 }
 
 // Reverse of a form that reads no state for one step of a scene alone: the adjoint gather of the
@@ -438,7 +469,9 @@ __global__ void __launch_bounds__(1024) k_ctrl_backward_open(CtrlPar c, const in
 __global__ void __launch_bounds__(1024) k_ctrl_backward_multi(const ScenePar* __restrict__ cur,
                                                               const CtrlPar* __restrict__ cs) {
   pdl_enter();
-  ctrl_backward_body<true>(cur[blockIdx.x], cs[blockIdx.x]);
+  __shared__ float stage[MLP_STAGE];
+  const CtrlPar& c = cs[blockIdx.x];
+  ctrl_backward_body<true>(cur[blockIdx.x], c, c.type == 2 ? mlp_params(c, stage) : nullptr);
 }
 
 // x (and, for the closed-loop form, v) adjoint of the controller input: the MLP's centroids
@@ -493,15 +526,12 @@ cudaError_t ctrl_step_forward(const ScenePar& sp, const ScenePar* dsp, const Ctr
   const bool com = c.type == 4;
   int n = 0;
   if (rows > 0) {
-    float* vrows = c.partials + size_t(rows) * RED_STRIDE;
-    if (sp.dim == 2) {
-      launch_pdl(k_group_rows<2>, dim3(rows), dim3(256), 0, s, dsp, c.partials, 0, c.perm, c.pgroup, flip);
-      if (com) launch_pdl(k_group_rows<2>, dim3(rows), dim3(256), 0, s, dsp, vrows, 2, c.perm, c.pgroup, flip);
-    } else {
-      launch_pdl(k_group_rows<3>, dim3(rows), dim3(256), 0, s, dsp, c.partials, 0, c.perm, c.pgroup, flip);
-      if (com) launch_pdl(k_group_rows<3>, dim3(rows), dim3(256), 0, s, dsp, vrows, 2, c.perm, c.pgroup, flip);
-    }
-    n += com ? 2 : 1;
+    const dim3 grid(rows, com ? 2 : 1);
+    if (sp.dim == 2)
+      launch_pdl(k_group_rows<2>, grid, dim3(256), 0, s, dsp, c.partials, c.perm, c.pgroup, flip);
+    else
+      launch_pdl(k_group_rows<3>, grid, dim3(256), 0, s, dsp, c.partials, c.perm, c.pgroup, flip);
+    n += 1;
   }
   if (com)
     launch_pdl(k_ctrl_forward_com, dim3(1), dim3(1024), 0, s, dsp, c, c.partials, rows, flip);
