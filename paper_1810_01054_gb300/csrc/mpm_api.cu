@@ -188,6 +188,7 @@ mpm_status storage_order(mpm_scene* s, const mpm_scene_desc* d, int dim) {
   };
   pass(cell, cells, s->h_order, by_cell);        // stable by cell
   pass(tile, p.n_tiles + 1, by_cell, s->h_order);  // then stable by tile
+  int occupied = 0, last_tile = -1;
   // within each (tile, cell) run: by position, then caller index
   auto before = [&](int i, int j) {
     for (int a = 0; a < dim; ++a) {
@@ -203,8 +204,11 @@ mpm_status storage_order(mpm_scene* s, const mpm_scene_desc* d, int dim) {
     while (r1 < N && tile[s->h_order[r1]] == t0 && cell[s->h_order[r1]] == c0) ++r1;
     if (t0 < p.n_tiles)  // finite positions only (a NaN has no order)
       std::sort(s->h_order.begin() + r0, s->h_order.begin() + r1, before);
+    if (t0 < p.n_tiles && t0 != last_tile) ++occupied;
+    last_tile = t0;
     r0 = r1;
   }
+  s->b.occupied = occupied;
   int* dorder = nullptr;
   CKS(dalloc(&dorder, size_t(N), s->allocs));
   CK(cudaMemcpy(dorder, s->h_order.data(), sizeof(int) * size_t(N), cudaMemcpyHostToDevice));

@@ -251,8 +251,11 @@ mpm_status compose(mpm_batch* B, SubBatch& sb) {
     sb.key_particles = particles;
     sb.key_tiles = tiles;
   }
-  sb.b.has_material = 0;
-  for (int m : sb.members) sb.b.has_material |= B->slots[m].s->hp.gmat ? 1 : 0;
+  sb.b.has_material = sb.b.occupied = 0;
+  for (int m : sb.members) {
+    sb.b.has_material |= B->slots[m].s->hp.gmat ? 1 : 0;
+    sb.b.occupied += B->slots[m].s->b.occupied;
+  }
   sb.need_keys = true;
   return MPM_OK;
 }

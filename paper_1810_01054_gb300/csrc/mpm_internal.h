@@ -169,6 +169,7 @@ struct BatchDev {
   float4* partial_b;    // [total_tiles * BLOCK_NODES] node blocks of the adjoint scatter
   float* gpartial;      // [total_tiles * MAX_GROUPS] per active tile group sums of dL/da
   int tile_edge;                // cells per tile edge of every scene in the batch (0 or 4; 8: 2D)
+  int occupied;                 // tiles that held particles when the scenes were created (3D CTA sizes)
   int has_material;             // some scene has per-particle material (gmat): material gradients
   int sm_count;                 // SMs of the device
   TileLaunch launch[TK_COUNT];  // launch shape of each tile kernel

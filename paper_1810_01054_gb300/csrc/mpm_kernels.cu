@@ -611,8 +611,8 @@ __device__ __forceinline__ void release_work(const BatchDev& b, int w) {
 //          over the tile's cells, insertion sort inside each cell) -- fixes every later sum order.
 // Phase B  one record per particle (fraction f, momentum part a, MLS matrix M = dx G, mass; plus
 //          the adjoint-scatter record (C) in the reverse pass), all staged in shared memory.
-// Phase C  work item = (cell, part): 2D one stencil node, 3D one x-slab of 9 nodes; a thread
-//          accumulates its item over the cell's particles in registers (fixed particle order).
+// Phase C  work item = (cell, part): 2D one stencil node, 3D one x-slab of 9 nodes (wide CTAs: one
+//          row of 3 nodes); a thread accumulates its item over the cell's particles in registers (fixed particle order).
 // Phase D  node block = fixed-order sum of the cell stencils covering each node -> global.
 template <int D, int TB, bool ADJ, int T = 256>
 struct P2GCfg {
@@ -625,8 +625,9 @@ struct P2GCfg {
   // floats per accumulator entry in shared memory: 3D entries are whole float4s (4, or 8 in the
   // reverse pass), read and summed as float4 in phase D
   static constexpr int CHS = D == 3 ? (CH + 3) / 4 * 4 : CH;
-  static constexpr int PARTS = D == 2 ? 9 : 3;             // work items per cell
-  static constexpr int NK = D == 2 ? 1 : 9;                // stencil nodes per work item
+  static constexpr bool ROWS = D == 2 || T >= 576;         // an item is one (x, y) of the stencil, else one x
+  static constexpr int PARTS = ROWS ? 9 : 3;               // work items per cell
+  static constexpr int NK = D == 2 ? 1 : ROWS ? 3 : 9;     // stencil nodes per work item
   static constexpr int THREADS = T;
   static constexpr int ITEMS = Tile<D, TB>::CELLS * PARTS;  // 2D 144 (576 with 8 x 8 tiles), 3D 192
   static constexpr int IPT = (ITEMS + T - 1) / T;          // work items per thread
@@ -638,18 +639,20 @@ struct P2GCfg {
   static constexpr size_t U1 = REC_BYTES > ACC_BYTES ? REC_BYTES : ACC_BYTES;
   static constexpr size_t U_BYTES = U1 > IDS_BYTES ? U1 : IDS_BYTES;
   static constexpr size_t SMEM = IDS_BYTES + U_BYTES;
-  static_assert(D == 2 || IPT == 1, "a 3D work item holds 9 nodes: one item per thread");
+  static constexpr bool TWO = T < REC_CAP;                 // a thread may own two entries of a tile's list
+  static_assert(D == 2 || IPT == 1, "a 3D work item holds 3 or 9 nodes: one item per thread");
   static_assert(Tile<D, TB>::BLOCK_NODES <= THREADS, "one node per thread in phase D");
 };
 
-// T threads per CTA (256; 128 in 2D, where a thread then owns up to two of the 144 work items):
-// the work items and every sum keep their order, so T changes no bit of the results.
+// T threads per CTA (256; 128 in 2D, where a thread then owns up to two of the 144 work items; 576 in
+// 3D for scenes of at most a tile per SM, a record and a row of three nodes per thread: a lone tile's
+// chain is what such a launch takes): every sum keeps its order, so T changes no bit of the results.
 // Resident CTAs: the 3D forward P2G keeps 3 of 256 threads per SM (85 registers, a few spills in
 // its record phase; 4 % faster on the 1M-particle cluster than 2 at 126 registers); the adjoint
 // scatter holds 63 accumulators and keeps 2.
 // BINS: the tile lists are bins (BatchDev::bin_ctl), else the sort's.
 template <int D, int TB, bool ADJ, int T, bool BINS>
-__global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_p2g(BatchDev b) {
+__global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_p2g(BatchDev b) {
   pdl_enter();
   using K = P2GCfg<D, TB, ADJ, T>;
   constexpr int B = Tile<D, TB>::B, CELLS = Tile<D, TB>::CELLS, NB = Tile<D, TB>::BLOCK_NODES,
@@ -714,7 +717,7 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
       canon = b.sorted + size_t(gt) * K::CAP;
       // the thread's entries are requested with the count (in bounds whatever the count)
       e0 = raw[tid];
-      e1 = raw[tid + K::THREADS];
+      if constexpr (K::TWO) e1 = raw[tid + K::THREADS];
       cnt = int(b.bin_ctl[BIN_COUNT + size_t(par) * b.total_tiles + gt]);
       if (tid == 0) b.active[slot] = gt;  // for the controller reverse
     } else {
@@ -759,8 +762,8 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
       item_thread[j] = it < K::ITEMS;
       my_cell[j] = it / K::PARTS;
       my_part[j] = it - K::PARTS * my_cell[j];
-      ikx[j] = D == 2 ? my_part[j] / 3 : my_part[j];  // stencil x offset of the item
-      iky[j] = D == 2 ? my_part[j] % 3 : 0;           // 2D: stencil y offset of the item
+      ikx[j] = K::ROWS ? my_part[j] / 3 : my_part[j];  // stencil x offset of the item
+      iky[j] = K::ROWS ? my_part[j] % 3 : 0;           // stencil y offset of the item (slabs: every one)
 #pragma unroll
       for (int k = 0; k < K::NK; ++k)
 #pragma unroll
@@ -885,8 +888,9 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
             q2s = fmaf(Ma[6], kxf, aa[2]);
           }
 #pragma unroll
-          for (int ky = 0; ky < 3; ++ky) {
-            const float wxy = wx * w[1][ky];
+          for (int jy = 0; jy < K::NK / 3; ++jy) {
+            const int ky = K::ROWS ? iky[j] : jy;
+            const float wxy = wx * (ky == 0 ? w[1][0] : (ky == 1 ? w[1][1] : w[1][2]));
             const float kyf = float(ky);
             const float2 v01 = __ffma2_rn(make_float2(Mv[1], Mv[4]), make_float2(kyf, kyf), u01);
             const float v2 = fmaf(Mv[7], kyf, u2s);
@@ -901,7 +905,7 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
             for (int kz = 0; kz < 3; ++kz) {
               const float N = wxy * w[2][kz];
               const float kzf = float(kz);
-              const int k = ky * 3 + kz;
+              const int k = jy * 3 + kz;
               const float2 NN = make_float2(N, N);
               const float2 t01 = __ffma2_rn(make_float2(Mv[2], Mv[5]), make_float2(kzf, kzf), v01);
               const float t2 = fmaf(Mv[8], kzf, v2);
@@ -976,7 +980,7 @@ __global__ void __launch_bounds__(T, T == 256 ? (D == 3 && !ADJ ? 3 : 2) : 4) k_
       // bucketed; its canonical position is the cell start plus the number of smaller ids in its
       // cell (order: cell, then particle id), and its record is written straight there.
       const uint32_t r0 = tid < cnt ? (BINS ? e0 : raw[tid]) : 0xffffffffu;
-      const uint32_t r1 = tid + K::THREADS < cnt ? (BINS ? e1 : raw[tid + K::THREADS]) : 0xffffffffu;
+      const uint32_t r1 = K::TWO && tid + K::THREADS < cnt ? (BINS ? e1 : raw[tid + K::THREADS]) : 0xffffffffu;
       float pre[Cfg<D>::S];
       int g0 = -1, g1 = -1;
       if (r0 != 0xffffffffu) {
@@ -1417,7 +1421,7 @@ struct G2PCfg {
 };
 
 template <int D, int TB, int T, bool BINS>
-__global__ void __launch_bounds__(T, 768 / T) k_g2p(BatchDev b, const SelectPar* __restrict__ sel) {
+__global__ void __launch_bounds__(T, T > 256 ? 1 : 768 / T) k_g2p(BatchDev b, const SelectPar* __restrict__ sel) {
   pdl_enter();
   using K = G2PCfg<D>;
   constexpr int B = Tile<D, TB>::B, NB = Tile<D, TB>::BLOCK_NODES, BN = Tile<D, TB>::BN;
@@ -1913,18 +1917,20 @@ __device__ __forceinline__ float adj_core(Part<D>& q, Part<D>& g1, const float* 
   return contrib;
 }
 
-// CTA size of the adjoint gather: fixed per dimension (its group sums are formed per warp, then
-// per CTA, so the size sets their rounding; batches never mix dimensions).  128 threads measured
-// faster in 3D, 256 in 2D.
+// CTA size of the adjoint gather: 128 threads in 3D and 256 in 2D measured fastest with many tiles per
+// SM; 3D scenes of at most two tiles, or one, per SM take 256 or 512, as a lone tile's rounds are what
+// such a launch takes.  Its group sums are formed per 32 particles of the tile's list and added in
+// list order, so the CTA size changes no bit of them.
 template <int D>
 constexpr int kAdjThreads = D == 3 ? 128 : 256;
 
-template <int D, int TB, bool MAT, bool BINS>
-__global__ void __launch_bounds__(kAdjThreads<D>, 512 / kAdjThreads<D>) k_adj_gather(BatchDev b) {
+template <int D, int TB, bool MAT, bool BINS, int T>
+__global__ void __launch_bounds__(T, 512 / T) k_adj_gather(BatchDev b) {
   pdl_enter();
   constexpr int B = Tile<D, TB>::B, NB = Tile<D, TB>::BLOCK_NODES, BN = Tile<D, TB>::BN;
   __shared__ float4 sv[NB], sb[NB];
-  __shared__ float wpart[8][MAX_GROUPS];
+  constexpr int FOLD = 512, CHUNKS = FOLD / 32;  // particles whose group sums are kept at once
+  __shared__ float wpart[CHUNKS][MAX_GROUPS], gsum[MAX_GROUPS];  // gsum: (K) over the tile's particles so far
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ SceneShared sh;
   __shared__ BinView bv;
@@ -1986,8 +1992,7 @@ __global__ void __launch_bounds__(kAdjThreads<D>, 512 / kAdjThreads<D>) k_adj_ga
     build_node_block<D, TB, true>(b, sp, BINS ? &bv : nullptr, t, sv, sb);
     cp_async_wait_all();  // the actuations (readable by all after the barrier)
     __syncthreads();
-    float lo = 0.0f, hi = 0.0f;  // per-warp group sums of (K), lane-owned
-    for (int e0 = 0; e0 < cnt; e0 += blockDim.x) {
+    for (int e0 = 0; e0 < cnt; e0 += T) {
       const int e = e0 + tid;
       int g = -1;
       float contrib = 0.0f;
@@ -2063,15 +2068,27 @@ __global__ void __launch_bounds__(kAdjThreads<D>, 512 / kAdjThreads<D>) k_adj_ga
           set_status(sp.status, ST_BINNING);
         }
       }
+      float lo = 0.0f, hi = 0.0f;  // group sums of the warp's 32 particles, lane-owned
       warp_group_add(g, contrib, lo, hi);
+      const int chunk = (e0 / 32 + warp) % CHUNKS;
+      wpart[chunk][lane] = lo;
+      wpart[chunk][lane + 32] = hi;
+      if ((e0 + T) % FOLD == 0 && e0 + T < cnt) {  // more to come (uniform across the CTA): fold these
+        __syncthreads();
+        if (tid < MAX_GROUPS) {
+          float t = e0 + T == FOLD ? 0.0f : gsum[tid];
+          for (int c = 0; c < CHUNKS; ++c) t += wpart[c][tid];
+          gsum[tid] = t;
+        }
+        __syncthreads();
+      }
     }
-    wpart[warp][lane] = lo;
-    wpart[warp][lane + 32] = hi;
     __syncthreads();
     if (tid < MAX_GROUPS) {
-      float s = 0.0f;
-      for (int w = 0; w < int(blockDim.x >> 5); ++w) s += wpart[w][tid];
-      b.gpartial[size_t(slot) * MAX_GROUPS + tid] = s;
+      const int last = cnt > FOLD ? (cnt - 1) / FOLD * FOLD : 0;  // first particle of the open fold
+      float t = last > 0 ? gsum[tid] : 0.0f;
+      for (int c = 0; c < (cnt - last + 31) / 32; ++c) t += wpart[c][tid];
+      b.gpartial[size_t(slot) * MAX_GROUPS + tid] = t;
     }
     __syncthreads();
   }
@@ -2133,6 +2150,11 @@ cudaError_t launch_sort(const BatchDev& b, cudaStream_t s, const SelectPar* sel)
 
 template <int D, int TB, bool ADJ, bool BINS>
 static cudaError_t p2g_configure_lists() {
+  if constexpr (D == 3) {
+    const cudaError_t w = cudaFuncSetAttribute(k_p2g<D, TB, ADJ, 576, BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               int(P2GCfg<D, TB, ADJ, 576>::SMEM));
+    if (w != cudaSuccess) return w;
+  }
   cudaError_t e = cudaFuncSetAttribute(k_p2g<D, TB, ADJ, 256, BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        int(P2GCfg<D, TB, ADJ, 256>::SMEM));
   if constexpr (D == 2) {
@@ -2165,8 +2187,23 @@ static int tile_grid(const BatchDev& b, int k) {
   return grid < 1 ? 1 : grid;
 }
 
+// 3D scenes of few tiles (counted at creation; every CTA size gives the same bits): at most `per_sm`
+// tiles per SM, where one resident wide CTA per SM holds them all.  A 7,919-particle body, closed-loop
+// controller, 24 steps with the reverse pass: 2456 us with the large scenes' CTAs, 2261 with these.
+template <int D>
+static bool few_tiles(const BatchDev& b, int per_sm) {
+  return D == 3 && b.occupied > 0 && b.occupied <= per_sm * b.sm_count;
+}
+
 template <int D, int TB, bool ADJ, bool BINS>
 static cudaError_t p2g_lists(const BatchDev& b, cudaStream_t s) {
+  if constexpr (D == 3)
+    if (few_tiles<D>(b, 1)) {
+      launch_pdl(k_p2g<D, TB, ADJ, 576, BINS>, dim3(std::min(b.total_tiles, b.sm_count)), dim3(576),
+                 P2GCfg<D, TB, ADJ, 576>::SMEM, s, b);
+      count_launches(1);
+      return cudaGetLastError();
+    }
   const int k = ADJ ? TK_P2G_ADJ : TK_P2G;
   const int grid = tile_grid(b, k);
   bool small = false;  // 128-thread CTAs (2D only)
@@ -2193,6 +2230,13 @@ cudaError_t launch_p2g(const BatchDev& b, bool with_adjoint, cudaStream_t s) {
 
 template <int D, int TB, bool BINS>
 static cudaError_t g2p_lists(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
+  if constexpr (D == 3)
+    if (few_tiles<D>(b, 1)) {
+      launch_pdl(k_g2p<D, TB, 512, BINS>, dim3(std::min(b.total_tiles, b.sm_count) + (sel ? 1 : 0)), dim3(512), 0, s, b,
+                 sel);
+      count_launches(1);
+      return cudaGetLastError();
+    }
   const int grid = tile_grid(b, TK_G2P) + (sel ? 1 : 0);
   if (b.launch[TK_G2P].threads == 128)
     launch_pdl(k_g2p<D, TB, 128, BINS>, dim3(grid), dim3(128), 0, s, b, sel);
@@ -2213,15 +2257,24 @@ cudaError_t launch_g2p(const BatchDev& b, cudaStream_t s, const SelectPar* sel) 
   return g2p_impl<D, 4>(b, s, sel);
 }
 
-template <int D, int TB, bool BINS>
-static cudaError_t adj_gather_lists(const BatchDev& b, cudaStream_t s) {
-  const int grid = tile_grid(b, TK_ADJ_GATHER);
+template <int D, int TB, bool BINS, int T>
+static cudaError_t adj_gather_threads(const BatchDev& b, int grid, cudaStream_t s) {
   if (b.has_material)
-    launch_pdl(k_adj_gather<D, TB, true, BINS>, dim3(grid), dim3(kAdjThreads<D>), 0, s, b);
+    launch_pdl(k_adj_gather<D, TB, true, BINS, T>, dim3(grid), dim3(T), 0, s, b);
   else
-    launch_pdl(k_adj_gather<D, TB, false, BINS>, dim3(grid), dim3(kAdjThreads<D>), 0, s, b);
+    launch_pdl(k_adj_gather<D, TB, false, BINS, T>, dim3(grid), dim3(T), 0, s, b);
   count_launches(1);
   return cudaGetLastError();
+}
+template <int D, int TB, bool BINS>
+static cudaError_t adj_gather_lists(const BatchDev& b, cudaStream_t s) {
+  if constexpr (D == 3) {
+    if (few_tiles<D>(b, 1))
+      return adj_gather_threads<D, TB, BINS, 512>(b, std::min(b.total_tiles, b.sm_count), s);
+    if (few_tiles<D>(b, 2))
+      return adj_gather_threads<D, TB, BINS, 256>(b, std::min(b.total_tiles, 2 * b.sm_count), s);
+  }
+  return adj_gather_threads<D, TB, BINS, kAdjThreads<D>>(b, tile_grid(b, TK_ADJ_GATHER), s);
 }
 template <int D, int TB>
 static cudaError_t adj_gather_impl(const BatchDev& b, cudaStream_t s) {

@@ -87,3 +87,35 @@ def test_steps_after_a_forward_only_batch_request(M, ctx, dim):
         assert np.array_equal(a, b)
     batch.close()
     sc.close()
+
+
+@pytest.mark.parametrize("N", [1500, 12000, 30000])  # a few, under and over 512 particles a tile
+def test_cta_sizes_of_3d_scenes_give_the_same_bits(M, ctx, N):
+    """A 3D scene of at most a tile per SM runs wide CTAs, a batch of two to three such scenes (at most
+    two tiles per SM) a wider adjoint gather, a larger one the CTAs of large scenes: the results are the
+    same bits."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    spec = S.blob(3, 48, N, 62, radius_cells=8.0, v_scale=0.3, c_scale=0.5, f_scale=0.03, n_groups=7, amp=2.0,
+                  bc_width=3, dt=5e-4)
+    t = np.floor(np.asarray(spec.x0) / spec.dx - 0.5).astype(int) // 4
+    tiles = len(np.unique((t[:, 0] * 12 + t[:, 1]) * 12 + t[:, 2]))
+    counts = (1, sms // tiles + 1, 2 * sms // tiles + 1)
+    assert tiles <= sms < counts[1] * tiles <= 2 * sms < counts[2] * tiles
+    T = 6
+    want = None
+    for B in counts:
+        scenes = [M.Scene(ctx, spec) for _ in range(B)]
+        batch = M.Batch(ctx, 3)
+        slots = [batch.admit(sc, T, True) for sc in scenes]
+        while not all(batch.poll(sl) for sl in slots):
+            batch.tick(4)
+        for sc in scenes:
+            got = sc.get_state() + sc.gradients()
+            want = want or got
+            for a, b in zip(got, want):
+                assert np.array_equal(a, b)
+        batch.close()
+        for sc in scenes:
+            sc.close()
+    assert np.abs(want[-1]).max() > 0
