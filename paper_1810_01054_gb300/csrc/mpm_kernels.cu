@@ -633,11 +633,20 @@ struct P2GCfg {
   static constexpr int IPT = (ITEMS + T - 1) / T;          // work items per thread
   static constexpr int REC_CAP = D == 2 ? 1024 : 512;      // records staged at once
   static constexpr int CAP = Tile<D, TB>::SORT_CAP;
-  static constexpr size_t REC_BYTES = size_t(REC_CAP) * RW * 4;
+  // 3D records are planes of float4 (4, or 7 in the reverse pass), read as such and already in the pairs
+  // the packed FMA takes.  A record sits at its row plus its cell: at eight particles a cell the rows a
+  // warp's items read are eight apart, which without the shift is the same 16 bytes of every 128 (an
+  // odd stride of words had the like: 38 % of P2G's shared wavefronts were bank conflicts).  The lists'
+  // room is what the fast path needs; the general path sorts in the records' place.  1M-particle
+  // cluster: adjoint scatter 105.6 -> 101.2 us, P2G 62.0 -> 60.6-62.0.
+  static constexpr int RP = REC_CAP + Tile<D, TB>::CELLS;  // records per plane
+  static constexpr size_t REC_BYTES = D == 3 ? size_t(RP) * (ADJ ? 7 : 4) * 16 : size_t(REC_CAP) * RW * 4;
   static constexpr size_t ACC_BYTES = size_t(Tile<D, TB>::CELLS) * Cfg<D>::STENCIL * CHS * 4;
-  static constexpr size_t IDS_BYTES = size_t(CAP) * 4;
+  static constexpr int FAST = 2 * T < REC_CAP ? 2 * T : REC_CAP;  // most particles of the fast path
+  static constexpr size_t IDS_BYTES = size_t(FAST) * 4;
+  static constexpr size_t SORT_BYTES = 2 * size_t(CAP) * 4;       // the general path's lists, before its records
   static constexpr size_t U1 = REC_BYTES > ACC_BYTES ? REC_BYTES : ACC_BYTES;
-  static constexpr size_t U_BYTES = U1 > IDS_BYTES ? U1 : IDS_BYTES;
+  static constexpr size_t U_BYTES = U1 > SORT_BYTES ? U1 : SORT_BYTES;
   static constexpr size_t SMEM = IDS_BYTES + U_BYTES;
   static constexpr bool TWO = T < REC_CAP;                 // a thread may own two entries of a tile's list
   static_assert(D == 2 || IPT == 1, "a 3D work item holds 3 or 9 nodes: one item per thread");
@@ -799,7 +808,8 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
       const float J = particle_G<D>(q, sp, as, g, pm, P, A, G, sig);
       if (!(J > 0.0f)) set_status(sp.status, ST_INVERTED);
       const float keep = wm > 0.0f ? 1.0f : 0.0f;
-      float* rec = U + size_t(row) * K::RW;
+      float rec3[D == 3 ? K::RF + K::RA : 1];  // 3D: the record in the order below, stored as planes
+      float* rec = D == 3 ? rec3 : U + size_t(row) * K::RW;
       int o = 0;
 #pragma unroll
       for (int a = 0; a < D; ++a) rec[o++] = f[a];
@@ -816,6 +826,14 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
 #pragma unroll
         for (int c = 0; c < D; ++c) rec[o++] = keep * dx * G[a][c];
       rec[o++] = wm;
+      if constexpr (D == 3) {
+        float4* p = reinterpret_cast<float4*>(U) + (row + int(kc));
+        const float *av = rec3 + 3, *Mv = rec3 + 6;
+        p[0] = make_float4(rec3[0], rec3[1], rec3[2], wm);
+        p[K::RP] = make_float4(av[0], av[1], Mv[0], Mv[3]);
+        p[2 * K::RP] = make_float4(Mv[1], Mv[4], Mv[2], Mv[5]);
+        p[3 * K::RP] = make_float4(av[2], Mv[6], Mv[7], Mv[8]);
+      }
       if constexpr (ADJ) {
         // (A) vbar' = gv1 + dt gx1 ; (B) Cbar' = gC1 + dt gF1 F^T ; record of (C):
         // vbar' + (4/dx^2) Cbar' (x_i - x_p) = [vbar' - (4/dx) Cbar' f] + (4/dx) Cbar' k
@@ -847,22 +865,29 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
 #pragma unroll
           for (int c = 0; c < D; ++c) rec[o++] = keep * Dx4 * Cb[a][c];
       }
+      if constexpr (D == 3 && ADJ) {
+        float4* p = reinterpret_cast<float4*>(U) + (row + int(kc)) + 4 * K::RP;
+        const float *aa = rec3 + K::RF, *Ma = aa + 3;
+        p[0] = make_float4(aa[0], aa[1], Ma[0], Ma[3]);
+        p[K::RP] = make_float4(Ma[1], Ma[4], Ma[2], Ma[5]);
+        p[2 * K::RP] = make_float4(aa[2], Ma[6], Ma[7], Ma[8]);
+      }
     };
 
     // Phase C over staged rows [lo, hi) (row = canonical position - c0): this thread's work item j
     // accumulates its stencil nodes over the cell's particles in canonical order.
     auto accumulate = [&](int j, int lo, int hi, int c0) {
       for (int ei = lo; ei < hi; ++ei) {
-        const float* rec = U + size_t(ei - c0) * K::RW;
-        const float mass = rec[K::RF - 1];
-        float w[D][3], dwd[3];
-#pragma unroll
-        for (int a = 0; a < D; ++a) bspline(rec[a], 1.0f, w[a], dwd);
-        const float* av = rec + D;      // a
-        const float* Mv = rec + 2 * D;  // M, row-major
-        // the item's own offsets select weights by value: a runtime index would put w in local memory
-        const float wx = ikx[j] == 0 ? w[0][0] : (ikx[j] == 1 ? w[0][1] : w[0][2]);
         if constexpr (D == 2) {
+          const float* rec = U + size_t(ei - c0) * K::RW;
+          const float mass = rec[K::RF - 1];
+          float w[D][3], dwd[3];
+#pragma unroll
+          for (int a = 0; a < D; ++a) bspline(rec[a], 1.0f, w[a], dwd);
+          const float* av = rec + D;      // a
+          const float* Mv = rec + 2 * D;  // M, row-major
+          // the item's own offsets select weights by value: a runtime index would put w in local memory
+          const float wx = ikx[j] == 0 ? w[0][0] : (ikx[j] == 1 ? w[0][1] : w[0][2]);
           const float N = wx * (iky[j] == 0 ? w[1][0] : (iky[j] == 1 ? w[1][1] : w[1][2]));
 #pragma unroll
           for (int a = 0; a < D; ++a) acc[j][0][a] += N * (av[a] + Mv[a * D] * float(ikx[j]) + Mv[a * D + 1] * float(iky[j]));
@@ -875,31 +900,39 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
               acc[j][0][K::CHF + a] += N * (aa[a] + Ma[a * D] * float(ikx[j]) + Ma[a * D + 1] * float(iky[j]));
           }
         } else {
-          // u = a + M[:,0] kx, then per row + M[:,1] ky and per node + M[:,2] kz (M row-major)
+          const float4* p = reinterpret_cast<const float4*>(U) + (ei - c0 + my_cell[j]);
+          const float4 p0 = p[0], p1 = p[K::RP], p2 = p[2 * K::RP], p3 = p[3 * K::RP];
+          const float rf[3] = {p0.x, p0.y, p0.z}, mass = p0.w;
+          float w[3][3], dwd[3];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) bspline(rf[a], 1.0f, w[a], dwd);
+          const float wx = ikx[j] == 0 ? w[0][0] : (ikx[j] == 1 ? w[0][1] : w[0][2]);
+          // u = a + M[:,0] kx, then per row + M[:,1] ky and per node + M[:,2] kz
           const float kxf = float(ikx[j]);
-          const float2 u01 = __ffma2_rn(make_float2(Mv[0], Mv[3]), make_float2(kxf, kxf), make_float2(av[0], av[1]));
-          const float u2s = fmaf(Mv[6], kxf, av[2]);
+          const float2 u01 = __ffma2_rn(make_float2(p1.z, p1.w), make_float2(kxf, kxf), make_float2(p1.x, p1.y));
+          const float u2s = fmaf(p3.y, kxf, p3.x);
+          float4 p4, p5, p6;
           float2 q01 = make_float2(0.0f, 0.0f);
           float q2s = 0.0f;
           if constexpr (ADJ) {
-            const float* aa = rec + K::RF;
-            const float* Ma = aa + D;
-            q01 = __ffma2_rn(make_float2(Ma[0], Ma[3]), make_float2(kxf, kxf), make_float2(aa[0], aa[1]));
-            q2s = fmaf(Ma[6], kxf, aa[2]);
+            p4 = p[4 * K::RP];
+            p5 = p[5 * K::RP];
+            p6 = p[6 * K::RP];
+            q01 = __ffma2_rn(make_float2(p4.z, p4.w), make_float2(kxf, kxf), make_float2(p4.x, p4.y));
+            q2s = fmaf(p6.y, kxf, p6.x);
           }
 #pragma unroll
           for (int jy = 0; jy < K::NK / 3; ++jy) {
             const int ky = K::ROWS ? iky[j] : jy;
             const float wxy = wx * (ky == 0 ? w[1][0] : (ky == 1 ? w[1][1] : w[1][2]));
             const float kyf = float(ky);
-            const float2 v01 = __ffma2_rn(make_float2(Mv[1], Mv[4]), make_float2(kyf, kyf), u01);
-            const float v2 = fmaf(Mv[7], kyf, u2s);
+            const float2 v01 = __ffma2_rn(make_float2(p2.x, p2.y), make_float2(kyf, kyf), u01);
+            const float v2 = fmaf(p3.z, kyf, u2s);
             float2 r01 = make_float2(0.0f, 0.0f);
             float r2 = 0.0f;
             if constexpr (ADJ) {
-              const float* Ma = rec + K::RF + D;
-              r01 = __ffma2_rn(make_float2(Ma[1], Ma[4]), make_float2(kyf, kyf), q01);
-              r2 = fmaf(Ma[7], kyf, q2s);
+              r01 = __ffma2_rn(make_float2(p5.x, p5.y), make_float2(kyf, kyf), q01);
+              r2 = fmaf(p6.z, kyf, q2s);
             }
 #pragma unroll
             for (int kz = 0; kz < 3; ++kz) {
@@ -907,14 +940,13 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
               const float kzf = float(kz);
               const int k = jy * 3 + kz;
               const float2 NN = make_float2(N, N);
-              const float2 t01 = __ffma2_rn(make_float2(Mv[2], Mv[5]), make_float2(kzf, kzf), v01);
-              const float t2 = fmaf(Mv[8], kzf, v2);
+              const float2 t01 = __ffma2_rn(make_float2(p2.z, p2.w), make_float2(kzf, kzf), v01);
+              const float t2 = fmaf(p3.w, kzf, v2);
               aP01[k] = __ffma2_rn(NN, t01, aP01[k]);
               aP2m[k] = __ffma2_rn(NN, make_float2(t2, mass), aP2m[k]);
               if constexpr (ADJ) {
-                const float* Ma = rec + K::RF + D;
-                const float2 s01 = __ffma2_rn(make_float2(Ma[2], Ma[5]), make_float2(kzf, kzf), r01);
-                const float s2 = fmaf(Ma[8], kzf, r2);
+                const float2 s01 = __ffma2_rn(make_float2(p5.z, p5.w), make_float2(kzf, kzf), r01);
+                const float s2 = fmaf(p6.w, kzf, r2);
                 aQ01[k] = __ffma2_rn(NN, s01, aQ01[k]);
                 aQ2[k] = fmaf(N, s2, aQ2[k]);
               }
@@ -974,7 +1006,7 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
       }
     };
 
-    if (cnt <= 2 * K::THREADS && cnt <= K::REC_CAP) {
+    if (cnt <= K::FAST) {
       // ---- fast path: every thread owns raw entries tid and tid + THREADS of the tile list.
       // Its first particle's state is requested at once and arrives while the tile is being
       // bucketed; its canonical position is the cell start plus the number of smaller ids in its
@@ -1027,6 +1059,7 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
     } else {
       // ---- general path: bucket, insertion-sort each cell's ids, stage records in chunks
       uint32_t* ent = reinterpret_cast<uint32_t*>(U);
+      uint32_t* gids = ent + K::CAP;
       if (tid < CELLS) cfill[tid] = 0;
       cp_async_wait_all();  // the actuations
       __syncthreads();
@@ -1043,23 +1076,23 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
       for (int i = tid; i < cnt; i += blockDim.x) {
         const uint32_t r = ent[i];
         const uint32_t c = r >> 26;
-        ids[cstart[c] + atomicAdd(&cfill[c], 1)] = r & 0x3ffffffu;
+        gids[cstart[c] + atomicAdd(&cfill[c], 1)] = r & 0x3ffffffu;
       }
       __syncthreads();
       if (tid < CELLS) {  // insertion sort of each cell's ids
         const int s0 = cstart[tid], s1 = cstart[tid + 1];
         for (int i = s0 + 1; i < s1; ++i) {
-          const uint32_t v = ids[i];
+          const uint32_t v = gids[i];
           int j = i - 1;
-          while (j >= s0 && ids[j] > v) {
-            ids[j + 1] = ids[j];
+          while (j >= s0 && gids[j] > v) {
+            gids[j + 1] = gids[j];
             --j;
           }
-          ids[j + 1] = v;
+          gids[j + 1] = v;
         }
       }
       __syncthreads();
-      for (int i = tid; i < cnt; i += blockDim.x) canon[i] = ids[i];
+      for (int i = tid; i < cnt; i += blockDim.x) canon[i] = gids[i];
       int cs[K::IPT], ce[K::IPT];
 #pragma unroll
       for (int j = 0; j < K::IPT; ++j) {
@@ -1070,7 +1103,7 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
         __syncthreads();  // previous records consumed (and phase A's scratch released)
         const int c1 = cnt < c0 + K::REC_CAP ? cnt : c0 + K::REC_CAP;
         for (int e = c0 + tid; e < c1; e += K::THREADS) {
-          const int id = int(ids[e]);
+          const int id = int(canon[e]);
           float r[Cfg<D>::S];
           load_planes<D, Cfg<D>::PLANES>(sp.planes, sp.npad, id, r);
           make_record(id, sp.key[id] & 63u, group_of(sp, id), r, e - c0);
