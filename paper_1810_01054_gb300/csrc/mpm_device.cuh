@@ -268,67 +268,79 @@ struct MaterialT {
 };
 using Material = MaterialT<float>;
 
-// P = mu (F - F^{-T}) + lambda ln J F^{-T} + F sigma_a, sigma_a = a Diag(dir).
-// Returns J (caller checks J > 0 before trusting P).
+// G = -(4/dx^2) dt V0 P F^T + m C (Eq. 4) with kG = -(4/dx^2) dt V0 and the neo-Hookean and actuation
+// stress P = mu (F - F^{-T}) + lambda ln J F^{-T} + F sigma_a, sigma_a = Diag(sig).  Formed as the
+// Kirchhoff stress P F^T = F Diag(mu + sig) F^T + (lambda ln J - mu) I: symmetric, without F^{-T} and P
+// themselves (3D: about 30 operations instead of 110, and no division; with stress_adjoint, on the
+// 1M-particle cluster: P2G 60.6 -> 56.7 us, adjoint scatter 101.2 -> 98.0, adjoint gather 111.9 ->
+// 105.8; errors against FP64 as before).  Returns J (caller checks J > 0 before trusting G).
 template <int D, class R>
-__device__ __forceinline__ R stress(const R (&F)[D][D], MaterialT<R> m, const R* sig_diag, R (&P)[D][D],
-                                    R (&A)[D][D]) {
-  R J = det<D>(F);
-  R Js = J > R(0) ? J : R(1);
-  inv_transpose<D>(F, Js, A);
-  R lJ = s_log(Js);
+__device__ __forceinline__ R kirchhoff_G(const R (&F)[D][D], const R (&C)[D][D], MaterialT<R> m, const R* sig, R kG,
+                                         R mass, R (&G)[D][D]) {
+  const R J = det<D>(F);
+  const R iso = m.la * s_log(J > R(0) ? J : R(1)) - m.mu;
 #pragma unroll
-  for (int i = 0; i < D; ++i)
+  for (int i = 0; i < D; ++i) {
+    R Fs[D];
 #pragma unroll
-    for (int j = 0; j < D; ++j) P[i][j] = m.mu * (F[i][j] - A[i][j]) + m.la * lJ * A[i][j] + F[i][j] * sig_diag[j];
+    for (int k = 0; k < D; ++k) Fs[k] = F[i][k] * (m.mu + sig[k]);
+#pragma unroll
+    for (int j = i; j < D; ++j) {
+      R t = i == j ? iso : R(0);
+#pragma unroll
+      for (int k = 0; k < D; ++k) t += Fs[k] * F[j][k];
+      G[i][j] = kG * t + mass * C[i][j];
+      if (j > i) G[j][i] = kG * t + mass * C[j][i];
+    }
+  }
   return J;
 }
 
-// G = -(4/dx^2) dt V0 P F^T + m C  (Eq. 4)
+// Adjoint of the stress part of G for Gbar = dL/dG (S4 (G), (H), (K) together): with S = Gbar + Gbar^T,
+//   dL/dF += kG (S F Diag(mu + sig) + lambda tr(Gbar) F^{-T}),  dL/dsig_c = kG/2 (F^T S F)_cc,
+//   dL/dmu = kG (1/2 F : S F - tr(Gbar)),  dL/dlambda = kG tr(Gbar) ln J.
+// The supplement's Hessian product of Pbar = kG Gbar F, Pbar sigma_a and kG Gbar^T P summed: their terms
+// in F^{-T} cancel up to the one of lambda, and neither ln J nor P is left.
 template <int D, class R>
-__device__ __forceinline__ void mls_G(const R (&P)[D][D], const R (&F)[D][D], const R (&C)[D][D], R kG, R mass,
-                                      R (&G)[D][D]) {
-#pragma unroll
-  for (int i = 0; i < D; ++i)
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      R s = R(0);
-#pragma unroll
-      for (int k = 0; k < D; ++k) s += P[i][k] * F[j][k];
-      G[i][j] = kG * s + mass * C[i][j];
-    }
-}
-
-// mu Pbar + (mu - lambda ln J) F^{-T} Pbar^T F^{-T} + lambda (F^{-T}:Pbar) F^{-T}
+struct StressAdj {
+  R F[D][D];   // dL/dF
+  R sig[D];    // dL/dsig
+  R mu, tr;    // dL/dmu; kG tr(Gbar)
+};
 template <int D, class R>
-__device__ __forceinline__ void nh_hessian_apply(const R (&A)[D][D], R J, MaterialT<R> m, const R (&Pb)[D][D],
-                                                 R (&H)[D][D]) {
-  R lJ = s_log(J > R(0) ? J : R(1));
-  R AP = R(0);
+__device__ __forceinline__ R stress_adjoint(const R (&F)[D][D], const R (&Gb)[D][D], MaterialT<R> m, const R* sig,
+                                            R kG, StressAdj<D, R>& o) {
+  R SF[D][D], tr = R(0), fsf = R(0);
 #pragma unroll
-  for (int i = 0; i < D; ++i)
+  for (int a = 0; a < D; ++a) tr += Gb[a][a];
 #pragma unroll
-    for (int j = 0; j < D; ++j) AP += A[i][j] * Pb[i][j];
-  R T[D][D];  // A Pb^T
+  for (int a = 0; a < D; ++a)
 #pragma unroll
-  for (int i = 0; i < D; ++i)
+    for (int c = 0; c < D; ++c) {
+      R t = R(0);
 #pragma unroll
-    for (int j = 0; j < D; ++j) {
-      R s = R(0);
-#pragma unroll
-      for (int k = 0; k < D; ++k) s += A[i][k] * Pb[j][k];
-      T[i][j] = s;
+      for (int k = 0; k < D; ++k) t += (Gb[a][k] + Gb[k][a]) * F[k][c];
+      SF[a][c] = t;
     }
-  R c = m.mu - m.la * lJ;
+  o.tr = kG * tr;
+  const R J = det<D>(F);
+  R A[D][D];
+  inv_transpose<D>(F, J > R(0) ? J : R(1), A);
+  const R lt = m.la * o.tr;
 #pragma unroll
-  for (int i = 0; i < D; ++i)
+  for (int c = 0; c < D; ++c) {
+    const R e = kG * (m.mu + sig[c]);
+    R t = R(0);
 #pragma unroll
-    for (int j = 0; j < D; ++j) {
-      R s = R(0);
-#pragma unroll
-      for (int k = 0; k < D; ++k) s += T[i][k] * A[k][j];
-      H[i][j] = m.mu * Pb[i][j] + c * s + m.la * AP * A[i][j];
+    for (int a = 0; a < D; ++a) {
+      o.F[a][c] = e * SF[a][c] + lt * A[a][c];
+      t += F[a][c] * SF[a][c];
     }
+    o.sig[c] = R(0.5) * kG * t;
+    fsf += t;
+  }
+  o.mu = R(0.5) * kG * fsf - o.tr;
+  return J;
 }
 
 // --------------------------------------------------------------------------- boundary (S5)

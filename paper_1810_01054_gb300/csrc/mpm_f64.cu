@@ -111,15 +111,6 @@ __device__ __forceinline__ int actuation64(const Par64& p, int id, double* sig) 
   return g;
 }
 
-// Stress P (elastic + F sigma_a), F^{-T}, J and the MLS momentum matrix G of Eq. 4.
-template <int D>
-__device__ __forceinline__ double stress_G64(const Par64& p, const Part<D, double>& q, const double* sig,
-                                             double (&P)[D][D], double (&A)[D][D], double (&G)[D][D]) {
-  const double J = stress<D>(q.F, p.mat, sig, P, A);
-  mls_G<D>(P, q.F, q.C, p.kG, p.mass, G);
-  return J;
-}
-
 // The thread's particle.  With L = 3 three neighbouring lanes share a particle (ten particles a
 // warp, two lanes idle), each working one x-slab of its stencil: a small scene's launch is bound by
 // one thread's chain of FP64 operations, and the slabs are independent.
@@ -202,9 +193,9 @@ __global__ void __launch_bounds__(F64_THREADS) k64_p2g(Par64 p) {
     set_status(p.status, ST_DOMAIN);
     return;
   }
-  double sig[D], P[D][D], A[D][D], G[D][D];
+  double sig[D], G[D][D];
   actuation64<D>(p, id, sig);
-  const double J = stress_G64<D>(p, q, sig, P, A, G);
+  const double J = kirchhoff_G<D>(q.F, q.C, p.mat, sig, p.kG, p.mass, G);
   if (!(J > 0.0)) set_status(p.status, ST_INVERTED);
   double vb[D] = {}, Cb[D][D] = {};
   if constexpr (ADJ) {
@@ -392,9 +383,9 @@ __global__ void __launch_bounds__(F64_THREADS) k64_adjoint(Par64 p) {
   if (live) {
     Part<D, double> g1, g0;
     load64<D>(p.adj_in, p.N, id, g1);
-    double sig[D], P[D][D], A[D][D], G[D][D];
+    double sig[D], G[D][D];
     const int grp = actuation64<D>(p, id, sig);
-    const double J = stress_G64<D>(p, q, sig, P, A, G);
+    kirchhoff_G<D>(q.F, q.C, p.mat, sig, p.kG, p.mass, G);
     double vb[D], Cb[D][D], mv[D];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -446,7 +437,6 @@ __global__ void __launch_bounds__(F64_THREADS) k64_adjoint(Par64 p) {
         Gb[a][c] = ln.total(Gb[a][c], some);
       }
     }
-    double Pb[D][D];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       double t = 0.0;
@@ -458,36 +448,24 @@ __global__ void __launch_bounds__(F64_THREADS) k64_adjoint(Par64 p) {
       for (int c = 0; c < D; ++c) {
         Cn[a][c] *= p.Dinv;
         g0.C[a][c] = p.mass * Gb[a][c];  // (I)
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < D; ++k) s += Gb[a][k] * q.F[k][c];
-        Pb[a][c] = p.kG * s;             // (G)
       }
     }
-    double H[D][D];
-    nh_hessian_apply<D>(A, J, p.mat, Pb, H);
+    StressAdj<D, double> sa;
+    stress_adjoint<D>(q.F, Gb, p.mat, sig, p.kG, sa);  // (G), (H), (K)
 #pragma unroll
     for (int a = 0; a < D; ++a)
 #pragma unroll
       for (int c = 0; c < D; ++c) {
-        double s = g1.F[a][c], t = 0.0;
+        double s = g1.F[a][c];
 #pragma unroll
-        for (int k = 0; k < D; ++k) {
-          s += p.dt * Cn[k][a] * g1.F[k][c];
-          t += Gb[k][a] * P[k][c];
-        }
-        g0.F[a][c] = s + H[a][c] + Pb[a][c] * sig[c] + p.kG * t;  // (H)
+        for (int k = 0; k < D; ++k) s += p.dt * Cn[k][a] * g1.F[k][c];
+        g0.F[a][c] = s + sa.F[a][c];     // (H)
       }
     store64<D>(p.adj_out, p.N, id, g0, ln.sub, L);
     if (want_act && grp >= 0 && ln.sub == 0) {  // (K)
       double contrib = 0.0;
 #pragma unroll
-      for (int a = 0; a < D; ++a) {
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < D; ++k) s += q.F[k][a] * Pb[k][a];
-        contrib += p.act_dir[grp * D + a] * s;
-      }
+      for (int a = 0; a < D; ++a) contrib += p.act_dir[grp * D + a] * sa.sig[a];
       atomicAdd(&gsum[grp], contrib);
     }
   }

@@ -174,17 +174,14 @@ __device__ __forceinline__ PMat pmat_of(const ScenePar& sp, int id) {
   return r;
 }
 
-// Per-particle quantities of P2G for a particle of group g and material pm: stress with
-// actuation and G of Eq. 4.  Returns J.
+// MLS matrix G of Eq. 4 for a particle of group g and material pm, stress with actuation included.
+// Returns J.
 template <int D>
 __device__ __forceinline__ float particle_G(const Part<D>& q, const ScenePar& sp, const ActSrc& as, int g,
-                                            const PMat& pm, float (&P)[D][D], float (&A)[D][D], float (&G)[D][D],
-                                            float* sig) {
+                                            const PMat& pm, float (&G)[D][D]) {
+  float sig[D];
   actuation<D>(as, g, sig);
-  float J = stress<D>(q.F, pm.mat, sig, P, A);
-  float kG = -4.0f * sp.inv_dx * sp.inv_dx * sp.dt * sp.vol;
-  mls_G<D>(P, q.F, q.C, kG, pm.mass, G);
-  return J;
+  return kirchhoff_G<D>(q.F, q.C, pm.mat, sig, -4.0f * sp.inv_dx * sp.inv_dx * sp.dt * sp.vol, pm.mass, G);
 }
 
 // ============================================================================ record selection
@@ -804,8 +801,8 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
           wm = 0.0f;
         }
       }
-      float P[D][D], A[D][D], G[D][D], sig[D];
-      const float J = particle_G<D>(q, sp, as, g, pm, P, A, G, sig);
+      float G[D][D];
+      const float J = particle_G<D>(q, sp, as, g, pm, G);
       if (!(J > 0.0f)) set_status(sp.status, ST_INVERTED);
       const float keep = wm > 0.0f ? 1.0f : 0.0f;
       float rec3[D == 3 ? K::RF + K::RA : 1];  // 3D: the record in the order below, stored as planes
@@ -1601,7 +1598,7 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : 768 / T) k_g2p(BatchDev b, co
 // ============================================================================ adjoint gather
 // Supplement S4: (F) vbar, (I) Cbar, (G) Pbar, (H) Fbar, (J) xbar, (K) sigma-bar -> dL/da.
 // `fetch(kx,ky,kz, v, pb)` returns (v*, m) in v and (pbar, mbar) in pb.  With MAT and per-particle
-// material (sp.gmat) this step's dL/dE_p = (F - F^{-T}):Pbar dmu/dE + ln J (F^{-T}:Pbar) dlambda/dE
+// material (sp.gmat) this step's dL/dE_p = dL/dmu dmu/dE + dL/dlambda dlambda/dE (stress_adjoint)
 // and dL/dm_p = sum_i N (mbar_i + pbar_i . (v_p + C_p (x_i - x_p))) are added into gmat[id].
 // A load the compiler keeps where it is written (not merged with an earlier load of the same
 // address), so that values needed only after a long loop need not stay in registers through it.
@@ -1622,11 +1619,8 @@ __device__ __forceinline__ float adj_core(Part<D>& q, Part<D>& g1, const float* 
   const float dt = sp.dt, dx = sp.dx, mass = pm.mass;
   const float Dinv = 4.0f * sp.inv_dx * sp.inv_dx;
   const float kG = -Dinv * dt * sp.vol;
-  float G[D][D], sig[D];
-  {
-    float P[D][D], A[D][D];  // recomputed after the stencil loop: not kept live across it
-    particle_G<D>(q, sp, as, g, pm, P, A, G, sig);
-  }
+  float G[D][D];
+  particle_G<D>(q, sp, as, g, pm, G);
   // s_i = vbar'.v* + Dinv v*^T Cbar' d + pbar.(m v + G d) + m mbar with d = (k - f) dx is affine in
   // the integer node offset k: alpha(k) = vbar' + Dinv Cbar' d and beta(k) = m v + G d are kept as
   // their value at the slab/row start plus one column per axis (Ac[c] = Dinv dx Cbar'[:, c],
@@ -1888,64 +1882,46 @@ __device__ __forceinline__ float adj_core(Part<D>& q, Part<D>& g1, const float* 
     g0.v[a] = mass * spb[a];  // (F)
   }
   const float sC = 4.0f * sp.inv_dx;
-  float Pb[D][D];
 #pragma unroll
   for (int a = 0; a < D; ++a)
 #pragma unroll
     for (int c = 0; c < D; ++c) {
       Cn[a][c] *= sC;
       g0.C[a][c] = mass * Gbar[a][c];  // (I)
-      float s = 0.0f;
-#pragma unroll
-      for (int k = 0; k < D; ++k) s += Gbar[a][k] * q.F[k][c];
-      Pb[a][c] = kG * s;  // (G)
     }
-  float P[D][D], A[D][D];
-  const float J = stress<D>(q.F, pm.mat, sig, P, A);
-  float H[D][D];
-  nh_hessian_apply<D>(A, J, pm.mat, Pb, H);
+  float sig[D];
+  actuation<D>(as, g, sig);
+  StressAdj<D, float> sa;
+  const float J = stress_adjoint<D>(q.F, Gbar, pm.mat, sig, kG, sa);  // (G), (H), (K)
   if (MAT && sp.gmat) {  // material gradients of this step (P2G is where E_p and m_p enter)
-    float gmu = 0.0f, gla = 0.0f, gm = smb;
+    float gm = smb;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       gm += q.v[a] * spb[a];
 #pragma unroll
-      for (int c = 0; c < D; ++c) {
-        gmu += (q.F[a][c] - A[a][c]) * Pb[a][c];
-        gla += A[a][c] * Pb[a][c];
-        gm += q.C[a][c] * Gbar[a][c];
-      }
+      for (int c = 0; c < D; ++c) gm += q.C[a][c] * Gbar[a][c];
     }
-    const float gE = gmu * sp.mu_per_E + logf(J > 0.0f ? J : 1.0f) * gla * sp.la_per_E;
+    const float gE = sa.mu * sp.mu_per_E + logf(J > 0.0f ? J : 1.0f) * sa.tr * sp.la_per_E;
     float2 acc = sp.gmat[id];
     acc.x += gE;
     acc.y += gm;
     sp.gmat[id] = acc;
   }
-  // (H) Fbar = (I + dt C^{n+1})^T Fbar' + H[Pbar] + Pbar sigma^T + kG Gbar^T P
+  // (H) Fbar = (I + dt C^{n+1})^T Fbar' and the stress part
 #pragma unroll
   for (int a = 0; a < D; ++a)
 #pragma unroll
     for (int c = 0; c < D; ++c) {
       float s = g1.F[a][c];
-      float t = 0.0f;
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        s += dt * Cn[k][a] * g1.F[k][c];
-        t += Gbar[k][a] * P[k][c];
-      }
-      g0.F[a][c] = s + H[a][c] + Pb[a][c] * sig[c] + kG * t;
+      for (int k = 0; k < D; ++k) s += dt * Cn[k][a] * g1.F[k][c];
+      g0.F[a][c] = s + sa.F[a][c];
     }
-  // (K) sigma-bar = F^T Pbar, contracted with the group's direction
+  // (K) sigma-bar contracted with the group's direction
   float contrib = 0.0f;
   if (g >= 0) {
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-      float s = 0.0f;
-#pragma unroll
-      for (int k = 0; k < D; ++k) s += q.F[k][a] * Pb[k][a];
-      contrib += as.dir[g * D + a] * s;
-    }
+    for (int a = 0; a < D; ++a) contrib += as.dir[g * D + a] * sa.sig[a];
   }
   return contrib;
 }
@@ -2349,9 +2325,9 @@ __global__ void k_plain_scatter(const ScenePar* __restrict__ dsp) {
     set_status(sp.status, ST_DOMAIN);
     return;
   }
-  float P[D][D], A[D][D], G[D][D], sig[D];
+  float G[D][D];
   const PMat pm = pmat_of(sp, id);
-  const float J = particle_G<D>(q, sp, ActSrc{sp.act, sp.act_dir}, group_of(sp, id), pm, P, A, G, sig);
+  const float J = particle_G<D>(q, sp, ActSrc{sp.act, sp.act_dir}, group_of(sp, id), pm, G);
   if (!(J > 0.0f)) set_status(sp.status, ST_INVERTED);
   float vb[D], Cb[D][D];
   if constexpr (ADJ) {

@@ -130,10 +130,9 @@ __global__ void __launch_bounds__(kNAThreads) k_na_p2g(NAPar p, float4* __restri
   const int g = p.group ? p.group[i] : -1;
 #pragma unroll
   for (int a = 0; a < D; ++a) sig[a] = (g >= 0 && g < p.G) ? p.act[g] * p.act_dir[g * D + a] : 0.f;
-  float P[D][D], A[D][D], G[D][D];
-  const float J = stress<D>(F, p.mat, sig, P, A);
+  float G[D][D];
+  const float J = kirchhoff_G<D>(F, C, p.mat, sig, -4.f * p.inv_dx * p.inv_dx * p.dt * p.vol, p.mass, G);
   if (!(J > 0.f)) set_status(p.status, ST_INVERTED);
-  mls_G<D>(P, F, C, -4.f * p.inv_dx * p.inv_dx * p.dt * p.vol, p.mass, G);
 #pragma unroll
   for (int kx = 0; kx < 3; ++kx)
 #pragma unroll
