@@ -510,9 +510,12 @@ mpm_status enqueue_reverse(mpm_scene* s, cudaStream_t st) {
   return enqueue_adjoint(s, s->b, st);
 }
 
-// True when the reverse graphs load the sorts on a branch (stored sorts, open-loop controller,
-// buffer set B allocated).
-bool load_branch(const mpm_scene* s) { return s->rcm_ws2 && s->ctrl_branch && s->d_gstep; }
+// True when the reverse graphs bin the states (or load their sorts) on a branch: open-loop controller,
+// buffer set B allocated, and every state of the run at hand with its sort: the sorts the recompute
+// kept, or with bins (which need only the state) also every state of the rollout.
+bool load_branch(const mpm_scene* s) {
+  return s->graphs_branch && s->ctrl_branch && s->d_gstep;
+}
 
 // `steps` reverse steps captured on ctx->capture with the sort loads on ctx->capture3: the first
 // step loads its sort in line (and keeps its step number n in d_gstep); the load of step j >= 1
@@ -752,28 +755,57 @@ mpm_status ensure_ws2_parts(mpm_scene* s) {
     CK(cudaEventCreateWithFlags(&s->ev_rcm[i], cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&s->ev_rev[i], cudaEventDisableTiming));
   }
-  if (s->ctrl_branch) {  // buffer set B of the reverse steps whose sorts load on a branch
-    BatchDev& bb = s->bB;  // only its sort arrays and record are used
-    bb = BatchDev{};
-    CKS(dalloc(&s->curB, 2, L));
-    CKS(dalloc(&s->keyB, s->npad, L));
-    CKS(dalloc(&s->actB, std::max(1, s->G), L));
-    CKS(dalloc(&s->d_gstep, 1, L));
-    CKS(dalloc(&bb.tile_start, nt + 1, L));
-    CKS(dalloc(&bb.tile_slot, nt, L));
-    CKS(dalloc(&bb.active, nt, L));
-    CKS(dalloc(&bb.n_active, 1, L));
-    if (bins)
-      CKS(alloc_bins(bb, s->dim, s->b.tile_edge, nt, L));
-    else
-      CKS(dalloc(&bb.sorted, s->npad, L));
-    bb.scenes = s->curB;
-    CK(cudaMemsetAsync(s->actB, 0, sizeof(float) * std::max(1, s->G), st));
-    for (cudaEvent_t& e : s->ev_load) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&s->ev_gather, cudaEventDisableTiming));
-  }
   CK(cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming));  // last: marks completion
   return MPM_OK;
+}
+
+// Buffer set B of the reverse steps that are binned, or whose sorts load, on a branch (allocated on the
+// first reverse pass that does; all or nothing).
+mpm_status ensure_set_b_parts(mpm_scene* s) {
+  const int nt = s->hp.n_tiles;
+  const bool bins = s->b.bin_ctl != nullptr;
+  std::vector<void*>& L = s->set_b_allocs;
+  cudaStream_t st = s->ctx->stream;
+  BatchDev& bb = s->bB;  // only its sort arrays and record are used
+  bb = BatchDev{};
+  CKS(dalloc(&s->curB, 2, L));
+  CKS(dalloc(&s->keyB, s->npad, L));
+  CKS(dalloc(&s->actB, std::max(1, s->G), L));
+  CKS(dalloc(&s->d_gstep, 1, L));
+  CKS(dalloc(&bb.tile_start, nt + 1, L));
+  CKS(dalloc(&bb.tile_slot, nt, L));
+  CKS(dalloc(&bb.active, nt, L));
+  CKS(dalloc(&bb.n_active, 1, L));
+  if (bins)
+    CKS(alloc_bins(bb, s->dim, s->b.tile_edge, nt, L));
+  else
+    CKS(dalloc(&bb.sorted, s->npad, L));
+  bb.scenes = s->curB;
+  CK(cudaMemsetAsync(s->actB, 0, sizeof(float) * std::max(1, s->G), st));
+  for (cudaEvent_t& e : s->ev_load) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  return cuda_fail(cudaEventCreateWithFlags(&s->ev_gather, cudaEventDisableTiming));
+}
+
+void free_set_b(mpm_scene* s) {
+  for (void* p : s->set_b_allocs) cudaFree(p);
+  s->set_b_allocs.clear();
+  s->curB = nullptr;
+  s->keyB = nullptr;
+  s->actB = nullptr;
+  s->d_gstep = nullptr;
+  for (cudaEvent_t& e : s->ev_load) {
+    if (e) cudaEventDestroy(e);
+    e = nullptr;
+  }
+  if (s->ev_gather) cudaEventDestroy(s->ev_gather);
+  s->ev_gather = nullptr;
+}
+
+mpm_status ensure_set_b(mpm_scene* s) {
+  if (!s->ctrl_branch || s->ev_gather) return MPM_OK;  // the event is the last thing made
+  const mpm_status st = ensure_set_b_parts(s);
+  if (st != MPM_OK) free_set_b(s);
+  return st;
 }
 
 void free_ws2(mpm_scene* s) {
@@ -790,16 +822,6 @@ void free_ws2(mpm_scene* s) {
   }
   if (s->ev_fork) cudaEventDestroy(s->ev_fork);
   s->ev_fork = nullptr;
-  s->curB = nullptr;
-  s->keyB = nullptr;
-  s->actB = nullptr;
-  s->d_gstep = nullptr;
-  for (cudaEvent_t& e : s->ev_load) {
-    if (e) cudaEventDestroy(e);
-    e = nullptr;
-  }
-  if (s->ev_gather) cudaEventDestroy(s->ev_gather);
-  s->ev_gather = nullptr;
 }
 
 }  // namespace
@@ -1006,6 +1028,8 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
   const bool overlap = !mean_x0_seed && !(flags & BW_NO_OVERLAP) && s->impl == MPM_IMPL_TILED && k > 1 && nseg > 1 &&
                        (s->roll_budget == 0 ||
                         (size_t(nseg) + 2 * size_t(k - 1)) * S + store_bytes <= s->roll_budget);
+  const bool branch = overlap || (!mean_x0_seed && !(flags & BW_NO_OVERLAP) && s->b.bin_ctl && k == 1);
+  if (branch) CKS(ensure_set_b(s));
   if (overlap) {
     CKS(ensure_ws2(s));
     if (int(s->seg2.size()) != k - 1) {
@@ -1018,7 +1042,8 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
       CKS(dalloc(&s->sort_store, (store_bytes - ctrl_bytes) / sizeof(uint32_t), s->roll_allocs));
     if (keep_ctrl && !s->ctrl_store) CKS(dalloc(&s->ctrl_store, ctrl_bytes / sizeof(float), s->roll_allocs));
   }
-  if (s->graphs_ws2 != overlap) {  // recompute and reverse graphs name the workspace and sort path
+  // recompute and reverse graphs name the workspace and the way states are binned
+  if (s->graphs_ws2 != overlap || s->graphs_branch != branch) {
     for (int ph : {PH_RCM, PH_PREP, PH_REV})
       for (auto& g : s->graphs[ph])
         if (g.exec) {
@@ -1026,6 +1051,7 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
           g = Graph();
         }
     s->graphs_ws2 = overlap;
+    s->graphs_branch = branch;
   }
   s->rcm_ws2 = overlap;
   // table 2: per segment the recompute records F_{sg,j} (state j -> j+1) and the reverse records
@@ -1160,6 +1186,9 @@ mpm_status recompute_segment(mpm_scene* s, int sg, cudaStream_t st) {
 mpm_status reverse_segments(mpm_scene* s) {
   const int T = s->roll_T, k = s->roll_k, nseg = s->roll_nseg;
   mpm_ctx* c = s->ctx;
+  // every state kept: no segment ends the run of reverse steps, which replays whole graphs (a graph
+  // per one-step segment took 20.2 us a step on 1,024 particles, 13.4 with these)
+  if (k == 1) return run_phase(s, PH_REV, T);
   const bool overlap = s->rcm_ws2 && !c->prof_mask && !tune_wants(s, PH_RCM) && !tune_wants(s, PH_REV) &&
                        !tune_wants(s, PH_PREP);
   if (!overlap) {
@@ -1502,6 +1531,7 @@ mpm_status mpm_scene_destroy(mpm_scene* s) {
   free_rollout(s);
   free_ml_pool(s);
   free_ws2(s);
+  free_set_b(s);
   invalidate_graphs(s);
   tune_release(s);
   for (void* p : s->allocs) cudaFree(p);
@@ -2046,9 +2076,9 @@ mpm_status mpm_set_ctrl_params(mpm_scene* s, const float* params, int n, int mem
   CK(cudaStreamSynchronize(s->ctx->stream));
   CK(cudaMemcpy(const_cast<float*>(s->ctrl.params), params, sizeof(float) * n,
                 mem_space == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice));
-  // a device-to-device copy may still run when the call returns, and the controller kernels read the
+  // a device-to-device copy may still run when the call returns, and the MLP's kernels read the
   // parameters ahead of their place in the stream
-  if (mem_space == 1) CK(cudaStreamSynchronize(cudaStreamLegacy));
+  if (mem_space == 1 && s->ctrl.type == MPM_CTRL_MLP) CK(cudaStreamSynchronize(cudaStreamLegacy));
   return MPM_OK;
 }
 

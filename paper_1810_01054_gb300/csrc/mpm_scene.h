@@ -149,13 +149,14 @@ struct mpm_scene {
   uint32_t* key2 = nullptr;
   float* act2 = nullptr;
   float4* grid2 = nullptr;
-  std::vector<void*> ws2_allocs;
+  std::vector<void*> ws2_allocs, set_b_allocs;
   std::vector<float4*> seg2;
   uint32_t* sort_store = nullptr;  // 2 x k slots (segment parity, state in segment) of sorts
   float* ctrl_store = nullptr;     // the same slots of controller inputs and actuations (controllers
                                    // that read the state)
   bool rcm_ws2 = false;     // the reverse tables send the recompute to workspace 2
   bool graphs_ws2 = false;  // workspace the recompute graphs were captured with
+  bool graphs_branch = false;  // whether the reverse graphs bin (or load sorts) on a branch
   size_t roll_budget = 0;
   cudaEvent_t ev_rcm[2] = {}, ev_rev[2] = {}, ev_fork = nullptr;
   // Reverse graphs of a tiled scene whose controller reads no state: each step's controller
