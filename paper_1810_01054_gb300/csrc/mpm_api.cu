@@ -1028,8 +1028,16 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
   const bool overlap = !mean_x0_seed && !(flags & BW_NO_OVERLAP) && s->impl == MPM_IMPL_TILED && k > 1 && nseg > 1 &&
                        (s->roll_budget == 0 ||
                         (size_t(nseg) + 2 * size_t(k - 1)) * S + store_bytes <= s->roll_budget);
-  const bool branch = overlap || (!mean_x0_seed && !(flags & BW_NO_OVERLAP) && s->b.bin_ctl && k == 1);
-  if (branch) CKS(ensure_set_b(s));
+  bool branch = overlap || (!mean_x0_seed && !(flags & BW_NO_OVERLAP) && s->b.bin_ctl && k == 1);
+  if (branch) {
+    const mpm_status st_b = ensure_set_b(s);
+    if (st_b == MPM_ERR_OOM && !overlap) {
+      cudaGetLastError();  // the failed allocation's error: the states are binned in line instead
+      branch = false;
+    } else {
+      CKS(st_b);
+    }
+  }
   if (overlap) {
     CKS(ensure_ws2(s));
     if (int(s->seg2.size()) != k - 1) {

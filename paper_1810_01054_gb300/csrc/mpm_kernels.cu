@@ -1,17 +1,18 @@
 // sm_103a kernels of the differentiable MLS-MPM step (ChainQueen, arXiv 1810.01054).
 //
 // Forward step (Section III, Eqs. 3-10), tiled form:
-//   k_hist / scan / k_scatter : bin particles by the tile of their stencil base cell
+//   tile bins                 : up to 2048 tiles, the kernel that moves a particle (k_g2p; k_keys at a
+//                               phase's start) appends it to the list of its stencil base's tile;
+//   k_keys / scan / k_scatter : beyond that a sort by tile (k_g2p writes the next step's keys)
 //   k_p2g                     : per tile, canonical (cell, id) order, per-particle stress and
 //                               MLS matrix G (Eq. 4), per-cell register accumulation of the
 //                               3^d stencil (Eqs. 3, 5), fixed-order reduction into the tile's
 //                               (B+2)^d node block -- no atomics on floating point anywhere
-//   k_grid                    : sums the <= 2^d node blocks covering each node in a fixed order,
-//                               Eq. 6, gravity, boundary (S5)
-//   k_g2p                     : per tile, node block staged in shared memory, Eqs. 7-10 and the
-//                               next step's bin key
-// Reverse step (Supplement S2-S5): k_p2g also scatters (C) from (A), (B) in the same pass; k_grid
-// applies (L), (D), (E); k_adj_gather evaluates (F)-(K), (J).
+//   k_g2p                     : per tile, the <= 2^d node blocks covering each node summed in a fixed
+//                               order into shared memory, Eq. 6, gravity, boundary (S5) there, then
+//                               Eqs. 7-10 and the next step's bin entry or key
+// Reverse step (Supplement S2-S5): k_p2g also scatters (C) from (A), (B) in the same pass;
+// k_adj_gather applies (L), (D), (E) to its node block and evaluates (F)-(K), (J).
 //
 // Every floating-point sum has a fixed order, so results are bitwise reproducible run to run and
 // independent of which other scenes share the launch.
