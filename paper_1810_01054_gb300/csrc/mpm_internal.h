@@ -158,11 +158,12 @@ struct BatchDev {
   //   word 1  parity the gathers read (written by P2G); the appending kernel fills the other one
   //   words BIN_MASK .., two masks of BIN_WORDS; then two counts of total_tiles
   // P2G clears the other parity's mask and counts; a phase starts from all zeros (launch_keys).
-  // The line at BIN_TILES: the lists take 8 or 16 KB a tile and set (their room cannot overflow before
-  // the tile's kernels refuse it), 64 MB at most, and a tile mask of 64 words is read by every CTA;
-  // beyond it a step is long enough that the sort's launches (19 of 143 us at one million particles)
-  // matter less.  Steps with bins against the sort: 1,024 particles (2D) 13.3 -> 10.9 us, the 31k
-  // walker 16.9 -> 13.9 us.
+  // The line at BIN_TILES: the two lists take 16 or 32 KB a tile and set (their room cannot overflow
+  // before the tile's kernels refuse it), 128 MB at most, and a tile mask of 128 words is a word per
+  // thread of the smallest CTA; beyond it a step is long enough that the sort's launches (19 of 143 us
+  // at one million particles) matter less.  Steps with bins against the sort: 1,024 particles (2D)
+  // 13.3 -> 10.9 us, the 31k walker 16.9 -> 13.9 us; 24 steps with the gradient of the 95k soft body
+  // (4096 tiles) 3479 -> 2947 us.
   uint32_t *bin_ctl, *bin_raw;
   int rec_flip;         // scenes[] holds one scene's records by parity (a scene alone, with bins)
   float4* partial;      // [total_tiles * BLOCK_NODES] node blocks of P2G
@@ -180,7 +181,7 @@ struct BatchDev {
   int* rewind_rows;
 };
 
-constexpr int BIN_TILES = 2048;                 // most tiles a batch with bins holds
+constexpr int BIN_TILES = 4096;                 // most tiles a batch with bins holds
 constexpr int BIN_WORDS = BIN_TILES / 32;       // words of a tile mask
 constexpr int BIN_MASK = 4;                     // first mask word in bin_ctl
 constexpr int BIN_COUNT = BIN_MASK + 2 * BIN_WORDS;  // first count word

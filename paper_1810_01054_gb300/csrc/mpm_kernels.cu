@@ -1,7 +1,7 @@
 // sm_103a kernels of the differentiable MLS-MPM step (ChainQueen, arXiv 1810.01054).
 //
 // Forward step (Section III, Eqs. 3-10), tiled form:
-//   tile bins                 : up to 2048 tiles, the kernel that moves a particle (k_g2p; k_keys at a
+//   tile bins                 : up to 4096 tiles, the kernel that moves a particle (k_g2p; k_keys at a
 //                               phase's start) appends it to the list of its stencil base's tile;
 //   k_keys / scan / k_scatter : beyond that a sort by tile (k_g2p writes the next step's keys)
 //   k_p2g                     : per tile, canonical (cell, id) order, per-particle stress and
@@ -272,20 +272,29 @@ __device__ __forceinline__ uint32_t bin_view(const BatchDev& b, int which, BinVi
   if (tid < SCENE_WORDS) reinterpret_cast<int*>(&sh.sp)[tid] = p ? r1 : r0;
   __syncthreads();
   if (tid < 32) {
-    const int c0 = __popc(v.mask[tid]), c1 = __popc(v.mask[tid + 32]);
-    int i0 = c0, i1 = c1;
+    // counts of the words tid, tid + 32, ..., two to an integer (a count stays below 2^16)
+    uint32_t c[BIN_WORDS / 64], inc[BIN_WORDS / 64], base = 0;
+#pragma unroll
+    for (int i = 0; i < BIN_WORDS / 64; ++i)
+      inc[i] = c[i] = uint32_t(__popc(v.mask[tid + 64 * i])) | uint32_t(__popc(v.mask[tid + 64 * i + 32])) << 16;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int a0 = __shfl_up_sync(0xffffffffu, i0, o), a1 = __shfl_up_sync(0xffffffffu, i1, o);
-      if (tid >= o) {
-        i0 += a0;
-        i1 += a1;
-      }
+      uint32_t up[BIN_WORDS / 64];
+#pragma unroll
+      for (int i = 0; i < BIN_WORDS / 64; ++i) up[i] = __shfl_up_sync(0xffffffffu, inc[i], o);
+#pragma unroll
+      for (int i = 0; i < BIN_WORDS / 64; ++i)
+        if (tid >= o) inc[i] += up[i];
     }
-    const int tot0 = __shfl_sync(0xffffffffu, i0, 31);
-    v.before[tid] = uint32_t(i0 - c0);
-    v.before[tid + 32] = uint32_t(tot0 + i1 - c1);
-    if (tid == 31) v.n = tot0 + i1;
+#pragma unroll
+    for (int i = 0; i < BIN_WORDS / 64; ++i) {
+      const uint32_t tot = __shfl_sync(0xffffffffu, inc[i], 31), ex = inc[i] - c[i];
+      v.before[tid + 64 * i] = base + (ex & 0xffffu);
+      base += tot & 0xffffu;
+      v.before[tid + 64 * i + 32] = base + (ex >> 16);
+      base += tot >> 16;
+    }
+    if (tid == 31) v.n = int(base);
   }
   __syncthreads();
   return p;
@@ -294,9 +303,9 @@ __device__ __forceinline__ uint32_t bin_view(const BatchDev& b, int which, BinVi
 // Tile of active slot `slot` < v.n (all 32 lanes of a warp call it).
 __device__ __forceinline__ int bin_tile(const BinView& v, int slot) {
   const int lane = threadIdx.x & 31;
-  const unsigned b0 = __ballot_sync(0xffffffffu, int(v.before[lane]) <= slot);
-  const unsigned b1 = __ballot_sync(0xffffffffu, int(v.before[lane + 32]) <= slot);
-  const int w = __popc(b0) + __popc(b1) - 1;  // the last word that starts at or before it
+  int w = -1;  // the last word that starts at or before it
+#pragma unroll
+  for (int i = 0; i < BIN_WORDS / 32; ++i) w += __popc(__ballot_sync(0xffffffffu, int(v.before[lane + 32 * i]) <= slot));
   const uint32_t word = v.mask[w];
   const int r = slot - int(v.before[w]);
   const unsigned hit = __ballot_sync(0xffffffffu, ((word >> lane) & 1u) && __popc(word & ((1u << lane) - 1u)) == r);

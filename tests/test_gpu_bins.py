@@ -1,4 +1,4 @@
-"""Tile bins against the sort: scenes of at most 2048 tiles keep a list per tile that the step itself
+"""Tile bins against the sort: scenes of at most 4096 tiles keep a list per tile that the step itself
 appends to, larger ones sort their particles by tile every step.  The same particles in a grid on
 either side of that line give the same bits (the grids differ only at walls nothing is near), over
 forward steps, checkpointed rollouts and their reverse passes.
@@ -35,8 +35,8 @@ def _body(dim, edge, ctrl, n):
     return s.copy(n_grid=n, v0=v, tile_edge=edge if dim == 2 else 0)
 
 
-# grids of 2048 tiles (or fewer) and just above, by dimension and tile edge
-GRIDS = {(2, 4): ((256, 128), (260, 128)), (2, 8): ((512, 256), (520, 256)), (3, 4): ((64, 64, 32), (68, 64, 32))}
+# grids of 4096 tiles and just above, by dimension and tile edge
+GRIDS = {(2, 4): ((256, 256), (260, 256)), (2, 8): ((512, 512), (520, 512)), (3, 4): ((64, 64, 64), (68, 64, 64))}
 
 
 @pytest.mark.parametrize("ctrl", [S.CTRL_SIN, S.CTRL_TABLE, S.CTRL_MLP, S.CTRL_COM])
@@ -46,10 +46,6 @@ def test_bins_give_the_bits_of_the_sort(M, ctx, shape, ctrl):
     res = []
     for n in GRIDS[shape]:
         spec = _body(dim, edge, ctrl, n)
-        if dim == 3:  # the blob sits lower than the short third axis
-            x = np.array(spec.x0)
-            x[:, 2] -= 0.15
-            spec = spec.copy(x0=x)
         got = []
         for steps, k in ((11, 1), (11, 4), (3, 2)):  # graph lengths 8 + 3 and 3; segments of 4, 4, 3
             sc = M.Scene(ctx, spec)
