@@ -69,12 +69,29 @@ mpm_status dalloc(T** p, size_t count, std::vector<void*>& list) {
 
 // Tile bins of a batch of `tiles` tiles (at most BIN_TILES): control words and the appended lists;
 // the canonical lists take the place of `sorted`.
+size_t bin_words(int dim, int edge, int tiles, size_t* ctl, size_t* room) {
+  *room = size_t(tiles) * bin_cap(dim, edge);
+  *ctl = (bin_ctl_words(tiles) + 63) / 64 * 64;
+  return *ctl + 2 * *room;
+}
 mpm_status alloc_bins(BatchDev& b, int dim, int edge, int tiles, std::vector<void*>& list) {
-  const size_t room = size_t(tiles) * bin_cap(dim, edge), ctl = (bin_ctl_words(tiles) + 63) / 64 * 64;
-  CKS(dalloc(&b.bin_ctl, ctl + 2 * room, list));
+  size_t ctl, room;
+  CKS(dalloc(&b.bin_ctl, bin_words(dim, edge, tiles, &ctl, &room), list));
   b.bin_raw = b.bin_ctl + ctl;
   b.sorted = b.bin_raw + room;
   return MPM_OK;
+}
+
+// Counts a new scene's bins against its context's BIN_BYTES; false (nothing counted) beyond.
+bool reserve_bins(mpm_scene* s, int edge, int tiles) {
+  size_t ctl, room;
+  const size_t bytes = bin_words(s->dim, edge, tiles, &ctl, &room) * sizeof(uint32_t);
+  if (s->ctx->bin_bytes.fetch_add(bytes) + bytes > BIN_BYTES) {
+    s->ctx->bin_bytes.fetch_sub(bytes);
+    return false;
+  }
+  s->bin_bytes = bytes;
+  return true;
 }
 
 int planes_of(int dim) { return dim == 2 ? Cfg<2>::PLANES : Cfg<3>::PLANES; }
@@ -1552,6 +1569,7 @@ mpm_status mpm_scene_destroy(mpm_scene* s) {
     if (q) cudaFree(q);
   for (cudaEvent_t e : s->ev_ctrl)
     if (e) cudaEventDestroy(e);
+  s->ctx->bin_bytes.fetch_sub(s->bin_bytes);
   s->ctx->live.fetch_sub(1);
   delete s;
   return MPM_OK;
@@ -1731,12 +1749,20 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   ALLOC(b.n_active, 1);
   ALLOC(b.block_sums, 2 * ((p.n_tiles + 2047) / 2048) + 2);
   ALLOC(b.work, 4);
-  if (s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES) {
-    TRY(alloc_bins(b, dim, edge, p.n_tiles, s->allocs));
-    b.rec_flip = 1;
-  } else {
-    ALLOC(b.sorted, s->npad);
+  bool bins = s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES && reserve_bins(s, edge, p.n_tiles);
+  if (bins) {
+    st = alloc_bins(b, dim, edge, p.n_tiles, s->allocs);
+    if (st == MPM_ERR_OOM) {
+      cudaGetLastError();  // the failed allocation's error: the scene sorts instead
+      bins = false;
+    } else if (st != MPM_OK) {
+      return fail(st);
+    }
   }
+  if (bins)
+    b.rec_flip = 1;
+  else
+    ALLOC(b.sorted, s->npad);
   if (s->impl == MPM_IMPL_TILED) {
     ALLOC(b.partial, size_t(p.n_tiles) * NB);
     ALLOC(b.partial_b, size_t(p.n_tiles) * NB);

@@ -182,6 +182,9 @@ struct BatchDev {
 };
 
 constexpr int BIN_TILES = 4096;                 // most tiles a batch with bins holds
+// Most bytes the bins of a context's scenes take (128 scenes of 4096 3D tiles, 4096 of 256 2D tiles);
+// further scenes sort, with the same results, so that thousands of small scenes still fit the device.
+constexpr size_t BIN_BYTES = size_t(16) << 30;
 constexpr int BIN_WORDS = BIN_TILES / 32;       // words of a tile mask
 constexpr int BIN_MASK = 4;                     // first mask word in bin_ctl
 constexpr int BIN_COUNT = BIN_MASK + 2 * BIN_WORDS;  // first count word

@@ -47,6 +47,7 @@ struct mpm_ctx {
   std::vector<int> prof_kind;
   int prof_used = 0;
   std::atomic<int> live{0};  // scenes and batches created on this context and not yet destroyed
+  std::atomic<size_t> bin_bytes{0};  // tile bins of its scenes, at most BIN_BYTES
 };
 
 struct Graph {
@@ -138,6 +139,7 @@ struct mpm_scene {
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
   TuneState tune;
+  size_t bin_bytes = 0;     // of the context's, this scene's tile bins
   bool keys_stale = false;  // a batch advanced the state since its bin keys were made
   int batch_refs = 0;  // batch slots holding the scene (admitted, not yet released)
   // The segment recompute's own workspace (tile arrays, selected record, bin keys, actuation,

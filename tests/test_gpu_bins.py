@@ -115,3 +115,27 @@ def test_cta_sizes_of_3d_scenes_give_the_same_bits(M, ctx, N):
         for sc in scenes:
             sc.close()
     assert np.abs(want[-1]).max() > 0
+
+
+def test_scenes_beyond_the_bins_room_sort(M, ctx):
+    """A context's scenes hold 16 GiB of tile bins between them (128 MB for 64^3 cells, the control
+    words beside); the next scene sorts, takes less memory and gives the same bits."""
+    import torch
+    spec = _body(3, 4, S.CTRL_SIN, (64, 64, 64))
+    free = [torch.cuda.mem_get_info()[0]]
+    scenes = []
+    for _ in range(130):
+        scenes.append(M.Scene(ctx, spec))
+        free.append(torch.cuda.mem_get_info()[0])
+    took = [a - b for a, b in zip(free, free[1:])]
+    assert min(took[:127]) - max(took[128:]) > 100 << 20
+    for sc in scenes[1:-1]:
+        sc.close()
+    got = []
+    for sc in (scenes[0], scenes[-1]):
+        sc.rollout(5, 2)
+        seed = np.ones((sc.N, 3))
+        got.append(sc.get_state() + sc.backward(seed))
+        sc.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
