@@ -163,7 +163,7 @@ struct BatchDev {
   // thread of the smallest CTA; beyond it a step is long enough that the sort's launches (19 of 143 us
   // at one million particles) matter less.  Steps with bins against the sort: 1,024 particles (2D)
   // 13.3 -> 10.9 us, the 31k walker 16.9 -> 13.9 us; 24 steps with the gradient of the 95k soft body
-  // (4096 tiles) 3479 -> 2947 us.
+  // (4096 tiles) 3434-3479 -> 2947-3040 us.
   uint32_t *bin_ctl, *bin_raw;
   int rec_flip;         // scenes[] holds one scene's records by parity (a scene alone, with bins)
   float4* partial;      // [total_tiles * BLOCK_NODES] node blocks of P2G
