@@ -138,7 +138,8 @@ constexpr int SCENE_WORDS = int(sizeof(ScenePar) / sizeof(int));
 static_assert(SCENE_WORDS <= 128, "one word per thread of the smallest tile kernel");
 
 // Requests the actuations of the staged record: asynchronous copies, so nobody waits for them here.
-// The caller waits for its own copies (cp_async_wait_all) before the barrier that precedes their use.
+// The caller waits for its own copies (cp_async_wait_all) before the barrier that precedes their use,
+// and on every way out of the kernel: a CTA's shared memory is handed on when it ends.
 template <int D>
 __device__ __forceinline__ void stage_actuation(SceneShared& sh) {
   const int G = sh.sp.G;
@@ -1208,6 +1209,7 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
     __syncthreads();
   }
   if (dyn) release_work(b, 0);
+  cp_async_wait_all();  // a CTA without a tile, or whose last one was skipped, still has the actuations under way
 }
 
 // ============================================================================ grid
@@ -2112,6 +2114,7 @@ __global__ void __launch_bounds__(T, 512 / T) k_adj_gather(BatchDev b) {
     __syncthreads();
   }
   if (dyn) release_work(b, 1);
+  cp_async_wait_all();  // a CTA without a tile, or whose last one was skipped, still has the actuations under way
 }
 
 // ============================================================================ launchers (tiled)
