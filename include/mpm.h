@@ -193,7 +193,9 @@ mpm_status mpm_get_state(mpm_scene* scene, int step, float* x, float* v, float* 
  * non-finite inputs are reported (MPM_ERR_ARG) by the next synchronising call. */
 mpm_status mpm_set_state(mpm_scene* scene, const float* x, const float* v, const float* C, const float* F,
                          int step, int mem_space);
-/* Replaces the controller parameters (n must equal the scene's parameter count). */
+/* Replaces the controller parameters (n must equal the scene's parameter count) for every step
+ * enqueued afterwards.  Device arrays are copied in the context stream's order, after the work the
+ * legacy default stream holds at the call; host arrays are copied before the call returns. */
 mpm_status mpm_set_ctrl_params(mpm_scene* scene, const float* params, int n, int mem_space);
 /* Per-particle material (an extension: the paper's co-design and inference examples treat
  * material parameters as optimisation variables, Sections V-A and V-C).  E [N] Young's modulus and

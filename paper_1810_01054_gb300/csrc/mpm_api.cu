@@ -67,6 +67,16 @@ mpm_status dalloc(T** p, size_t count, std::vector<void*>& list) {
   return MPM_OK;
 }
 
+// Copies host data to device memory ahead of whatever the stream runs next, and waits: a cudaMemcpy
+// would go to the legacy stream, which nothing on a non-blocking stream waits for, and from pageable
+// memory it may return before the data has landed.
+mpm_status upload(cudaStream_t st, void* dst, const void* src, size_t bytes) {
+  if (bytes == 0) return MPM_OK;
+  CK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st));
+  CK(cudaStreamSynchronize(st));
+  return MPM_OK;
+}
+
 // Tile bins of a batch of `tiles` tiles (at most BIN_TILES): control words and the appended lists;
 // the canonical lists take the place of `sorted`.
 size_t bin_words(int dim, int edge, int tiles, size_t* ctl, size_t* room) {
@@ -228,7 +238,7 @@ mpm_status storage_order(mpm_scene* s, const mpm_scene_desc* d, int dim) {
   s->b.occupied = occupied;
   int* dorder = nullptr;
   CKS(dalloc(&dorder, size_t(N), s->allocs));
-  CK(cudaMemcpy(dorder, s->h_order.data(), sizeof(int) * size_t(N), cudaMemcpyHostToDevice));
+  CKS(upload(s->ctx->stream, dorder, s->h_order.data(), sizeof(int) * size_t(N)));
   s->d_order = dorder;
   return MPM_OK;
 }
@@ -279,9 +289,7 @@ bool refresh_branch_sel(mpm_scene* s) {
 
 mpm_status upload_sel(mpm_scene* s) {
   refresh_branch_sel(s);
-  CK(cudaStreamSynchronize(s->ctx->stream));
-  CK(cudaMemcpy(s->dsel, s->hsel, sizeof(s->hsel), cudaMemcpyHostToDevice));
-  return MPM_OK;
+  return upload(s->ctx->stream, s->dsel, s->hsel, sizeof(s->hsel));
 }
 
 // Upload a table of scene records unless the device already holds exactly this table.
@@ -290,9 +298,9 @@ mpm_status upload_table(mpm_scene* s, int which, const std::vector<ScenePar>& co
   const bool same = t.host.size() == confs.size() &&
                     std::memcmp(t.host.data(), confs.data(), sizeof(ScenePar) * confs.size()) == 0;
   if (same) return MPM_OK;
-  CK(cudaStreamSynchronize(s->ctx->stream));
   bool moved = false;
   if (int(confs.size()) > t.cap) {
+    CK(cudaStreamSynchronize(s->ctx->stream));
     if (t.dev) cudaFree(t.dev);
     t.dev = nullptr;
     t.cap = 0;
@@ -300,7 +308,7 @@ mpm_status upload_table(mpm_scene* s, int which, const std::vector<ScenePar>& co
     t.cap = int(confs.size());
     moved = true;
   }
-  CK(cudaMemcpy(t.dev, confs.data(), sizeof(ScenePar) * confs.size(), cudaMemcpyHostToDevice));
+  CKS(upload(s->ctx->stream, t.dev, confs.data(), sizeof(ScenePar) * confs.size()));
   t.host = confs;
   if (moved) {
     for (int ph = 0; ph < PH_COUNT; ++ph) {
@@ -324,8 +332,8 @@ mpm_status upload_map(mpm_scene* s, int which, const std::vector<int>& m, int ba
       sel_changed = true;
     }
   if (!same) {
-    CK(cudaStreamSynchronize(s->ctx->stream));
     if (int(m.size()) > mp.cap) {
+      CK(cudaStreamSynchronize(s->ctx->stream));
       if (mp.dev) cudaFree(mp.dev);
       mp.dev = nullptr;
       mp.cap = 0;
@@ -335,7 +343,7 @@ mpm_status upload_map(mpm_scene* s, int which, const std::vector<int>& m, int ba
         if (ph >= 0) s->hsel[ph].map = mp.dev;
       sel_changed = true;
     }
-    if (!m.empty()) CK(cudaMemcpy(mp.dev, m.data(), sizeof(int) * m.size(), cudaMemcpyHostToDevice));
+    CKS(upload(s->ctx->stream, mp.dev, m.data(), sizeof(int) * m.size()));
     mp.host = m;
   }
   if (sel_changed) CKS(upload_sel(s));
@@ -1569,6 +1577,7 @@ mpm_status mpm_scene_destroy(mpm_scene* s) {
     if (q) cudaFree(q);
   for (cudaEvent_t e : s->ev_ctrl)
     if (e) cudaEventDestroy(e);
+  if (s->ev_params) cudaEventDestroy(s->ev_params);
   s->ctx->bin_bytes.fetch_sub(s->bin_bytes);
   s->ctx->live.fetch_sub(1);
   delete s;
@@ -1852,6 +1861,7 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
     cp.perm = perm;
     cp.pgroup = pgroup;
   }
+  // (these copies go to the legacy stream; read_status below copies back behind them)
   TRY(cuda_fail(cudaMemcpy(act_dir, hdir.data(), sizeof(float) * hdir.size(), cudaMemcpyHostToDevice)));
   TRY(cuda_fail(cudaMemcpy(params, hparams.data(), sizeof(float) * hparams.size(), cudaMemcpyHostToDevice)));
   TRY(cuda_fail(cudaMemcpy(inv_count, hinv.data(), sizeof(float) * hinv.size(), cudaMemcpyHostToDevice)));
@@ -2107,12 +2117,20 @@ mpm_status mpm_set_ctrl_params(mpm_scene* s, const float* params, int n, int mem
   if (!s || n != s->nparams || (n > 0 && !params)) return MPM_ERR_ARG;
   if (s->batch_refs > 0) return MPM_ERR_STATE;
   if (n == 0) return MPM_OK;
-  CK(cudaStreamSynchronize(s->ctx->stream));
-  CK(cudaMemcpy(const_cast<float*>(s->ctrl.params), params, sizeof(float) * n,
-                mem_space == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice));
-  // a device-to-device copy may still run when the call returns, and the MLP's kernels read the
-  // parameters ahead of their place in the stream
-  if (mem_space == 1 && s->ctrl.type == MPM_CTRL_MLP) CK(cudaStreamSynchronize(cudaStreamLegacy));
+  // The copy takes its place on the scene's stream, so every kernel launched after it reads the new
+  // parameters: also the MLP's, which read them ahead of the kernel before (a copy has no early end
+  // that they could overtake).
+  cudaStream_t st = s->ctx->stream;
+  float* dst = const_cast<float*>(s->ctrl.params);
+  if (mem_space != 1) return upload(st, dst, params, sizeof(float) * n);
+  // device arrays may come from the legacy stream and be written there again: it and the copy wait
+  // for each other, the host for neither
+  if (!s->ev_params) CK(cudaEventCreateWithFlags(&s->ev_params, cudaEventDisableTiming));
+  CK(cudaEventRecord(s->ev_params, cudaStreamLegacy));
+  CK(cudaStreamWaitEvent(st, s->ev_params, 0));
+  CK(cudaMemcpyAsync(dst, params, sizeof(float) * n, cudaMemcpyDeviceToDevice, st));
+  CK(cudaEventRecord(s->ev_params, st));
+  CK(cudaStreamWaitEvent(cudaStreamLegacy, s->ev_params, 0));
   return MPM_OK;
 }
 
@@ -2151,11 +2169,11 @@ mpm_status mpm_scene_set_material(mpm_scene* s, const float* E, const float* mas
   std::vector<float> tmp(std::max(N, 1));
   if (E && N > 0) {
     for (int p = 0; p < N; ++p) tmp[p] = hE[s->h_order[p]];
-    CK(cudaMemcpy(s->d_pE, tmp.data(), fb, cudaMemcpyHostToDevice));
+    CKS(upload(s->ctx->stream, s->d_pE, tmp.data(), fb));
   }
   if (mass && N > 0) {
     for (int p = 0; p < N; ++p) tmp[p] = hm[s->h_order[p]];
-    CK(cudaMemcpy(s->d_pmass, tmp.data(), fb, cudaMemcpyHostToDevice));
+    CKS(upload(s->ctx->stream, s->d_pmass, tmp.data(), fb));
   }
   s->hp.pE = E ? s->d_pE : nullptr;
   s->hp.pmass = mass ? s->d_pmass : nullptr;

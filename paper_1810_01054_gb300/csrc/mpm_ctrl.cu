@@ -173,8 +173,8 @@ __device__ __forceinline__ void dot_rows(const float* A, int so, int sj, const f
 // The MLP's parameters (W1, b1, W2, b2, W3, b3, contiguous) copied to shared memory in one pass
 // when they fit (the soft body's 48-64-64-16 network: 8336 floats), so the layers read no global
 // memory; else the global copy.  Asynchronous copies, requested before pdl_enter() (parameters only
-// change between launches, behind a wait for the stream), so they arrive while the kernel before
-// still runs; mlp_params_ready() before the barrier that precedes their use.  Every thread calls both.
+// change by a copy on the stream, and no kernel starts before such a copy has ended), so they arrive
+// while the kernel before still runs; mlp_params_ready() before the barrier that precedes their use.  Every thread calls both.
 constexpr int MLP_STAGE = 8704;
 __device__ __forceinline__ const float* mlp_params(const CtrlPar& c, float* stage) {
   const int G = c.G, Z = G * c.dim, H = c.hidden;

@@ -178,6 +178,7 @@ struct mpm_scene {
   bool ctrl_join = false;          // a branch is captured and not yet joined
   int* d_rows = nullptr;           // active-slot count of the last adjoint gather
   cudaEvent_t ev_ctrl[2] = {};     // fork, join
+  cudaEvent_t ev_params = nullptr; // orders a device upload of the controller parameters
   // while set, set_counter appends (counter, value) here instead of launching a write: the batch
   // scheduler writes the counters of all its scenes with one launch
   std::vector<std::pair<int*, int>>* ctr_sink = nullptr;
