@@ -63,6 +63,14 @@ mpm_status mpm_ctx_create(mpm_ctx** out, int device, void* cuda_stream);
 /* Destroys the context.  Every scene and batch created on it must be destroyed first:
  * MPM_ERR_STATE (and nothing freed) while any is alive. */
 mpm_status mpm_ctx_destroy(mpm_ctx* ctx);
+/* Tile bins: a tiled scene, or a batch, of at most 4096 tiles keeps a list per tile (16 or 32 KB a tile)
+ * instead of sorting its particles every step.  A context's bins take at most `most` bytes together
+ * (16 GiB unless set; every list counts: a scene's, the two further sets a checkpointed reverse pass
+ * of it may take, a batch's); a scene or batch created, or a reverse pass run, where they or the
+ * device's memory have no room sorts instead, with the same bits.  *held: the bytes taken now (NULL
+ * outputs are skipped).  A bound below what is held frees nothing. */
+mpm_status mpm_ctx_set_bin_bytes(mpm_ctx* ctx, size_t most);
+mpm_status mpm_ctx_bin_bytes(const mpm_ctx* ctx, size_t* held, size_t* most);
 /* Waits for the context's stream; returns the first CUDA error seen. */
 mpm_status mpm_sync(mpm_ctx* ctx);
 const char* mpm_status_str(mpm_status s);
@@ -143,7 +151,8 @@ mpm_status mpm_step(mpm_scene* scene, int n_steps);
  * recompute buffers and (beyond 4096 tiles) the sorts an overlapped reverse pass keeps fit, so that the fewest
  * steps are recomputed and the recompute runs beside the reverse steps; else about sqrt(n_steps);
  * mpm_scene_plan_rollout reports the choice); the states in between are recomputed by
- * mpm_backward.  mem_budget_bytes = 0 means no
+ * mpm_backward.  The further tile bins of the reverse pass are taken from what the budget leaves
+ * beside that.  mem_budget_bytes = 0 means no
  * limit.
  * With ckpt_interval = 0 and a budget below that single-level store ((ceil(T/k) + k - 1) states),
  * the rollout keeps a multi-level store instead: a recursive schedule (store a state, reverse the

@@ -77,33 +77,6 @@ mpm_status upload(cudaStream_t st, void* dst, const void* src, size_t bytes) {
   return MPM_OK;
 }
 
-// Tile bins of a batch of `tiles` tiles (at most BIN_TILES): control words and the appended lists;
-// the canonical lists take the place of `sorted`.
-size_t bin_words(int dim, int edge, int tiles, size_t* ctl, size_t* room) {
-  *room = size_t(tiles) * bin_cap(dim, edge);
-  *ctl = (bin_ctl_words(tiles) + 63) / 64 * 64;
-  return *ctl + 2 * *room;
-}
-mpm_status alloc_bins(BatchDev& b, int dim, int edge, int tiles, std::vector<void*>& list) {
-  size_t ctl, room;
-  CKS(dalloc(&b.bin_ctl, bin_words(dim, edge, tiles, &ctl, &room), list));
-  b.bin_raw = b.bin_ctl + ctl;
-  b.sorted = b.bin_raw + room;
-  return MPM_OK;
-}
-
-// Counts a new scene's bins against its context's BIN_BYTES; false (nothing counted) beyond.
-bool reserve_bins(mpm_scene* s, int edge, int tiles) {
-  size_t ctl, room;
-  const size_t bytes = bin_words(s->dim, edge, tiles, &ctl, &room) * sizeof(uint32_t);
-  if (s->ctx->bin_bytes.fetch_add(bytes) + bytes > BIN_BYTES) {
-    s->ctx->bin_bytes.fetch_sub(bytes);
-    return false;
-  }
-  s->bin_bytes = bytes;
-  return true;
-}
-
 int planes_of(int dim) { return dim == 2 ? Cfg<2>::PLANES : Cfg<3>::PLANES; }
 // Nodes of a tile's node block ((edge + 2)^dim).
 int block_nodes(int dim, int edge) {
@@ -438,7 +411,7 @@ mpm_status enqueue_forward(mpm_scene* s, int ph, cudaStream_t st) {
     CK(two ? launch_sort<2>(b, st, s->dsel + ph) : launch_sort<3>(b, st, s->dsel + ph));
     // keep the sort of this state for its reverse step (before P2G rewrites the tile lists in
     // canonical order without their cell tags)
-    if (ph == PH_RCM && s->rcm_ws2)
+    if (ph == PH_RCM && s->rcm_ws2 && s->sort_store)
       CK(two ? launch_store_sort<2>(b, nullptr, st) : launch_store_sort<3>(b, nullptr, st));
   }
   {
@@ -730,6 +703,38 @@ void free_rollout(mpm_scene* s) {
   s->have_rollout = false;
 }
 
+// The graphs of the reverse pass name the workspaces and the way states are binned.
+void drop_reverse_graphs(mpm_scene* s) {
+  for (int ph : {PH_RCM, PH_PREP, PH_REV})
+    for (auto& g : s->graphs[ph])
+      if (g.exec) {
+        cudaGraphExecDestroy(g.exec);
+        g = Graph();
+      }
+}
+
+// Gives up one of the scene's further sets of bins.
+mpm_status give_up_bins(mpm_scene* s, BinSet& set) {
+  if (!set.mem) return MPM_OK;
+  CK(cudaStreamSynchronize(s->ctx->stream));
+  drop_reverse_graphs(s);
+  drop_bins(s->ctx, set);
+  return MPM_OK;
+}
+
+// Takes (or keeps) a further set of bins for a reverse pass if *room bytes of its budget hold it and the
+// context and the device have it, and lessens *room by it; else gives it up.
+mpm_status further_bins(mpm_scene* s, BinSet& set, size_t* room) {
+  const size_t bytes = bin_set_bytes(s->dim, s->b.tile_edge, s->hp.n_tiles);
+  if (bytes > *room) return give_up_bins(s, set);
+  if (!set.mem) {
+    CKS(take_bins(s->ctx, set, bytes));
+    if (set.mem) drop_reverse_graphs(s);
+  }
+  *room -= set.bytes;
+  return MPM_OK;
+}
+
 void free_ws2(mpm_scene* s);
 
 // Workspace 2 (allocated on the first reverse pass that overlaps its recompute; all or nothing).
@@ -759,11 +764,8 @@ mpm_status ensure_ws2_parts(mpm_scene* s) {
   CKS(dalloc(&b.block_sums, 2 * ((nt + 2047) / 2048) + 2, L));
   CKS(dalloc(&b.work, 4, L));
   CK(cudaMemsetAsync(b.work, 0, sizeof(uint32_t) * 4, s->ctx->stream));
-  const bool bins = s->b.bin_ctl != nullptr;
-  if (bins)
-    CKS(alloc_bins(b, s->dim, s->b.tile_edge, nt, L));
-  else
-    CKS(dalloc(&b.sorted, s->npad, L));
+  CKS(dalloc(&s->sorted2, s->npad, L));
+  use_bins(b, s->bins2, s->dim, b.tile_edge, nt, s->sorted2);
   CKS(dalloc(&b.partial, size_t(nt) * NB, L));
   CKS(dalloc(&b.partial_b, size_t(nt) * NB, L));
   b.scenes = s->cur2;
@@ -788,7 +790,6 @@ mpm_status ensure_ws2_parts(mpm_scene* s) {
 // first reverse pass that does; all or nothing).
 mpm_status ensure_set_b_parts(mpm_scene* s) {
   const int nt = s->hp.n_tiles;
-  const bool bins = s->b.bin_ctl != nullptr;
   std::vector<void*>& L = s->set_b_allocs;
   cudaStream_t st = s->ctx->stream;
   BatchDev& bb = s->bB;  // only its sort arrays and record are used
@@ -801,10 +802,7 @@ mpm_status ensure_set_b_parts(mpm_scene* s) {
   CKS(dalloc(&bb.tile_slot, nt, L));
   CKS(dalloc(&bb.active, nt, L));
   CKS(dalloc(&bb.n_active, 1, L));
-  if (bins)
-    CKS(alloc_bins(bb, s->dim, s->b.tile_edge, nt, L));
-  else
-    CKS(dalloc(&bb.sorted, s->npad, L));
+  if (!s->b.bin_ctl) CKS(dalloc(&bb.sorted, s->npad, L));  // else its lists are the set's bins
   bb.scenes = s->curB;
   CK(cudaMemsetAsync(s->actB, 0, sizeof(float) * std::max(1, s->G), st));
   for (cudaEvent_t& e : s->ev_load) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -852,6 +850,47 @@ void free_ws2(mpm_scene* s) {
 }  // namespace
 
 namespace gbmpm {
+
+namespace {
+// Words of a set's control block (rounded so that the lists start on a line) and of each list.
+size_t bin_ctl_room(int tiles) { return (bin_ctl_words(tiles) + 63) / 64 * 64; }
+size_t bin_list_room(int dim, int edge, int tiles) { return size_t(tiles) * bin_cap(dim, edge); }
+}  // namespace
+
+size_t bin_set_bytes(int dim, int edge, int tiles) {
+  return (bin_ctl_room(tiles) + 2 * bin_list_room(dim, edge, tiles)) * sizeof(uint32_t);
+}
+
+mpm_status take_bins(mpm_ctx* c, BinSet& set, size_t bytes) {
+  if (c->bin_bytes.fetch_add(bytes) + bytes > c->bin_limit) {
+    c->bin_bytes.fetch_sub(bytes);
+    return MPM_OK;
+  }
+  void* p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess) {
+    c->bin_bytes.fetch_sub(bytes);
+    if (e != cudaErrorMemoryAllocation) return MPM_ERR_CUDA;
+    cudaGetLastError();
+    return MPM_OK;
+  }
+  set.mem = static_cast<uint32_t*>(p);
+  set.bytes = bytes;
+  return MPM_OK;
+}
+
+void drop_bins(mpm_ctx* c, BinSet& set) {
+  if (!set.mem) return;
+  cudaFree(set.mem);
+  c->bin_bytes.fetch_sub(set.bytes);
+  set = BinSet();
+}
+
+void use_bins(BatchDev& b, const BinSet& set, int dim, int edge, int tiles, uint32_t* sorted) {
+  b.bin_ctl = set.mem;
+  b.bin_raw = set.mem ? set.mem + bin_ctl_room(tiles) : nullptr;
+  b.sorted = set.mem ? b.bin_raw + bin_list_room(dim, edge, tiles) : sorted;
+}
 
 mpm_status enqueue_step(mpm_scene* s, int ph, cudaStream_t st) { return enqueue_phase(s, ph, st); }
 
@@ -902,7 +941,9 @@ mpm_status rollout_records(mpm_scene* s, int T, int k, size_t budget, bool copy_
 // read the state, their inputs.
 size_t overlap_store_bytes(const mpm_scene* s, int k) {
   const size_t ctrl = ctrl_reads_state(s->ctrl) ? 2 * size_t(k) * CTRL_SLOT_FLOATS * sizeof(float) : 0;
-  if (s->b.bin_ctl) return ctrl;  // the reverse steps bin their states again
+  // with bins the reverse steps bin their states again; the bins they and the recompute take besides
+  // come from what the budget leaves (prepare_backward)
+  if (s->b.bin_ctl) return ctrl;
   return 2 * size_t(k) * sort_slot_words(s->npad, s->hp.n_tiles) * sizeof(uint32_t) + ctrl;
 }
 
@@ -1053,7 +1094,9 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
   const bool overlap = !mean_x0_seed && !(flags & BW_NO_OVERLAP) && s->impl == MPM_IMPL_TILED && k > 1 && nseg > 1 &&
                        (s->roll_budget == 0 ||
                         (size_t(nseg) + 2 * size_t(k - 1)) * S + store_bytes <= s->roll_budget);
-  bool branch = overlap || (!mean_x0_seed && !(flags & BW_NO_OVERLAP) && s->b.bin_ctl && k == 1);
+  const bool bins = s->b.bin_ctl != nullptr;
+  bool branch = s->ctrl_branch &&
+                (overlap || (!mean_x0_seed && !(flags & BW_NO_OVERLAP) && bins && k == 1));
   if (branch) {
     const mpm_status st_b = ensure_set_b(s);
     if (st_b == MPM_ERR_OOM && !overlap) {
@@ -1063,26 +1106,40 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
       CKS(st_b);
     }
   }
+  if (overlap) CKS(ensure_ws2(s));
+  // A scene with bins gives set B and workspace 2 bins of their own from what the budget leaves beside
+  // the states, while the context and the device have them.  Set B first: the reverse steps are the
+  // critical path.  Without them set B is not used (the states are binned in line), and the recompute
+  // sorts.  What a budget has no room or use for is given back.
+  size_t room = s->roll_budget == 0 ? SIZE_MAX
+                : overlap           ? s->roll_budget - ((size_t(nseg) + 2 * size_t(k - 1)) * S + store_bytes)
+                                    : s->roll_budget - std::min(s->roll_budget, (size_t(nseg) + size_t(k - 1)) * S);
+  if (bins && branch) {
+    CKS(further_bins(s, s->binsB, &room));
+    use_bins(s->bB, s->binsB, dim, s->b.tile_edge, s->hp.n_tiles, nullptr);
+    branch = s->bB.bin_ctl != nullptr;
+  } else if (s->roll_budget != 0) {
+    CKS(give_up_bins(s, s->binsB));
+  }
+  if (bins && overlap) {
+    CKS(further_bins(s, s->bins2, &room));
+    use_bins(s->b2, s->bins2, dim, s->b.tile_edge, s->hp.n_tiles, s->sorted2);
+  } else if (s->roll_budget != 0) {
+    CKS(give_up_bins(s, s->bins2));
+  }
   if (overlap) {
-    CKS(ensure_ws2(s));
     if (int(s->seg2.size()) != k - 1) {
       std::vector<float4*> segs(k - 1, nullptr);  // the scene keeps them only once all exist
       for (int i = 0; i < k - 1; ++i) CKS(dalloc(&segs[i], S / sizeof(float4), s->roll_allocs));
       s->seg2 = segs;
     }
     // the sorts of every recomputed state, by segment parity (each reverse step loads its own)
-    if (!s->sort_store && !s->b.bin_ctl)
+    if (!s->sort_store && !bins)
       CKS(dalloc(&s->sort_store, (store_bytes - ctrl_bytes) / sizeof(uint32_t), s->roll_allocs));
     if (keep_ctrl && !s->ctrl_store) CKS(dalloc(&s->ctrl_store, ctrl_bytes / sizeof(float), s->roll_allocs));
   }
-  // recompute and reverse graphs name the workspace and the way states are binned
   if (s->graphs_ws2 != overlap || s->graphs_branch != branch) {
-    for (int ph : {PH_RCM, PH_PREP, PH_REV})
-      for (auto& g : s->graphs[ph])
-        if (g.exec) {
-          cudaGraphExecDestroy(g.exec);
-          g = Graph();
-        }
+    drop_reverse_graphs(s);
     s->graphs_ws2 = overlap;
     s->graphs_branch = branch;
   }
@@ -1196,7 +1253,7 @@ mpm_status recompute_segment(mpm_scene* s, int sg, cudaStream_t st) {
   CK(launch_set_int(s->d_step, n0 + sg * k, st));
   CKS(run_phase(s, PH_PREP, 1, st));  // bin keys of the checkpoint the recompute starts from
   if (L > 1) CKS(run_phase(s, PH_RCM, L - 1, st));
-  if (s->rcm_ws2 && !s->b.bin_ctl) {
+  if (s->rcm_ws2 && s->sort_store) {
     // the segment's last state has its keys (from the last recompute step, or the checkpoint's
     // own for L = 1) but no scatter yet: sort it into its slot and leave the counters clear
     BatchDev& b2 = workspace(s, PH_RCM);
@@ -1409,6 +1466,10 @@ mpm_status ml_rollout(mpm_scene* s, int T, size_t budget) {
   if (c.cost >= ML_INF) return MPM_ERR_OOM;
   const int P = 2 + c.peak;
   free_rollout(s);  // the single-level buffers' memory belongs to the budget
+  for (BinSet* set : {&s->bins2, &s->binsB}) {  // and its passes, without overlap, use neither of these
+    const mpm_status st = give_up_bins(s, *set);
+    if (st != MPM_OK) return st;
+  }
   if (int(s->ml_pool.size()) != P) {
     free_ml_pool(s);
     s->ml_pool.assign(P, nullptr);
@@ -1549,6 +1610,19 @@ mpm_status mpm_ctx_destroy(mpm_ctx* c) {
   return MPM_OK;
 }
 
+mpm_status mpm_ctx_set_bin_bytes(mpm_ctx* c, size_t most) {
+  if (!c) return MPM_ERR_ARG;
+  c->bin_limit = most;
+  return MPM_OK;
+}
+
+mpm_status mpm_ctx_bin_bytes(const mpm_ctx* c, size_t* held, size_t* most) {
+  if (!c) return MPM_ERR_ARG;
+  if (held) *held = c->bin_bytes.load();
+  if (most) *most = c->bin_limit.load();
+  return MPM_OK;
+}
+
 mpm_status mpm_sync(mpm_ctx* c) {
   if (!c) return MPM_ERR_ARG;
   CK(cudaStreamSynchronize(c->stream));
@@ -1578,7 +1652,7 @@ mpm_status mpm_scene_destroy(mpm_scene* s) {
   for (cudaEvent_t e : s->ev_ctrl)
     if (e) cudaEventDestroy(e);
   if (s->ev_params) cudaEventDestroy(s->ev_params);
-  s->ctx->bin_bytes.fetch_sub(s->bin_bytes);
+  for (BinSet* set : {&s->bins, &s->bins2, &s->binsB}) drop_bins(s->ctx, *set);
   s->ctx->live.fetch_sub(1);
   delete s;
   return MPM_OK;
@@ -1758,20 +1832,11 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   ALLOC(b.n_active, 1);
   ALLOC(b.block_sums, 2 * ((p.n_tiles + 2047) / 2048) + 2);
   ALLOC(b.work, 4);
-  bool bins = s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES && reserve_bins(s, edge, p.n_tiles);
-  if (bins) {
-    st = alloc_bins(b, dim, edge, p.n_tiles, s->allocs);
-    if (st == MPM_ERR_OOM) {
-      cudaGetLastError();  // the failed allocation's error: the scene sorts instead
-      bins = false;
-    } else if (st != MPM_OK) {
-      return fail(st);
-    }
-  }
-  if (bins)
-    b.rec_flip = 1;
-  else
-    ALLOC(b.sorted, s->npad);
+  if (s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES)
+    TRY(take_bins(c, s->bins, bin_set_bytes(dim, edge, p.n_tiles)));
+  if (!s->bins.mem) ALLOC(b.sorted, s->npad);
+  use_bins(b, s->bins, dim, edge, p.n_tiles, b.sorted);
+  b.rec_flip = s->bins.mem ? 1 : 0;
   if (s->impl == MPM_IMPL_TILED) {
     ALLOC(b.partial, size_t(p.n_tiles) * NB);
     ALLOC(b.partial_b, size_t(p.n_tiles) * NB);

@@ -58,7 +58,9 @@ struct SubBatch {
   TuneState tune;
   long long key_particles = -1, key_tiles = -1;
   int trial_wait = 0;  // steps of this key left before its trials start (0: none pending)
-  uint32_t *bin_ctl = nullptr, *bin_raw = nullptr;  // tile bins, for compositions of at most BIN_TILES tiles
+  BinSet bins;        // tile bins, for compositions of at most bin_tiles tiles (none: they sort)
+  int bin_tiles = 0;
+  uint32_t* sorted = nullptr;
   float4 *partial = nullptr, *partial_b = nullptr;  // node blocks (each half its own: they run at once)
   int cap_edge = 0;  // tile edge the node-block arrays are sized for
 };
@@ -84,7 +86,7 @@ void dfree(T*& p) {
   p = nullptr;
 }
 
-void free_sub(SubBatch& sb) {
+void free_sub(mpm_ctx* ctx, SubBatch& sb) {
   batch_tune_release(sb.tune);
   sb.key_particles = sb.key_tiles = -1;
   dfree(sb.meta);
@@ -103,9 +105,9 @@ void free_sub(SubBatch& sb) {
   dfree(sb.b.n_active);
   dfree(sb.b.block_sums);
   dfree(sb.b.work);
-  dfree(sb.b.sorted);
-  dfree(sb.bin_ctl);
-  dfree(sb.bin_raw);
+  dfree(sb.sorted);
+  drop_bins(ctx, sb.bins);
+  sb.bin_tiles = 0;
   dfree(sb.b.gpartial);
   dfree(sb.partial);
   dfree(sb.partial_b);
@@ -144,7 +146,7 @@ mpm_status grow(mpm_batch* B, SubBatch& sb, int n_scenes, int tiles, int particl
   if (sc <= sb.cap_scenes && tl <= sb.cap_tiles && pc <= sb.cap_particles && sb.cap_edge == B->edge)
     return MPM_OK;
   CK(cudaStreamSynchronize(B->ctx->stream));
-  free_sub(sb);
+  free_sub(B->ctx, sb);
   auto round = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
   sb.off_ctrl = round(sizeof(SelectPar) * sc);
   sb.off_pbase = sb.off_ctrl + round(sizeof(CtrlPar) * sc);
@@ -169,11 +171,9 @@ mpm_status grow(mpm_batch* B, SubBatch& sb, int n_scenes, int tiles, int particl
   CK(cudaMalloc(&sb.b.block_sums, sizeof(uint32_t) * (2 * ((tl + 2047) / 2048) + 2)));
   CK(cudaMalloc(&sb.b.work, sizeof(uint32_t) * 4));
   CK(cudaMemsetAsync(sb.b.work, 0, sizeof(uint32_t) * 4, B->ctx->stream));
-  const int bt = std::min(tl, BIN_TILES);
-  const size_t room = size_t(bt) * bin_cap(B->dim, B->edge);
-  CK(cudaMalloc(&sb.bin_ctl, sizeof(uint32_t) * bin_ctl_words(bt)));
-  CK(cudaMalloc(&sb.bin_raw, sizeof(uint32_t) * room));
-  CK(cudaMalloc(&sb.b.sorted, sizeof(uint32_t) * std::max(size_t(pc), room)));
+  CK(cudaMalloc(&sb.sorted, sizeof(uint32_t) * pc));
+  CKS(take_bins(B->ctx, sb.bins, bin_set_bytes(B->dim, B->edge, std::min(tl, BIN_TILES))));
+  sb.bin_tiles = sb.bins.mem ? std::min(tl, BIN_TILES) : 0;
   CK(cudaMalloc(&sb.b.gpartial, sizeof(float) * size_t(tl) * MAX_GROUPS));
   CK(cudaMemsetAsync(sb.b.tile_count, 0, sizeof(uint32_t) * tl, B->ctx->stream));
   CK(cudaMemsetAsync(sb.b.tile_fill, 0, sizeof(uint32_t) * tl, B->ctx->stream));
@@ -234,8 +234,7 @@ mpm_status compose(mpm_batch* B, SubBatch& sb) {
     CK(cudaEventRecord(sb.copied[sb.turn], st));
     sb.turn ^= 1;
   }
-  sb.b.bin_ctl = tiles <= BIN_TILES ? sb.bin_ctl : nullptr;
-  sb.b.bin_raw = sb.bin_raw;
+  use_bins(sb.b, tiles <= sb.bin_tiles ? sb.bins : BinSet(), B->dim, B->edge, sb.bin_tiles, sb.sorted);
   sb.b.scenes = sb.cur;
   sb.b.tile_edge = B->edge;
   sb.b.n_scenes = int(sb.members.size());
@@ -500,8 +499,8 @@ mpm_status mpm_batch_destroy(mpm_batch* B) {
   cudaStreamSynchronize(B->ctx->aux);
   for (Slot& sl : B->slots)  // the scenes of unreleased slots are the caller's again
     if (sl.state != S_FREE && sl.s) sl.s->batch_refs -= 1;
-  free_sub(B->fwd);
-  free_sub(B->rev);
+  free_sub(B->ctx, B->fwd);
+  free_sub(B->ctx, B->rev);
   dfree(B->d_status);
   cudaEventDestroy(B->fork);
   cudaEventDestroy(B->join);

@@ -182,8 +182,10 @@ struct BatchDev {
 };
 
 constexpr int BIN_TILES = 4096;                 // most tiles a batch with bins holds
-// Most bytes the bins of a context's scenes take (128 scenes of 4096 3D tiles, 4096 of 256 2D tiles);
-// further scenes sort, with the same results, so that thousands of small scenes still fit the device.
+// Most bytes the bins of a context's scenes and batches take unless mpm_ctx_set_bin_bytes says otherwise
+// (127 sets of 4096 3D tiles, 4000 of 256 2D tiles), every set counted: a scene's, the two its reverse
+// pass may take besides, a batch's.  What gets none sorts, with the same results, so that thousands
+// of small scenes still fit the device.
 constexpr size_t BIN_BYTES = size_t(16) << 30;
 constexpr int BIN_WORDS = BIN_TILES / 32;       // words of a tile mask
 constexpr int BIN_MASK = 4;                     // first mask word in bin_ctl

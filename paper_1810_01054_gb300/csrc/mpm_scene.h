@@ -47,7 +47,14 @@ struct mpm_ctx {
   std::vector<int> prof_kind;
   int prof_used = 0;
   std::atomic<int> live{0};  // scenes and batches created on this context and not yet destroyed
-  std::atomic<size_t> bin_bytes{0};  // tile bins of its scenes, at most BIN_BYTES
+  std::atomic<size_t> bin_bytes{0};  // tile bins of its scenes and batches
+  std::atomic<size_t> bin_limit{gbmpm::BIN_BYTES};  // the most they may take
+};
+
+// One set of tile bins (control words, appended and canonical lists), counted against its context's bound.
+struct BinSet {
+  uint32_t* mem = nullptr;
+  size_t bytes = 0;
 };
 
 struct Graph {
@@ -139,7 +146,7 @@ struct mpm_scene {
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
   TuneState tune;
-  size_t bin_bytes = 0;     // of the context's, this scene's tile bins
+  BinSet bins, bins2, binsB;  // tile bins: the scene's, workspace 2's, set B's (mem NULL: has none)
   bool keys_stale = false;  // a batch advanced the state since its bin keys were made
   int batch_refs = 0;  // batch slots holding the scene (admitted, not yet released)
   // The segment recompute's own workspace (tile arrays, selected record, bin keys, actuation,
@@ -151,6 +158,7 @@ struct mpm_scene {
   uint32_t* key2 = nullptr;
   float* act2 = nullptr;
   float4* grid2 = nullptr;
+  uint32_t* sorted2 = nullptr;  // the recompute sorts into it without bins of its own
   std::vector<void*> ws2_allocs, set_b_allocs;
   std::vector<float4*> seg2;
   uint32_t* sort_store = nullptr;  // 2 x k slots (segment parity, state in segment) of sorts
@@ -187,6 +195,14 @@ struct mpm_scene {
 
 namespace gbmpm {
 // Helpers the batch scheduler shares with the single-scene entry points (mpm_api.cu).
+// Tile bins of a batch of `tiles` tiles (at most BIN_TILES): the bytes of a set; a set taken from the
+// context's bound and the device (set.mem stays NULL, with MPM_OK, when either has no room: the
+// caller sorts instead); a set given back; and the pointers of b over the set, or over `sorted`
+// without one.
+size_t bin_set_bytes(int dim, int edge, int tiles);
+mpm_status take_bins(mpm_ctx* c, BinSet& set, size_t bytes);
+void drop_bins(mpm_ctx* c, BinSet& set);
+void use_bins(BatchDev& b, const BinSet& set, int dim, int edge, int tiles, uint32_t* sorted);
 mpm_status prepare_rollout(mpm_scene* s, int T, int k, size_t budget);
 // flags of prepare_backward used by the multi-level store for its later ranges
 enum BackwardFlags {

@@ -133,6 +133,8 @@ _lock = threading.Lock()
 _SIGS = {
     "mpm_ctx_create": [C.POINTER(C.c_void_p), C.c_int, C.c_void_p],
     "mpm_ctx_destroy": [C.c_void_p],
+    "mpm_ctx_set_bin_bytes": [C.c_void_p, C.c_size_t],
+    "mpm_ctx_bin_bytes": [C.c_void_p, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t)],
     "mpm_sync": [C.c_void_p],
     "mpm_status_str": [C.c_int],
     "mpm_scene_create": [C.c_void_p, C.POINTER(SceneDesc), C.POINTER(C.c_void_p)],
@@ -305,6 +307,16 @@ class Context:
 
     def sync(self):
         _check(lib().mpm_sync(self.handle), "mpm_sync")
+
+    def set_bin_bytes(self, most: int):
+        """Most device bytes the tile bins of the context's scenes and batches take together."""
+        _check(lib().mpm_ctx_set_bin_bytes(self.handle, int(most)), "mpm_ctx_set_bin_bytes")
+
+    def bin_bytes(self):
+        """(bytes of tile bins held now, the most they may take)."""
+        held, most = C.c_size_t(), C.c_size_t()
+        _check(lib().mpm_ctx_bin_bytes(self.handle, C.byref(held), C.byref(most)), "mpm_ctx_bin_bytes")
+        return int(held.value), int(most.value)
 
     def profile_start(self, kinds, max_launches: int = 1 << 16):
         mask = 0
