@@ -41,8 +41,7 @@ namespace {
 
 mpm_status cuda_fail(cudaError_t e) {
   if (e == cudaSuccess) return MPM_OK;
-  if (e == cudaErrorMemoryAllocation) return MPM_ERR_OOM;
-  return MPM_ERR_CUDA;
+  return out_of_memory(e) ? MPM_ERR_OOM : MPM_ERR_CUDA;
 }
 
 #define CK(expr)                                 \
@@ -870,9 +869,7 @@ mpm_status take_bins(mpm_ctx* c, BinSet& set, size_t bytes) {
   const cudaError_t e = cudaMalloc(&p, bytes);
   if (e != cudaSuccess) {
     c->bin_bytes.fetch_sub(bytes);
-    if (e != cudaErrorMemoryAllocation) return MPM_ERR_CUDA;
-    cudaGetLastError();
-    return MPM_OK;
+    return out_of_memory(e) ? MPM_OK : MPM_ERR_CUDA;
   }
   set.mem = static_cast<uint32_t*>(p);
   set.bytes = bytes;
@@ -1099,12 +1096,10 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
                 (overlap || (!mean_x0_seed && !(flags & BW_NO_OVERLAP) && bins && k == 1));
   if (branch) {
     const mpm_status st_b = ensure_set_b(s);
-    if (st_b == MPM_ERR_OOM && !overlap) {
-      cudaGetLastError();  // the failed allocation's error: the states are binned in line instead
-      branch = false;
-    } else {
+    if (st_b == MPM_ERR_OOM && !overlap)
+      branch = false;  // the states are binned in line instead
+    else
       CKS(st_b);
-    }
   }
   if (overlap) CKS(ensure_ws2(s));
   // A scene with bins gives set B and workspace 2 bins of their own from what the budget leaves beside

@@ -72,7 +72,7 @@ constexpr int kTrialWait = 32;
 #define CK(expr)                                                                   \
   do {                                                                             \
     cudaError_t e_ = (expr);                                                       \
-    if (e_ != cudaSuccess) return e_ == cudaErrorMemoryAllocation ? MPM_ERR_OOM : MPM_ERR_CUDA; \
+    if (e_ != cudaSuccess) return out_of_memory(e_) ? MPM_ERR_OOM : MPM_ERR_CUDA;       \
   } while (0)
 #define CKS(expr)                \
   do {                           \
@@ -535,8 +535,7 @@ mpm_status mpm_batch_admit(mpm_batch* B, mpm_scene* s, int n_steps, int want_gra
   }
   mpm_status st = prepare_rollout(s, n_steps, k, 0);
   if (st == MPM_ERR_OOM && k != sqrt_interval(n_steps)) {
-    cudaGetLastError();  // the failed allocation's error: the smaller store is tried instead
-    k = sqrt_interval(n_steps);
+    k = sqrt_interval(n_steps);  // the smaller store
     st = prepare_rollout(s, n_steps, k, 0);
   }
   if (st != MPM_OK) return st;

@@ -573,7 +573,7 @@ namespace {
 
 mpm_status cuda_status(cudaError_t e) {
   if (e == cudaSuccess) return MPM_OK;
-  return e == cudaErrorMemoryAllocation ? MPM_ERR_OOM : MPM_ERR_CUDA;
+  return gbmpm::out_of_memory(e) ? MPM_ERR_OOM : MPM_ERR_CUDA;
 }
 
 #define CK64(expr)                                    \

@@ -41,6 +41,14 @@ cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
   return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 
+// True for a failed allocation, whose error is then cleared: the call answers MPM_ERR_OOM once, and the
+// next one is not taken to have failed by the error left pending.
+inline bool out_of_memory(cudaError_t e) {
+  if (e != cudaErrorMemoryAllocation) return false;
+  cudaGetLastError();
+  return true;
+}
+
 constexpr uint32_t KEY_INVALID = 0xffffffffu;
 constexpr int MAX_GROUPS = 64;  // actuation groups per scene
 constexpr int MAX_HIDDEN = 128; // controller MLP width

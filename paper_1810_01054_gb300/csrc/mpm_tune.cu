@@ -20,7 +20,7 @@
 #define CK(expr)                                                                               \
   do {                                                                                         \
     cudaError_t e_ = (expr);                                                                   \
-    if (e_ != cudaSuccess) return e_ == cudaErrorMemoryAllocation ? MPM_ERR_OOM : MPM_ERR_CUDA; \
+    if (e_ != cudaSuccess) return out_of_memory(e_) ? MPM_ERR_OOM : MPM_ERR_CUDA;                   \
   } while (0)
 #define CKS(expr)                \
   do {                           \

@@ -151,3 +151,27 @@ def test_bins_the_device_cannot_hold_are_not_counted(M, ctx):
     finally:
         del fill
         torch.cuda.empty_cache()
+
+
+def test_out_of_memory_is_answered_once(M, ctx):
+    """A call that found no device memory leaves no error behind for the next one."""
+    import torch
+    spec = _spec()
+    sc = M.Scene(ctx, spec)
+    sc.step(2)
+    sc.get_state()
+    T = 64 * MB // sc.info()["state_bytes"]
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - 16 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(M.MPMError) as e:
+            sc.rollout(T, 1)  # 64 MB of states
+        assert e.value.status == -2
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    want = _pass(sc, spec, 6, 2)
+    other = M.Scene(ctx, spec)
+    _same(_pass(other, spec, 6, 2), want)
+    other.close()
+    sc.close()
