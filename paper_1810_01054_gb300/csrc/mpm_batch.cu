@@ -177,11 +177,11 @@ mpm_status grow(mpm_batch* B, SubBatch& sb, int n_scenes, int tiles, int particl
   CK(cudaMalloc(&sb.b.gpartial, sizeof(float) * size_t(tl) * MAX_GROUPS));
   CK(cudaMemsetAsync(sb.b.tile_count, 0, sizeof(uint32_t) * tl, B->ctx->stream));
   CK(cudaMemsetAsync(sb.b.tile_fill, 0, sizeof(uint32_t) * tl, B->ctx->stream));
-  sb.cap_scenes = sc;
-  sb.cap_tiles = tl;
-  sb.cap_particles = pc;
   CK(cudaMalloc(&sb.partial, sizeof(float4) * size_t(tl) * block_nodes(B->dim, B->edge)));
   CK(cudaMalloc(&sb.partial_b, sizeof(float4) * size_t(tl) * block_nodes(B->dim, B->edge)));
+  sb.cap_scenes = sc;  // only now: after a failed allocation the next call starts over
+  sb.cap_tiles = tl;
+  sb.cap_particles = pc;
   sb.cap_edge = B->edge;
   return MPM_OK;
 }

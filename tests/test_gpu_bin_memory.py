@@ -175,3 +175,35 @@ def test_out_of_memory_is_answered_once(M, ctx):
     _same(_pass(other, spec, 6, 2), want)
     other.close()
     sc.close()
+
+
+def test_a_batch_that_ran_out_of_memory_goes_on_when_there_is_some(M, ctx):
+    """A composition that does not fit is answered with MPM_ERR_OOM; the same call later allocates anew."""
+    import torch
+    spec = _spec()
+    ctx.set_bin_bytes(0)
+    scenes = [M.Scene(ctx, spec) for _ in range(3)]
+    batch = M.Batch(ctx, 3)
+    slot = batch.admit(scenes[0], 5, False)  # the batch's arrays are sized for one scene
+    while not batch.poll(slot):
+        batch.tick(5)
+    want = list(scenes[0].get_state())
+    batch.release(slot)
+    slots = [batch.admit(sc, 5, False) for sc in scenes[1:]]
+    torch.cuda.empty_cache()
+    # two scenes' node blocks are 28 MB twice, one scene's (given back first) 14 MB twice
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - 16 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(M.MPMError) as e:
+            batch.tick(5)
+        assert e.value.status == -2
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    while not all(batch.poll(sl) for sl in slots):
+        batch.tick(5)
+    for sc in scenes[1:]:
+        _same(list(sc.get_state()), want)
+    batch.close()
+    for sc in scenes:
+        sc.close()
