@@ -391,6 +391,10 @@ __device__ __forceinline__ void block_scan2(uint32_t& a, uint32_t& c, uint32_t& 
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_PER_THREAD = 2;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_PER_THREAD;
+// Small batches scan the tile histogram inside the scatter (k_scatter<D, true>): one sort launch a step
+// instead of three.  The P2G that follows every scatter clears the counters.
+__host__ __device__ __forceinline__ bool fused_scan(const BatchDev& b) { return b.total_tiles <= SCAN_TILE; }
+
 // Phase 1 of the tile scan: per-block totals of particle counts and of active tiles.
 template <bool SEL>
 __global__ void k_scan_reduce(BatchDev b, const SelectPar* __restrict__ sel) {
@@ -477,20 +481,73 @@ __global__ void k_scan_down(BatchDev b) {
   }
 }
 
-// Scatter of the particles into their tiles' ranges of `sorted`.
-template <int D>
-__global__ void __launch_bounds__(256) k_scatter(BatchDev b) {
+// Scatter of the particles into their tiles' ranges of `sorted`.  With FUSED (total_tiles <=
+// SCAN_TILE) the tile scan is done here instead of by the scan kernels: every CTA scans the whole
+// histogram in shared memory (it is small), CTA 0 publishes tile_start, tile_slot, the active list
+// and n_active; the P2G that follows clears the per-step counters.
+// With SEL (a single scene, fused scan) one extra CTA, launched after the scatter's own, makes the
+// step's selection (see k_keys) alongside them; the scatter reads only the record's step-invariant
+// fields (keys, offsets, status), which it takes from the phase's first record instead of the
+// one being published.
+template <int D, bool FUSED, bool SEL>
+__global__ void __launch_bounds__(256) k_scatter(BatchDev b, const SelectPar* __restrict__ sel) {
   pdl_enter();
+  if (SEL && blockIdx.x == gridDim.x - 1) {
+    select_publish(*sel, b.scenes);
+    return;
+  }
+  constexpr int PER = FUSED ? SCAN_TILE / 256 : 1;
+  __shared__ uint32_t sstart[FUSED ? SCAN_TILE + 1 : 1];
+  if constexpr (FUSED) {
+    const int nt = b.total_tiles, t0 = threadIdx.x * PER;
+    uint32_t cnt[PER], s = 0, c = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      cnt[i] = t0 + i < nt ? b.tile_count[t0 + i] : 0u;
+      s += cnt[i];
+      c += cnt[i] > 0;
+    }
+    uint32_t ts, tc;
+    block_scan2(s, c, ts, tc);
+    const bool pub = blockIdx.x == 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int t = t0 + i;
+      if (t < nt) {
+        sstart[t] = s;
+        if (pub) {
+          b.tile_start[t] = s;
+          if (cnt[i] > 0) {
+            b.tile_slot[t] = int(c);
+            b.active[c] = t;
+          } else {
+            b.tile_slot[t] = -1;
+          }
+        }
+        s += cnt[i];
+        c += cnt[i] > 0;
+      }
+    }
+    if (threadIdx.x == 0) {
+      sstart[nt] = ts;
+      if (pub) {
+        b.tile_start[nt] = ts;
+        *b.n_active = int(tc);
+      }
+    }
+    __syncthreads();
+  }
   int gp = blockIdx.x * blockDim.x + threadIdx.x;
   if (gp >= b.total_particles) return;
-  const ScenePar& sp = b.scenes[find_scene(b.scene_pbase, b.n_scenes, gp)];
-  int p = gp - sp.pbase;
+  const ScenePar& sp = SEL ? sel->table[0] : b.scenes[find_scene(b.scene_pbase, b.n_scenes, gp)];
+  const int pbase = SEL ? sel->pbase : sp.pbase, tbase = SEL ? sel->tile_base : sp.tile_base;
+  int p = gp - pbase;
   const uint32_t k = sp.key[p];
-  const int t = k != KEY_INVALID ? int(sp.tile_base + (k >> 6)) : -1;
+  const int t = k != KEY_INVALID ? int(tbase + (k >> 6)) : -1;
   const uint32_t rank = warp_aggregated_inc(b.tile_fill, t);
   if (t < 0) return;
-  const uint32_t start = b.tile_start[t];
-  const uint32_t end = b.tile_start[t + 1];
+  const uint32_t start = FUSED ? sstart[t] : b.tile_start[t];
+  const uint32_t end = FUSED ? sstart[t + 1] : b.tile_start[t + 1];
   if (start + rank >= end) {  // a key the histogram did not count: record it, write nothing
     set_status(sp.status, ST_BINNING);
     return;
@@ -708,7 +765,9 @@ __global__ void __launch_bounds__(T, T > 256 ? 1 : T == 256 ? (D == 3 && !ADJ ? 
     if (b.total_tiles > 0) first_gt = b.active[int(blockIdx.x) < b.total_tiles ? blockIdx.x : 0];
     n_active = *b.n_active;
     stage_scene<D, true>(b.scenes, sh);
-    // the scatter's counts are cleared here: every step starts from zero
+    // the per-step counters are cleared here whichever scan ran (the fused one leaves them set, the
+    // separate one leaves the scatter's fill counts): every step then starts from zero, also when a
+    // batch's composition moves it between the two scans
     for (int i = blockIdx.x * blockDim.x + tid; i < b.total_tiles; i += gridDim.x * blockDim.x) {
       b.tile_count[i] = 0u;
       b.tile_fill[i] = 0u;
@@ -2159,13 +2218,24 @@ cudaError_t launch_keys(const BatchDev& b, cudaStream_t s, const SelectPar* sel,
 template <int D>
 cudaError_t launch_sort(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
   if (b.bin_ctl) return cudaSuccess;  // the particles are in their tiles' lists already
+  if (fused_scan(b)) {  // scan inside the scatter; at least one CTA so the scan results are written
+    const int nblk = b.total_particles > 0 ? (b.total_particles + 255) / 256 : 1;
+    if (sel)
+      launch_pdl(k_scatter<D, true, true>, dim3(nblk + 1), dim3(256), 0, s, b, sel);
+    else
+      launch_pdl(k_scatter<D, true, false>, dim3(nblk), dim3(256), 0, s, b, sel);
+    count_launches(1);
+    return cudaGetLastError();
+  }
   const int nblk = (b.total_tiles + SCAN_TILE - 1) / SCAN_TILE;
   if (sel)
     launch_pdl(k_scan_reduce<true>, dim3(nblk + 1), dim3(SCAN_THREADS), 0, s, b, sel);
   else
     launch_pdl(k_scan_reduce<false>, dim3(nblk), dim3(SCAN_THREADS), 0, s, b, sel);
   launch_pdl(k_scan_down, dim3(nblk), dim3(SCAN_THREADS), 0, s, b);
-  if (b.total_particles > 0) launch_pdl(k_scatter<D>, dim3((b.total_particles + 255) / 256), dim3(256), 0, s, b);
+  if (b.total_particles > 0)
+    launch_pdl(k_scatter<D, false, false>, dim3((b.total_particles + 255) / 256), dim3(256), 0, s, b,
+               static_cast<const SelectPar*>(nullptr));
   count_launches((b.total_particles > 0 ? 1 : 0) + 2);
   return cudaGetLastError();
 }
