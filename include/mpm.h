@@ -364,7 +364,8 @@ enum { MPM_TK_P2G = 0, MPM_TK_G2P = 1, MPM_TK_P2G_ADJ = 2, MPM_TK_ADJ_GATHER = 3
 mpm_status mpm_scene_set_tuning(mpm_scene* scene, int mode);
 /* Launch shape of tile kernel `kernel` for this scene; *tuned = 1 once it came from the cache or
  * from trials, 0 while it is the default or still being tried.  A 3D launch over at most one tile per
- * SM (the adjoint gather: two) runs wider CTAs instead, one (two) per SM. */
+ * SM (the adjoint gather: two) runs wider CTAs instead, one (two) per SM: *tuned = 1, and the shape
+ * given is not used, until a synchronising call has seen the scene's particles in more tiles. */
 mpm_status mpm_scene_launch(const mpm_scene* scene, int kernel, int* ctas_per_sm, int* threads, int* tuned);
 /* The process-wide cache.  shape[2k], shape[2k+1] = CTAs per SM and threads of tile kernel k.
  *  mpm_tune_cache_lookup  *found = 1 and shape filled when the key of (dim, particles, grid

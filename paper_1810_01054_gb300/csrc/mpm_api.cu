@@ -386,6 +386,7 @@ ScenePar rec_rev(const mpm_scene* s, float4* st, const float4* ain, float4* aout
 BatchDev& workspace(mpm_scene* s, int ph) {
   if ((ph == PH_RCM || ph == PH_PREP) && s->rcm_ws2) {
     for (int k = 0; k < TK_COUNT; ++k) s->b2.launch[k] = s->b.launch[k];
+    s->b2.occupied = s->b.occupied;
     return s->b2;
   }
   return s->b;
@@ -922,10 +923,18 @@ mpm_status set_counter(mpm_scene* s, int* dctr, int value) {
 }
 
 mpm_status read_status(mpm_scene* s) {
-  int v = 0;
+  int v[2] = {0, 0};
   CK(cudaStreamSynchronize(s->ctx->stream));
-  CK(cudaMemcpy(&v, s->d_status, sizeof(int), cudaMemcpyDeviceToHost));
-  return mpm_status(v);
+  CK(cudaMemcpy(v, s->d_status, sizeof(v), cudaMemcpyDeviceToHost));
+  if (v[1] > s->b.occupied) {  // the body spread, or set_state spread it: its CTA sizes follow
+    const bool few[2] = {few_tiles(s->dim, s->b, 1), few_tiles(s->dim, s->b, 2)};
+    s->b.occupied = v[1];
+    if (few[0] != few_tiles(s->dim, s->b, 1) || few[1] != few_tiles(s->dim, s->b, 2)) {
+      invalidate_graphs(s);
+      CKS(tune_unfix(s));
+    }
+  }
+  return mpm_status(v[0]);
 }
 
 
@@ -1768,7 +1777,7 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   ALLOC(sig, s->npad);
   ALLOC(s->d_step, 1);
   ALLOC(s->d_bstep, 1);
-  ALLOC(s->d_status, 1);
+  ALLOC(s->d_status, 2);
   ALLOC(s->cur, 2);
   ALLOC(s->dsel, SEL_COUNT);
   p.planes = p.planes_out = s->state;
@@ -1824,7 +1833,7 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   ALLOC(b.tile_start, p.n_tiles + 1);
   ALLOC(b.tile_slot, p.n_tiles);
   ALLOC(b.active, p.n_tiles);
-  ALLOC(b.n_active, 1);
+  b.n_active = s->d_status + 1;
   ALLOC(b.block_sums, 2 * ((p.n_tiles + 2047) / 2048) + 2);
   ALLOC(b.work, 4);
   if (s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES)
@@ -1858,7 +1867,7 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   TRY(cuda_fail(cudaMemsetAsync(b.tile_fill, 0, sizeof(uint32_t) * p.n_tiles, stream)));
   TRY(cuda_fail(cudaMemsetAsync(b.work, 0, sizeof(uint32_t) * 4, stream)));
   TRY(cuda_fail(cudaMemsetAsync(tile_scene, 0, sizeof(int) * p.n_tiles, stream)));
-  TRY(cuda_fail(cudaMemsetAsync(s->d_status, 0, sizeof(int), stream)));
+  TRY(cuda_fail(cudaMemsetAsync(s->d_status, 0, 2 * sizeof(int), stream)));
   TRY(cuda_fail(cudaMemsetAsync(s->d_step, 0, sizeof(int), stream)));
   TRY(cuda_fail(cudaMemsetAsync(s->d_bstep, 0, sizeof(int), stream)));
   TRY(cuda_fail(cudaMemsetAsync(grid, 0, sizeof(float4) * s->n_nodes, stream)));

@@ -31,6 +31,7 @@ struct Slot {
   mpm_scene* s = nullptr;
   int state = S_FREE;
   int T = 0, want_grad = 0, done_steps = 0, seg = 0, left = 0;
+  int tiles = 0;  // most tiles its particles were seen in (a share of the composition's)
   size_t mem = 0, kept = 0;  // checkpoint bytes charged to the budget; bytes of a request that keeps every state
   mpm_status status = MPM_OK;
 };
@@ -57,9 +58,15 @@ struct SubBatch {
   // launch shapes: the cache entry of the composition's key, else trials during its steps
   TuneState tune;
   long long key_particles = -1, key_tiles = -1;
+  unsigned key_kernels = 0;  // kernels of the key whose launch shapes are tuned
   int trial_wait = 0;  // steps of this key left before its trials start (0: none pending)
   BinSet bins;        // tile bins, for compositions of at most bin_tiles tiles (none: they sort)
   int bin_tiles = 0;
+  // 3D compositions of few tiles: the active tiles of the last step of a tick, copied to `seen` (pinned)
+  // without waiting and looked at by a later tick if the composition is still the same
+  long long composed = 0, seen_composed = -1;  // compositions so far; the one `seen` is of (-1: none)
+  int* seen = nullptr;
+  cudaEvent_t seen_at = nullptr;
   uint32_t* sorted = nullptr;
   float4 *partial = nullptr, *partial_b = nullptr;  // node blocks (each half its own: they run at once)
   int cap_edge = 0;  // tile edge the node-block arrays are sized for
@@ -96,6 +103,11 @@ void free_sub(mpm_ctx* ctx, SubBatch& sb) {
     if (sb.copied[i]) cudaEventDestroy(sb.copied[i]);
     sb.copied[i] = nullptr;
   }
+  if (sb.seen) cudaFreeHost(sb.seen);
+  if (sb.seen_at) cudaEventDestroy(sb.seen_at);
+  sb.seen = nullptr;
+  sb.seen_at = nullptr;
+  sb.seen_composed = -1;
   dfree(sb.cur);
   dfree(sb.b.tile_count);
   dfree(sb.b.tile_fill);
@@ -241,27 +253,62 @@ mpm_status compose(mpm_batch* B, SubBatch& sb) {
   sb.b.scene_pbase = sb.pbase;
   sb.b.total_particles = particles;
   sb.b.total_tiles = tiles;
-  // a new workload key takes its shapes anew; an empty composition keeps the last key's shapes
-  // and trials (a lockstep batch alternates each half between its members and nothing)
-  if (!sb.members.empty() && (particles != sb.key_particles || tiles != sb.key_tiles)) {
-    default_launch(sb.b, B->ctx->sm_count);
-    CKS(batch_tune_init(sb.tune, sb.b, B->dim, 0u));  // cached shapes, no trials yet
-    sb.trial_wait = batch_tune_cached(sb.b, B->dim, half_kernels(B, sb)) ? 0 : kTrialWait;
-    sb.key_particles = particles;
-    sb.key_tiles = tiles;
-  }
   sb.b.has_material = sb.b.occupied = 0;
   for (int m : sb.members) {
     sb.b.has_material |= B->slots[m].s->hp.gmat ? 1 : 0;
-    sb.b.occupied += B->slots[m].s->b.occupied;
+    sb.b.occupied += B->slots[m].tiles;
+  }
+  sb.composed += 1;
+  sb.b.sm_count = B->ctx->sm_count;
+  // a new workload key takes its shapes anew; an empty composition keeps the last key's shapes
+  // and trials (a lockstep batch alternates each half between its members and nothing)
+  const unsigned kernels = tunable(B->dim, sb.b, half_kernels(B, sb));
+  if (!sb.members.empty() && (particles != sb.key_particles || tiles != sb.key_tiles || kernels != sb.key_kernels)) {
+    default_launch(sb.b, B->ctx->sm_count);
+    CKS(batch_tune_init(sb.tune, sb.b, B->dim, 0u));  // cached shapes, no trials yet
+    sb.trial_wait = (kernels == 0 || batch_tune_cached(sb.b, B->dim, kernels)) ? 0 : kTrialWait;
+    sb.key_particles = particles;
+    sb.key_tiles = tiles;
+    sb.key_kernels = kernels;
   }
   sb.need_keys = true;
   return MPM_OK;
 }
 
+// Asks for the active tiles of the half's last step, while they decide its CTA sizes.
+mpm_status ask_tiles(mpm_batch* B, SubBatch& sb) {
+  if (B->dim != 3 || sb.members.empty() || sb.seen_composed >= 0 || !few_tiles(3, sb.b, 2)) return MPM_OK;
+  if (!sb.seen) {
+    CK(cudaMallocHost(&sb.seen, sizeof(int)));
+    CK(cudaEventCreateWithFlags(&sb.seen_at, cudaEventDisableTiming));
+  }
+  CK(cudaMemcpyAsync(sb.seen, sb.b.n_active, sizeof(int), cudaMemcpyDeviceToHost, B->ctx->stream));
+  CK(cudaEventRecord(sb.seen_at, B->ctx->stream));
+  sb.seen_composed = sb.composed;
+  return MPM_OK;
+}
+
+// Looks at them, if they have arrived: a body that spread over more tiles leaves the wide CTAs.  Its
+// composition's tiles are known only together, so its scenes' shares grow alike.
+void look_at_tiles(mpm_batch* B, SubBatch& sb) {
+  if (sb.seen_composed < 0) return;
+  if (cudaEventQuery(sb.seen_at) != cudaSuccess) {
+    cudaGetLastError();  // not ready is no failure
+    return;
+  }
+  const bool same = sb.seen_composed == sb.composed;
+  sb.seen_composed = -1;
+  if (!same || *sb.seen <= sb.b.occupied) return;
+  for (int m : sb.members) {
+    int& o = B->slots[m].tiles;
+    o = int((long long)(o) * *sb.seen / sb.b.occupied) + 1;
+  }
+  B->dirty = true;
+}
+
 // Counts a step of the half's key; its trials start once the key has run kTrialWait steps.
 mpm_status trial_clock(mpm_batch* B, SubBatch& sb) {
-  if (sb.trial_wait > 0 && --sb.trial_wait == 0) CKS(batch_tune_init(sb.tune, sb.b, B->dim, half_kernels(B, sb)));
+  if (sb.trial_wait > 0 && --sb.trial_wait == 0) CKS(batch_tune_init(sb.tune, sb.b, B->dim, sb.key_kernels));
   return MPM_OK;
 }
 
@@ -546,6 +593,7 @@ mpm_status mpm_batch_admit(mpm_batch* B, mpm_scene* s, int n_steps, int want_gra
   sl.state = S_FWD;
   sl.T = n_steps;
   sl.want_grad = want_grad;
+  sl.tiles = s->b.occupied;
   sl.mem = request_bytes(s, n_steps, k);
   sl.kept = k == 1 && n_steps > 16 ? sl.mem : 0;
   B->used += sl.mem;
@@ -558,6 +606,8 @@ mpm_status mpm_batch_admit(mpm_batch* B, mpm_scene* s, int n_steps, int want_gra
 
 mpm_status mpm_batch_tick(mpm_batch* B, int max_steps) {
   if (!B || max_steps < 1) return MPM_ERR_ARG;
+  look_at_tiles(B, B->fwd);
+  look_at_tiles(B, B->rev);
   for (int it = 0; it < max_steps; ++it) {
     bool busy = false;
     for (const Slot& sl : B->slots) busy = busy || sl.state == S_FWD || sl.state == S_RCM || sl.state == S_REV;
@@ -579,6 +629,8 @@ mpm_status mpm_batch_tick(mpm_batch* B, int max_steps) {
     CK(cudaStreamWaitEvent(ms, B->join, 0));
     CKS(advance(B));
   }
+  CKS(ask_tiles(B, B->fwd));
+  CKS(ask_tiles(B, B->rev));
   CKS(finish_requests(B));
   CK(cudaGetLastError());
   return MPM_OK;

@@ -178,7 +178,7 @@ struct BatchDev {
   float4* partial_b;    // [total_tiles * BLOCK_NODES] node blocks of the adjoint scatter
   float* gpartial;      // [total_tiles * MAX_GROUPS] per active tile group sums of dL/da
   int tile_edge;                // cells per tile edge of every scene in the batch (0 or 4; 8: 2D)
-  int occupied;                 // tiles that held particles when the scenes were created (3D CTA sizes)
+  int occupied;                 // most tiles seen to hold particles: at creation, at a sync (3D CTA sizes)
   int has_material;             // some scene has per-particle material (gmat): material gradients
   int sm_count;                 // SMs of the device
   TileLaunch launch[TK_COUNT];  // launch shape of each tile kernel
@@ -202,6 +202,18 @@ inline size_t bin_ctl_words(int tiles) { return BIN_COUNT + 2 * size_t(tiles); }
 // Most entries of a tile's list: what its kernels stage (Tile<D, TB>::SORT_CAP).
 inline int bin_cap(int dim, int edge) { return dim == 2 && edge != 8 ? Tile<2, 4>::SORT_CAP : Tile<2, 8>::SORT_CAP; }
 static_assert(Tile<2, 8>::SORT_CAP == Tile<3, 4>::SORT_CAP, "bin_cap");
+
+// 3D scenes of few tiles: at most `per_sm` tiles per SM, where one resident wide CTA per SM holds them all
+// (every CTA size gives the same bits).  A 7,919-particle body, closed-loop controller, 24 steps with
+// the reverse pass: 2456 us with the large scenes' CTAs, 2261 with these; but 24 steps of 8,000
+// particles in 684 tiles take 901 us with the wide CTAs and 518 without, in 1,640 tiles 1761 and
+// 832.  So a scene leaves the class when more tiles are seen, and does not come back: a body that
+// comes and goes keeps the shapes that suit many tiles.
+inline bool few_tiles(int dim, const BatchDev& b, int per_sm) {
+  return dim == 3 && b.occupied > 0 && b.occupied <= per_sm * b.sm_count;
+}
+// Whether tile kernel k of b runs those CTAs, whatever its launch shape (which is not tuned then).
+inline bool shape_fixed(int dim, const BatchDev& b, int k) { return few_tiles(dim, b, k == TK_ADJ_GATHER ? 2 : 1); }
 
 // Sets every tile kernel of b to the default launch shape.
 inline void default_launch(BatchDev& b, int sm_count) {

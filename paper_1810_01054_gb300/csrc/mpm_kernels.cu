@@ -2279,18 +2279,10 @@ static int tile_grid(const BatchDev& b, int k) {
   return grid < 1 ? 1 : grid;
 }
 
-// 3D scenes of few tiles (counted at creation; every CTA size gives the same bits): at most `per_sm`
-// tiles per SM, where one resident wide CTA per SM holds them all.  A 7,919-particle body, closed-loop
-// controller, 24 steps with the reverse pass: 2456 us with the large scenes' CTAs, 2261 with these.
-template <int D>
-static bool few_tiles(const BatchDev& b, int per_sm) {
-  return D == 3 && b.occupied > 0 && b.occupied <= per_sm * b.sm_count;
-}
-
 template <int D, int TB, bool ADJ, bool BINS>
 static cudaError_t p2g_lists(const BatchDev& b, cudaStream_t s) {
   if constexpr (D == 3)
-    if (few_tiles<D>(b, 1)) {
+    if (few_tiles(D, b, 1)) {
       launch_pdl(k_p2g<D, TB, ADJ, 576, BINS>, dim3(std::min(b.total_tiles, b.sm_count)), dim3(576),
                  P2GCfg<D, TB, ADJ, 576>::SMEM, s, b);
       count_launches(1);
@@ -2323,7 +2315,7 @@ cudaError_t launch_p2g(const BatchDev& b, bool with_adjoint, cudaStream_t s) {
 template <int D, int TB, bool BINS>
 static cudaError_t g2p_lists(const BatchDev& b, cudaStream_t s, const SelectPar* sel) {
   if constexpr (D == 3)
-    if (few_tiles<D>(b, 1)) {
+    if (few_tiles(D, b, 1)) {
       launch_pdl(k_g2p<D, TB, 512, BINS>, dim3(std::min(b.total_tiles, b.sm_count) + (sel ? 1 : 0)), dim3(512), 0, s, b,
                  sel);
       count_launches(1);
@@ -2361,9 +2353,9 @@ static cudaError_t adj_gather_threads(const BatchDev& b, int grid, cudaStream_t 
 template <int D, int TB, bool BINS>
 static cudaError_t adj_gather_lists(const BatchDev& b, cudaStream_t s) {
   if constexpr (D == 3) {
-    if (few_tiles<D>(b, 1))
+    if (few_tiles(D, b, 1))
       return adj_gather_threads<D, TB, BINS, 512>(b, std::min(b.total_tiles, b.sm_count), s);
-    if (few_tiles<D>(b, 2))
+    if (few_tiles(D, b, 2))
       return adj_gather_threads<D, TB, BINS, 256>(b, std::min(b.total_tiles, 2 * b.sm_count), s);
   }
   return adj_gather_threads<D, TB, BINS, kAdjThreads<D>>(b, tile_grid(b, TK_ADJ_GATHER), s);

@@ -67,7 +67,8 @@ struct Graph {
 struct TuneState {
   int mode = 1;                         // MPM_TUNE_*
   bool pending[gbmpm::TK_COUNT] = {};   // kernel still being tried
-  bool tuned[gbmpm::TK_COUNT] = {};     // shape came from the cache or from trials
+  bool tuned[gbmpm::TK_COUNT] = {};     // shape came from the cache or from trials, or is fixed
+  bool fixed[gbmpm::TK_COUNT] = {};     // few tiles: the kernel runs wide CTAs, nothing is tried or stored
   int cand[gbmpm::TK_COUNT] = {};       // candidate under trial
   int rep[gbmpm::TK_COUNT] = {};        // timed launches of it so far
   int best[gbmpm::TK_COUNT] = {};
@@ -98,7 +99,7 @@ struct mpm_scene {
   float4* adj[2] = {nullptr, nullptr};
   int* d_step = nullptr;     // forward step counter (controller time)
   int* d_bstep = nullptr;    // reverse step counter
-  int* d_status = nullptr;
+  int* d_status = nullptr;   // status word, then the active tiles of the last P2G (b.n_active)
   // per-particle material (mpm_scene_set_material): E_p, m_p and the (gE, gm) accumulator
   float* d_pE = nullptr;
   float* d_pmass = nullptr;
@@ -254,6 +255,10 @@ struct ProfScope {
 // Looks the scene's workload up in the cache, or arms trials for its tile kernels (mode AUTO/FORCE).
 mpm_status tune_init(mpm_scene* s);
 void tune_release(mpm_scene* s);
+// More tiles were seen: kernels whose shape is no longer fixed take it from the cache, or are tried.
+mpm_status tune_unfix(mpm_scene* s);
+// The kernels of the mask whose launch shape counts for b.
+unsigned tunable(int dim, const BatchDev& b, unsigned kernels);
 // True while a tile kernel that phase ph launches is still being tried.
 bool tune_wants(const mpm_scene* s, int ph);
 // One directly-launched step of phase ph with the candidate shapes under trial, timed.

@@ -3,10 +3,11 @@
 // edge that mpm_tune_tile_edge measured fastest for a 2D workload.
 //
 // A trial step is an ordinary simulation step: the tile kernels process every tile whole inside
-// one CTA, so neither the number of CTAs nor (for G2P, whose outputs are per particle) the CTA
-// size changes a single bit of the results.  The adjoint gather's group sums are formed per warp
-// and then per CTA, so its CTA size would change their rounding: it is fixed per dimension and
-// only its CTAs per SM are tuned.
+// one CTA, so neither the number of CTAs nor the CTA size changes a single bit of the results (the
+// adjoint gather's group sums are formed per 32 particles and added in list order).  The adjoint
+// gather's CTA size is not tuned, only its CTAs per SM: 128 threads in 3D and 256 in 2D measured
+// fastest, and the few tiles of a small 3D scene take wider ones.  Kernels that do (few_tiles) are
+// neither tried nor stored: the cache's shapes are of scenes that run them.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -178,13 +179,46 @@ void env_load_locked() {
   if (p && *p) load_locked(p);  // a missing or unreadable file starts an empty cache
 }
 
-bool lookup(const Key& key, Entry* out) {
+constexpr unsigned kAllKernels = (1u << TK_COUNT) - 1;
+
+// True when the key's entry has every kernel of the mask tuned.
+bool lookup(const Key& key, unsigned kernels, Entry* out) {
   std::lock_guard<std::mutex> lk(g_mu);
   env_load_locked();
   auto it = g_cache.find(key);
-  if (it == g_cache.end() || g_partial.count(key)) return false;
+  if (it == g_cache.end()) return false;
+  auto m = g_partial.find(key);
+  if (m != g_partial.end() && (m->second & kernels) != kernels) return false;
   *out = it->second;
   return true;
+}
+
+// The shapes of the mask's kernels into the key's entry; a key whose four kernels are not all tuned yet
+// stays out of the cache file.
+void store_some(const Key& key, const TileLaunch* l, unsigned kernels) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  env_load_locked();
+  auto it = g_cache.find(key);
+  Entry e;
+  unsigned mask = 0;
+  if (it != g_cache.end()) {
+    e = it->second;
+    auto m = g_partial.find(key);
+    mask = m == g_partial.end() ? kAllKernels : m->second;
+  } else {
+    for (int k = 0; k < TK_COUNT; ++k) e.l[k] = kDefaultLaunch;
+  }
+  for (int k = 0; k < TK_COUNT; ++k)
+    if (kernels & (1u << k)) e.l[k] = l[k];
+  mask |= kernels;
+  g_cache[key] = e;
+  if ((mask & kAllKernels) == kAllKernels) {
+    g_partial.erase(key);
+    const char* p = std::getenv("GBMPM_TUNE_CACHE");
+    if (p && *p) save_locked(p);
+  } else {
+    g_partial[key] = mask;
+  }
 }
 
 void store(const Key& key, const Entry& e) {
@@ -225,6 +259,34 @@ bool phase_runs(int ph, int k) {
   return false;
 }
 
+// The kernels t has not settled: their shapes from the cache (AUTO), or trials armed for them.
+mpm_status settle(mpm_scene* s) {
+  TuneState& t = s->tune;
+  unsigned open = 0;
+  for (int k = 0; k < TK_COUNT; ++k)
+    if (!t.tuned[k]) open |= 1u << k;
+  if (open == 0) return MPM_OK;
+  Entry e;
+  if (t.mode == MPM_TUNE_AUTO && lookup(scene_key(s), open, &e)) {
+    for (int k = 0; k < TK_COUNT; ++k)
+      if (open & (1u << k)) {
+        s->b.launch[k] = e.l[k];
+        t.pending[k] = false;
+        t.tuned[k] = true;
+      }
+    return MPM_OK;
+  }
+  for (int k = 0; k < TK_COUNT; ++k)
+    for (int j = 0; j < 2; ++j)
+      if (!t.ev[k][j]) CK(cudaEventCreate(&t.ev[k][j]));
+  for (int k = 0; k < TK_COUNT; ++k)
+    if ((open & (1u << k)) && !t.pending[k]) {
+      t.pending[k] = true;
+      t.cand[k] = t.rep[k] = t.best[k] = 0;
+    }
+  return MPM_OK;
+}
+
 void destroy_events(mpm_scene* s) {
   for (int k = 0; k < TK_COUNT; ++k)
     for (int j = 0; j < 2; ++j)
@@ -239,24 +301,26 @@ void destroy_events(mpm_scene* s) {
 mpm_status tune_init(mpm_scene* s) {
   TuneState& t = s->tune;
   for (int k = 0; k < TK_COUNT; ++k) {
-    t.pending[k] = t.tuned[k] = false;
+    t.pending[k] = t.tuned[k] = t.fixed[k] = false;
     t.cand[k] = t.rep[k] = t.best[k] = 0;
   }
   default_launch(s->b, s->ctx->sm_count);
   if (s->impl != MPM_IMPL_TILED || t.mode == MPM_TUNE_OFF) return MPM_OK;
-  Entry e;
-  if (t.mode == MPM_TUNE_AUTO && lookup(scene_key(s), &e)) {
-    for (int k = 0; k < TK_COUNT; ++k) {
-      s->b.launch[k] = e.l[k];
-      t.tuned[k] = true;
-    }
-    return MPM_OK;
-  }
+  for (int k = 0; k < TK_COUNT; ++k) t.fixed[k] = t.tuned[k] = shape_fixed(s->dim, s->b, k);
+  return settle(s);
+}
+
+mpm_status tune_unfix(mpm_scene* s) {
+  TuneState& t = s->tune;
   for (int k = 0; k < TK_COUNT; ++k)
-    for (int j = 0; j < 2; ++j)
-      if (!t.ev[k][j]) CK(cudaEventCreate(&t.ev[k][j]));
-  for (int k = 0; k < TK_COUNT; ++k) t.pending[k] = true;
-  return MPM_OK;
+    if (t.fixed[k] && !shape_fixed(s->dim, s->b, k)) t.fixed[k] = t.tuned[k] = false;
+  return t.mode == MPM_TUNE_OFF || s->impl != MPM_IMPL_TILED ? MPM_OK : settle(s);
+}
+
+unsigned tunable(int dim, const BatchDev& b, unsigned kernels) {
+  for (int k = 0; k < TK_COUNT; ++k)
+    if (shape_fixed(dim, b, k)) kernels &= ~(1u << k);
+  return kernels;
 }
 
 void tune_release(mpm_scene* s) { destroy_events(s); }
@@ -343,9 +407,10 @@ mpm_status tune_step(mpm_scene* s, int ph) {
     bool all = true;
     for (int k = 0; k < TK_COUNT; ++k) all = all && t.tuned[k];
     if (all) {
-      Entry e;
-      for (int k = 0; k < TK_COUNT; ++k) e.l[k] = s->b.launch[k];
-      store(scene_key(s), e);
+      unsigned tried = 0;
+      for (int k = 0; k < TK_COUNT; ++k)
+        if (!t.fixed[k]) tried |= 1u << k;
+      store_some(scene_key(s), s->b.launch, tried);
       destroy_events(s);
     }
   }
@@ -432,34 +497,10 @@ mpm_status batch_tune_end(TuneState& t, BatchDev& b, int dim) {
   bool left = false;
   for (int k = 0; k < TK_COUNT; ++k) left = left || t.pending[k];
   if (finished && !left) {
-    // merge this composition's kernels into the key's entry; a key whose four kernels are not all
-    // tuned yet stays out of the cache file
-    const Key key = make_key(dim, b.total_particles, b.total_tiles, b.sm_count);
-    std::lock_guard<std::mutex> lk(g_mu);
-    env_load_locked();
-    auto it = g_cache.find(key);
-    Entry e;
-    unsigned mask = 0;
-    if (it != g_cache.end()) {
-      e = it->second;
-      auto m = g_partial.find(key);
-      mask = m == g_partial.end() ? ~0u : m->second;
-    } else {
-      for (int k = 0; k < TK_COUNT; ++k) e.l[k] = kDefaultLaunch;
-    }
+    unsigned mask = 0;  // this composition's kernels
     for (int k = 0; k < TK_COUNT; ++k)
-      if (t.tuned[k]) {
-        e.l[k] = b.launch[k];
-        mask |= 1u << k;
-      }
-    g_cache[key] = e;
-    if ((mask & ((1u << TK_COUNT) - 1)) == (1u << TK_COUNT) - 1) {
-      g_partial.erase(key);
-      const char* p = std::getenv("GBMPM_TUNE_CACHE");
-      if (p && *p) save_locked(p);
-    } else {
-      g_partial[key] = mask;
-    }
+      if (t.tuned[k]) mask |= 1u << k;
+    store_some(make_key(dim, b.total_particles, b.total_tiles, b.sm_count), b.launch, mask);
     destroy_batch_events(t);
   }
   return MPM_OK;
@@ -494,7 +535,7 @@ mpm_status mpm_tune_cache_lookup(int dim, long long particles, long long grid_ti
                                  int* found) {
   if ((dim != 2 && dim != 3) || sm_count < 1 || !shape || !found) return MPM_ERR_ARG;
   Entry e;
-  *found = lookup(make_key(dim, particles, grid_tiles, sm_count), &e) ? 1 : 0;
+  *found = lookup(make_key(dim, particles, grid_tiles, sm_count), kAllKernels, &e) ? 1 : 0;
   if (*found)
     for (int k = 0; k < TK_COUNT; ++k) {
       shape[2 * k] = e.l[k].ctas_per_sm;
