@@ -694,6 +694,8 @@ void free_rollout(mpm_scene* s) {
   if (!s->roll_allocs.empty()) cudaStreamSynchronize(s->ctx->stream);
   for (void* p : s->roll_allocs) cudaFree(p);
   s->roll_allocs.clear();
+  s->ctx->kept_bytes -= s->kept_bytes;
+  s->kept_bytes = 0;
   s->ckpt.clear();
   s->seg.clear();
   s->pool_backed = false;

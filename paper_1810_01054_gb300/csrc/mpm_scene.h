@@ -48,6 +48,7 @@ struct mpm_ctx {
   int prof_used = 0;
   std::atomic<int> live{0};  // scenes and batches created on this context and not yet destroyed
   std::atomic<size_t> bin_bytes{0};  // tile bins of its scenes and batches
+  std::atomic<size_t> kept_bytes{0};  // states its scenes hold because a batch kept every one
   std::atomic<size_t> bin_limit{gbmpm::BIN_BYTES};  // the most they may take
 };
 
@@ -169,6 +170,7 @@ struct mpm_scene {
   bool graphs_ws2 = false;  // workspace the recompute graphs were captured with
   bool graphs_branch = false;  // whether the reverse graphs bin (or load sorts) on a branch
   size_t roll_budget = 0;
+  size_t kept_bytes = 0;       // of the context's, this scene's rollout buffers
   cudaEvent_t ev_rcm[2] = {}, ev_rev[2] = {}, ev_fork = nullptr;
   // Reverse graphs of a tiled scene whose controller reads no state: each step's controller
   // reverse is captured on a branch (ctx->capture2) that the next step's adjoint gather joins, so it
