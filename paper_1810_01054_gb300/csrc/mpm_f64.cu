@@ -51,7 +51,7 @@ struct Par64 {
   double* adj_out;         // adjoint of state n (reverse)
   double* grid;            // [nodes][4]
   double* grid_b;          // [nodes][4]
-  double *grid_next, *grid_b_next;  // the next step's grids, cleared by this step's grid update
+  double *grid_next, *grid_b_next;  // the next step's grids, cleared by this step's grid update (NULL: none)
   double* g_act;           // [G] dL/da of this step (reverse), nullptr = not wanted
   int* status;
 };
@@ -245,8 +245,9 @@ __global__ void __launch_bounds__(F64_THREADS) k64_grid(Par64 p, int n_nodes) {
   if (nl >= n_nodes) return;
 #pragma unroll
   for (int a = 0; a < 4; ++a) {  // the next step's sums start from zero
-    p.grid_next[size_t(nl) * 4 + a] = 0.0;
-    if constexpr (ADJ) p.grid_b_next[size_t(nl) * 4 + a] = 0.0;
+    if (p.grid_next) p.grid_next[size_t(nl) * 4 + a] = 0.0;
+    if constexpr (ADJ)
+      if (p.grid_next) p.grid_b_next[size_t(nl) * 4 + a] = 0.0;
   }
   int node[D];
   {
@@ -556,6 +557,7 @@ struct mpm_scene64 {
   double* act = nullptr;       // [L][G] actuation table
   double* g_act = nullptr;     // [L][G] dL/dU of the last reverse pass
   int L = 0;
+  double* grid2 = nullptr;     // second pair of grids (step_par); hp.grid is the first
   double* hist = nullptr;      // [T + 1][S][N] states of the last rollout
   int T = -1;                  // steps of the last rollout (-1: none)
   size_t hist_cap = 0;         // states hist can hold
@@ -588,10 +590,25 @@ mpm_status cuda_status(cudaError_t e) {
     if (s_ != MPM_OK) return s_; \
   } while (0)
 
+void drop_graphs(mpm_scene64* s);
+
+// Device memory for the scene; where there is none left, what its second pair of grids holds.
+mpm_status device_alloc(mpm_scene64* s, void** q, size_t bytes) {
+  cudaError_t e = cudaMalloc(q, bytes);
+  if (s->grid2 && gbmpm::out_of_memory(e)) {
+    CK64(cudaStreamSynchronize(s->ctx->stream));
+    drop_graphs(s);  // they name it
+    cudaFree(s->grid2);
+    s->grid2 = nullptr;
+    e = cudaMalloc(q, bytes);
+  }
+  return cuda_status(e);
+}
+
 template <class T>
 mpm_status alloc64(mpm_scene64* s, T** p, size_t count) {
   void* q = nullptr;
-  CK64(cudaMalloc(&q, std::max<size_t>(count * sizeof(T), 16)));
+  CKS64(device_alloc(s, &q, std::max<size_t>(count * sizeof(T), 16)));
   s->allocs.push_back(q);
   *p = static_cast<T*>(q);
   return MPM_OK;
@@ -667,7 +684,8 @@ void drop_graphs(mpm_scene64* s) {
 }
 
 // The grids are held twice: the i-th step of a pass sums into one pair while its grid update clears
-// the other.  The first step's pair is cleared when the pass starts.
+// the other.  The first step's pair is cleared when the pass starts.  Where the device has no room for
+// the second pair, every step's launches follow a clear of the first.
 mpm_status clear_grids(mpm_scene64* s, cudaStream_t str) {
   CK64(cudaMemsetAsync(s->hp.grid, 0, sizeof(double) * 8 * size_t(s->n_nodes), str));
   return MPM_OK;
@@ -676,11 +694,12 @@ mpm_status clear_grids(mpm_scene64* s, cudaStream_t str) {
 // Scene constants and the grids of the i-th step of a pass.
 Par64 step_par(const mpm_scene64* s, int i) {
   Par64 p = s->hp;
-  const size_t pair = size_t(8) * s->n_nodes, odd = size_t(i & 1) * pair;
-  p.grid = s->hp.grid + odd;
-  p.grid_b = p.grid + pair / 2;
-  p.grid_next = s->hp.grid + (pair - odd);
-  p.grid_b_next = p.grid_next + pair / 2;
+  const size_t half = size_t(4) * s->n_nodes;
+  const bool odd = s->grid2 && (i & 1);
+  p.grid = odd ? s->grid2 : s->hp.grid;
+  p.grid_b = p.grid + half;
+  p.grid_next = odd ? s->hp.grid : s->grid2;
+  p.grid_b_next = p.grid_next ? p.grid_next + half : nullptr;
   return p;
 }
 
@@ -691,6 +710,7 @@ mpm_status enqueue_rollout(mpm_scene64* s, int T, cudaStream_t str) {
   CK64(cudaMemsetAsync(s->hp.status, 0, sizeof(int), str));
   CK64(cudaMemcpyAsync(s->hist, s->init, sizeof(double) * stride, cudaMemcpyDeviceToDevice, str));
   for (int t = 0; t < T; ++t) {
+    if (t > 0 && !s->grid2) CKS64(clear_grids(s, str));
     Par64 p = step_par(s, t);
     p.st = s->hist + size_t(t) * stride;
     p.st_out = s->hist + size_t(t + 1) * stride;
@@ -708,6 +728,7 @@ mpm_status enqueue_reverse(mpm_scene64* s, int T, cudaStream_t str) {
   if (size_t(s->L) * s->G > 0) CK64(cudaMemsetAsync(s->g_act, 0, sizeof(double) * size_t(s->L) * s->G, str));
   int cur = 0;
   for (int t = T - 1; t >= 0; --t) {
+    if (t < T - 1 && !s->grid2) CKS64(clear_grids(s, str));
     Par64 p = step_par(s, T - 1 - t);
     p.st = s->hist + size_t(t) * stride;
     p.adj_in = s->adj[cur];
@@ -764,6 +785,7 @@ mpm_status mpm64_destroy(mpm_scene64* s) {
   drop_graphs(s);
   for (void* p : s->allocs) cudaFree(p);
   if (s->hist) cudaFree(s->hist);
+  if (s->grid2) cudaFree(s->grid2);
   s->ctx->live.fetch_sub(1);
   delete s;
   return MPM_OK;
@@ -843,7 +865,7 @@ mpm_status mpm64_create(mpm_ctx* c, const mpm_scene64_desc* d, mpm_scene64** out
   if ((st = alloc64(s, &s->init, SN)) != MPM_OK) return fail(st);
   if ((st = alloc64(s, &s->adj[0], SN)) != MPM_OK) return fail(st);
   if ((st = alloc64(s, &s->adj[1], SN)) != MPM_OK) return fail(st);
-  if ((st = alloc64(s, &p.grid, size_t(16) * s->n_nodes)) != MPM_OK) return fail(st);  // two pairs (step_par)
+  if ((st = alloc64(s, &p.grid, size_t(8) * s->n_nodes)) != MPM_OK) return fail(st);  // a pair; the second last
   if ((st = alloc64(s, &group, std::max(1, s->N))) != MPM_OK) return fail(st);
   if ((st = alloc64(s, &act_dir, std::max(1, s->G * dim))) != MPM_OK) return fail(st);
   if ((st = alloc64(s, &p.status, 1)) != MPM_OK) return fail(st);
@@ -864,6 +886,10 @@ mpm_status mpm64_create(mpm_ctx* c, const mpm_scene64_desc* d, mpm_scene64** out
   if (cudaMemsetAsync(p.status, 0, sizeof(int), str) != cudaSuccess) return fail(MPM_ERR_CUDA);
   if ((st = upload_state(s, s->init, d->x0, d->v0, d->C0, d->F0)) != MPM_OK) return fail(st);
   if ((st = mpm64_set_actuation(s, d->act, d->n_act_steps)) != MPM_OK) return fail(st);
+  void* second = nullptr;
+  st = device_alloc(s, &second, sizeof(double) * 8 * size_t(s->n_nodes));
+  if (st != MPM_OK && st != MPM_ERR_OOM) return fail(st);
+  s->grid2 = static_cast<double*>(second);
   *out = s;
   return MPM_OK;
 }
@@ -915,7 +941,7 @@ mpm_status mpm64_rollout(mpm_scene64* s, int T) {
     s->hist_cap = 0;
     s->T = -1;
     void* q = nullptr;
-    CK64(cudaMalloc(&q, state * (size_t(T) + 1)));
+    CKS64(device_alloc(s, &q, state * (size_t(T) + 1)));
     s->hist = static_cast<double*>(q);
     s->hist_cap = size_t(T) + 1;
   }
