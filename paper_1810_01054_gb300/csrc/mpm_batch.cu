@@ -521,6 +521,35 @@ int request_interval(const mpm_batch* B, const mpm_scene* s, int T, int want_gra
   return need <= KEEP_ONE && B->ctx->kept_bytes - s->kept_bytes + need <= KEEP_ALL ? 1 : sqrt_interval(T);
 }
 
+// Up to max_steps batched steps.
+mpm_status run_steps(mpm_batch* B, int max_steps) {
+  look_at_tiles(B, B->fwd);
+  look_at_tiles(B, B->rev);
+  for (int it = 0; it < max_steps; ++it) {
+    bool busy = false;
+    for (const Slot& sl : B->slots) busy = busy || sl.state == S_FWD || sl.state == S_RCM || sl.state == S_REV;
+    if (!busy) break;
+    if (B->dirty) CKS(recompose(B));
+    // the two halves touch disjoint scenes and buffers: the reverse half runs on the second
+    // stream beside the forward half, joined before the bookkeeping
+    cudaStream_t ms = B->ctx->stream, as = B->ctx->aux;
+    CK(cudaEventRecord(B->fork, ms));
+    CK(cudaStreamWaitEvent(as, B->fork, 0));
+    if (B->dim == 2) {
+      CKS(forward_step<2>(B, ms));
+      CKS(reverse_step<2>(B, as));
+    } else {
+      CKS(forward_step<3>(B, ms));
+      CKS(reverse_step<3>(B, as));
+    }
+    CK(cudaEventRecord(B->join, as));
+    CK(cudaStreamWaitEvent(ms, B->join, 0));
+    CKS(advance(B));
+  }
+  CKS(ask_tiles(B, B->fwd));
+  return ask_tiles(B, B->rev);
+}
+
 }  // namespace
 
 extern "C" {
@@ -612,32 +641,12 @@ mpm_status mpm_batch_admit(mpm_batch* B, mpm_scene* s, int n_steps, int want_gra
 
 mpm_status mpm_batch_tick(mpm_batch* B, int max_steps) {
   if (!B || max_steps < 1) return MPM_ERR_ARG;
-  look_at_tiles(B, B->fwd);
-  look_at_tiles(B, B->rev);
-  for (int it = 0; it < max_steps; ++it) {
-    bool busy = false;
-    for (const Slot& sl : B->slots) busy = busy || sl.state == S_FWD || sl.state == S_RCM || sl.state == S_REV;
-    if (!busy) break;
-    if (B->dirty) CKS(recompose(B));
-    // the two halves touch disjoint scenes and buffers: the reverse half runs on the second
-    // stream beside the forward half, joined before the bookkeeping
-    cudaStream_t ms = B->ctx->stream, as = B->ctx->aux;
-    CK(cudaEventRecord(B->fork, ms));
-    CK(cudaStreamWaitEvent(as, B->fork, 0));
-    if (B->dim == 2) {
-      CKS(forward_step<2>(B, ms));
-      CKS(reverse_step<2>(B, as));
-    } else {
-      CKS(forward_step<3>(B, ms));
-      CKS(reverse_step<3>(B, as));
-    }
-    CK(cudaEventRecord(B->join, as));
-    CK(cudaStreamWaitEvent(ms, B->join, 0));
-    CKS(advance(B));
-  }
-  CKS(ask_tiles(B, B->fwd));
-  CKS(ask_tiles(B, B->rev));
-  CKS(finish_requests(B));
+  const mpm_status ran = run_steps(B, max_steps);
+  // the requests that finished are closed even if a later step could not run (the arrays of a new
+  // composition that do not fit): their release may be what makes room
+  const mpm_status closed = finish_requests(B);
+  CKS(ran);
+  CKS(closed);
   CK(cudaGetLastError());
   return MPM_OK;
 }

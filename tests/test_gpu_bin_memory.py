@@ -207,3 +207,43 @@ def test_a_batch_that_ran_out_of_memory_goes_on_when_there_is_some(M, ctx):
     batch.close()
     for sc in scenes:
         sc.close()
+
+
+def test_requests_that_finished_close_though_the_next_composition_does_not_fit(M, ctx):
+    """A tick in which a short request ends before a longer one's next phase finds no memory: the first is
+    done and can be released, which lets the second go on."""
+    import torch
+    spec = _spec()
+    ctx.set_bin_bytes(0)
+    alone = M.Scene(ctx, spec)
+    alone.step(3)
+    want = list(alone.get_state())
+    alone.close()
+    short, long = M.Scene(ctx, spec), M.Scene(ctx, spec)
+    batch = M.Batch(ctx, 3)
+    a, b = batch.admit(short, 3, False), batch.admit(long, 6, True)
+    batch.tick(1)  # the forward half's arrays
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - 16 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(M.MPMError) as e:
+            batch.tick(20)  # the reverse half's node blocks take 28 MB
+        assert e.value.status == -2
+        assert batch.poll(a) and not batch.poll(b)
+        _same(list(short.get_state()), want)
+        batch.release(a)
+        short.close()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    while not batch.poll(b):
+        batch.tick(5)
+    single = M.Scene(ctx, spec)
+    single.rollout(6, 1)
+    seed = np.zeros((single.N, 3))
+    seed[:, 0] = 1.0 / single.N
+    ref = list(single.get_state()) + list(single.backward(seed))
+    _same(list(long.get_state()) + list(long.gradients()), ref)
+    batch.close()
+    for sc in (long, single):
+        sc.close()
