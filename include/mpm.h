@@ -148,8 +148,8 @@ mpm_status mpm_step(mpm_scene* scene, int n_steps);
  * asynchronously; the checkpoint buffers are kept for the next rollout of the same shape.
  * storing the state every ckpt_interval steps (0 = choose from mem_budget_bytes: every step if
  * all states fit; else, in the tiled form, the smallest interval whose checkpoints, two sets of
- * recompute buffers and (beyond 4096 tiles) the sorts an overlapped reverse pass keeps fit, so that the fewest
- * steps are recomputed and the recompute runs beside the reverse steps; else about sqrt(n_steps);
+ * recompute buffers and (in scenes without bins) the sorts an overlapped reverse pass keeps fit, so
+ * that the fewest steps are recomputed and the recompute runs beside the reverse steps; else about sqrt(n_steps);
  * mpm_scene_plan_rollout reports the choice); the states in between are recomputed by
  * mpm_backward.  The further tile bins of the reverse pass are taken from what the budget leaves
  * beside that.  mem_budget_bytes = 0 means no

@@ -379,7 +379,7 @@ ScenePar rec_rev(const mpm_scene* s, float4* st, const float4* ain, float4* aout
 // ---------------------------------------------------------------------------- step sequences
 // Forward step of phase ph (PH_STEP, PH_ROLL, PH_RCM) on stream st.
 // The tiled form makes the step's record selection inside its first kernel (the sort here, the
-// keys in the reverse step); the plain form launches it separately.  The sort does not depend on
+// keys in the reverse step; with bins the G2P before makes it); the plain form launches it separately.  The sort does not depend on
 // the controller, so the controller's forward runs after it.
 // Workspace of phase ph: the recompute (and the bin keys of its checkpoint) use workspace 2 when
 // the reverse tables say so; its launch shapes follow the scene's.

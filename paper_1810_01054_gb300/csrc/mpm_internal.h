@@ -168,10 +168,11 @@ struct BatchDev {
   // P2G clears the other parity's mask and counts; a phase starts from all zeros (launch_keys).
   // The line at BIN_TILES: the two lists take 16 or 32 KB a tile and set (their room cannot overflow
   // before the tile's kernels refuse it), 128 MB at most, and a tile mask of 128 words is a word per
-  // thread of the smallest CTA; beyond it a step is long enough that the sort's launches (19 of 143 us
-  // at one million particles) matter less.  Steps with bins against the sort: 1,024 particles (2D)
-  // 13.3 -> 10.9 us, the 31k walker 16.9 -> 13.9 us; 24 steps with the gradient of the 95k soft body
-  // (4096 tiles) 3434-3479 -> 2947-3040 us.
+  // thread of the smallest CTA; beyond it a step is long enough that the sort's launches (19 of 127 us
+  // at one million particles) matter less.  Calls with the sort and with bins: 64 steps of 1,024
+  // particles (2D) 783-803 and 648-700 us, 48 steps of the 31k walker 740-748 and 649-655; with the
+  // gradient, 48 steps of 1,024 particles 2116-2151 and 1536-1630, 24 of the 95k soft body (4096
+  // tiles) 3508-3522 and 3260-3263.
   uint32_t *bin_ctl, *bin_raw;
   int rec_flip;         // scenes[] holds one scene's records by parity (a scene alone, with bins)
   float4* partial;      // [total_tiles * BLOCK_NODES] node blocks of P2G

@@ -3,7 +3,8 @@
 // Forward step (Section III, Eqs. 3-10), tiled form:
 //   tile bins                 : up to 4096 tiles, the kernel that moves a particle (k_g2p; k_keys at a
 //                               phase's start) appends it to the list of its stencil base's tile;
-//   k_keys / scan / k_scatter : beyond that a sort by tile (k_g2p writes the next step's keys)
+//   k_keys / scan / k_scatter : beyond that, or without room for bins, a sort by tile (k_g2p writes the
+//                               next step's keys)
 //   k_p2g                     : per tile, canonical (cell, id) order, per-particle stress and
 //                               MLS matrix G (Eq. 4), per-cell register accumulation of the
 //                               3^d stencil (Eqs. 3, 5), fixed-order reduction into the tile's
@@ -2728,7 +2729,8 @@ __global__ void __launch_bounds__(PACK_THREADS) k_unpack(int N, int npad, const 
 // table[map[*ctr - base]] (map NULL: table[0]), with the batch offsets patched in; the
 // sinusoid controllers' actuation a_g(t_n) is evaluated here too.  Every step of a rollout is
 // then the same launch sequence, which CUDA graphs replay.  (A single tiled scene makes this
-// selection inside the first kernel of its step instead: k_keys, k_scatter, k_scan_reduce.)
+// selection inside a kernel of its steps instead: with bins an extra CTA of k_g2p selects the next
+// step's, a step that sorts its own in k_scatter or k_scan_reduce, a reverse step in k_keys.)
 __global__ void k_select(const SelectPar* __restrict__ sel, ScenePar* __restrict__ cur, const uint32_t* flip) {
   pdl_enter();
   select_publish(sel[blockIdx.x], cur + (flip ? *flip & 1u : blockIdx.x));
