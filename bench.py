@@ -721,7 +721,7 @@ def measure_paper_cube(args, dev, stream, sizes=((3, 20), (3, 40), (3, 80), (2, 
 F64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # FP64 arithmetic of the per-particle adjoint kernel (S4 (F)-(K), (J)), DADD + DMUL + 2 DFMA thread
 # instructions per particle from the ncu counters of the 3D capture (profiles/k64_fp64_box_cluster_3d.md)
-F64_ADJ_FLOPS_3D = 3700.0
+F64_ADJ_FLOPS_3D = 3440.0
 
 
 def table_of(spec, T):
