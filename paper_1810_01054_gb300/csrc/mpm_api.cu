@@ -928,7 +928,9 @@ mpm_status read_status(mpm_scene* s) {
   int v[2] = {0, 0};
   CK(cudaStreamSynchronize(s->ctx->stream));
   CK(cudaMemcpy(v, s->d_status, sizeof(v), cudaMemcpyDeviceToHost));
-  if (v[1] > s->b.occupied) {  // the body spread, or set_state spread it: its CTA sizes follow
+  // the body spread, or set_state spread it: its CTA sizes follow (0: the plain form, or nothing was
+  // in the grid at creation, which leaves the shapes of many tiles)
+  if (s->b.occupied > 0 && v[1] > s->b.occupied) {
     const bool few[2] = {few_tiles(s->dim, s->b, 1), few_tiles(s->dim, s->b, 2)};
     s->b.occupied = v[1];
     if (few[0] != few_tiles(s->dim, s->b, 1) || few[1] != few_tiles(s->dim, s->b, 2)) {

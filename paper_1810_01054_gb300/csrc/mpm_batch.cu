@@ -299,11 +299,15 @@ void look_at_tiles(mpm_batch* B, SubBatch& sb) {
   const bool same = sb.seen_composed == sb.composed;
   sb.seen_composed = -1;
   if (!same || *sb.seen <= sb.b.occupied) return;
+  const unsigned before = tunable(B->dim, sb.b, ~0u);
+  int sum = 0;
   for (int m : sb.members) {
     int& o = B->slots[m].tiles;
     o = int((long long)(o) * *sb.seen / sb.b.occupied) + 1;
+    sum += o;
   }
-  B->dirty = true;
+  sb.b.occupied = sum;
+  if (tunable(B->dim, sb.b, ~0u) != before) B->dirty = true;  // composed anew with other launch shapes
 }
 
 // Counts a step of the half's key; its trials start once the key has run kTrialWait steps.
