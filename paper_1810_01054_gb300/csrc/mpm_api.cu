@@ -737,6 +737,16 @@ mpm_status further_bins(mpm_scene* s, BinSet& set, size_t* room) {
   return MPM_OK;
 }
 
+// Device memory for the scene's rollouts and reverse passes; where there is none left, what the further
+// sets of bins hold.
+template <class T>
+mpm_status scene_alloc(mpm_scene* s, T** p, size_t count, std::vector<void*>& list) {
+  mpm_status st = dalloc(p, count, list);
+  if (st != MPM_ERR_OOM || !(s->bins2.mem || s->binsB.mem)) return st;
+  for (BinSet* set : {&s->bins2, &s->binsB}) CKS(give_up_bins(s, *set));
+  return dalloc(p, count, list);
+}
+
 void free_ws2(mpm_scene* s);
 
 // Workspace 2 (allocated on the first reverse pass that overlaps its recompute; all or nothing).
@@ -995,7 +1005,7 @@ mpm_status prepare_rollout(mpm_scene* s, int T, int k, size_t budget) {
     free_rollout(s);  // buffers of another shape
     s->ckpt.assign(nseg, nullptr);
     for (int i = 0; i < nseg; ++i) {
-      mpm_status st = dalloc(&s->ckpt[i], S / sizeof(float4), s->roll_allocs);
+      mpm_status st = scene_alloc(s, &s->ckpt[i], S / sizeof(float4), s->roll_allocs);
       if (st != MPM_OK) {
         free_rollout(s);
         return st;
@@ -1003,7 +1013,7 @@ mpm_status prepare_rollout(mpm_scene* s, int T, int k, size_t budget) {
     }
     s->seg.assign(std::max(0, k - 1), nullptr);
     for (int i = 0; i < k - 1; ++i) {
-      mpm_status st = dalloc(&s->seg[i], S / sizeof(float4), s->roll_allocs);
+      mpm_status st = scene_alloc(s, &s->seg[i], S / sizeof(float4), s->roll_allocs);
       if (st != MPM_OK) {
         free_rollout(s);
         return st;
@@ -1114,10 +1124,21 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
     else
       CKS(st_b);
   }
-  if (overlap) CKS(ensure_ws2(s));
+  if (overlap) {
+    CKS(ensure_ws2(s));
+    if (int(s->seg2.size()) != k - 1) {
+      std::vector<float4*> segs(k - 1, nullptr);  // the scene keeps them only once all exist
+      for (int i = 0; i < k - 1; ++i) CKS(scene_alloc(s, &segs[i], S / sizeof(float4), s->roll_allocs));
+      s->seg2 = segs;
+    }
+    // the sorts of every recomputed state, by segment parity (each reverse step loads its own)
+    if (!s->sort_store && !bins)
+      CKS(dalloc(&s->sort_store, (store_bytes - ctrl_bytes) / sizeof(uint32_t), s->roll_allocs));
+    if (keep_ctrl && !s->ctrl_store) CKS(scene_alloc(s, &s->ctrl_store, ctrl_bytes / sizeof(float), s->roll_allocs));
+  }
   // A scene with bins gives set B and workspace 2 bins of their own from what the budget leaves beside
-  // the states, while the context and the device have them.  Set B first: the reverse steps are the
-  // critical path.  Without them set B is not used (the states are binned in line), and the recompute
+  // the states, while the context and (after the buffers above) the device have them.  Set B first: the
+  // reverse steps are the critical path.  Without them set B is not used (the states are binned in line), and the recompute
   // sorts.  What a budget has no room or use for is given back.
   size_t room = s->roll_budget == 0 ? SIZE_MAX
                 : overlap           ? s->roll_budget - ((size_t(nseg) + 2 * size_t(k - 1)) * S + store_bytes)
@@ -1134,17 +1155,6 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
     use_bins(s->b2, s->bins2, dim, s->b.tile_edge, s->hp.n_tiles, s->sorted2);
   } else if (s->roll_budget != 0) {
     CKS(give_up_bins(s, s->bins2));
-  }
-  if (overlap) {
-    if (int(s->seg2.size()) != k - 1) {
-      std::vector<float4*> segs(k - 1, nullptr);  // the scene keeps them only once all exist
-      for (int i = 0; i < k - 1; ++i) CKS(dalloc(&segs[i], S / sizeof(float4), s->roll_allocs));
-      s->seg2 = segs;
-    }
-    // the sorts of every recomputed state, by segment parity (each reverse step loads its own)
-    if (!s->sort_store && !bins)
-      CKS(dalloc(&s->sort_store, (store_bytes - ctrl_bytes) / sizeof(uint32_t), s->roll_allocs));
-    if (keep_ctrl && !s->ctrl_store) CKS(dalloc(&s->ctrl_store, ctrl_bytes / sizeof(float), s->roll_allocs));
   }
   if (s->graphs_ws2 != overlap || s->graphs_branch != branch) {
     drop_reverse_graphs(s);
@@ -1840,11 +1850,6 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   b.n_active = s->d_status + 1;
   ALLOC(b.block_sums, 2 * ((p.n_tiles + 2047) / 2048) + 2);
   ALLOC(b.work, 4);
-  if (s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES)
-    TRY(take_bins(c, s->bins, bin_set_bytes(dim, edge, p.n_tiles)));
-  if (!s->bins.mem) ALLOC(b.sorted, s->npad);
-  use_bins(b, s->bins, dim, edge, p.n_tiles, b.sorted);
-  b.rec_flip = s->bins.mem ? 1 : 0;
   if (s->impl == MPM_IMPL_TILED) {
     ALLOC(b.partial, size_t(p.n_tiles) * NB);
     ALLOC(b.partial_b, size_t(p.n_tiles) * NB);
@@ -1956,6 +1961,12 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   TRY(upload_table(s, 0, t0));
   s->hsel[PH_STEP].table = s->tables[0].dev;
   TRY(upload_sel(s));
+  ALLOC(b.sorted, s->npad);
+  // bins last: they are what the scene can do without
+  if (s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES)
+    TRY(take_bins(c, s->bins, bin_set_bytes(dim, edge, p.n_tiles)));
+  use_bins(b, s->bins, dim, edge, p.n_tiles, b.sorted);
+  b.rec_flip = s->bins.mem ? 1 : 0;
   TRY(tune_init(s));
   TRY(enqueue_keys(s, PH_STEP, stream));
   TRY(read_status(s));

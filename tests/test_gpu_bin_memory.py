@@ -247,3 +247,39 @@ def test_requests_that_finished_close_though_the_next_composition_does_not_fit(M
     batch.close()
     for sc in (long, single):
         sc.close()
+
+
+def test_bins_yield_to_what_a_scene_cannot_do_without(M, ctx):
+    """A scene whose other arrays fit beside no bins is created without them; a rollout's states take the
+    memory of the reverse pass's further sets."""
+    import torch
+    spec = _spec()
+    sc = M.Scene(ctx, spec)
+    want = _pass(sc, spec, 6, 2)
+    held, size = ctx.bin_bytes()[0], sc.info()["state_bytes"]  # three sets
+
+    def fill(leave):
+        torch.cuda.empty_cache()
+        return torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+
+    hold = fill(16 * MB)
+    T = 64 * MB // size
+    got = _pass(sc, spec, T, 1)  # 64 MB of states
+    del hold
+    torch.cuda.empty_cache()
+    assert ctx.bin_bytes()[0] < held
+    other = M.Scene(ctx, spec)
+    _same(_pass(other, spec, T, 1), got)
+    other.close()
+    _same(_pass(sc, spec, 6, 2), want)
+    sc.close()
+    hold = fill(150 * MB)  # the bins alone would fit (134 MB), not with the 40 MB of the rest
+    try:
+        sc = M.Scene(ctx, spec)
+        assert ctx.bin_bytes()[0] == 0
+        sc.step(6)
+        _same(list(sc.get_state()), want[:4])
+        sc.close()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
