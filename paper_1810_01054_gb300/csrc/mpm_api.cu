@@ -1124,8 +1124,23 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
     else
       CKS(st_b);
   }
+  if (overlap) CKS(ensure_ws2(s));
+  // A scene with bins gives set B and workspace 2 bins of their own from what the budget leaves beside
+  // the states, while the context and (beside the buffers below) the device have them.  Set B first: the
+  // reverse steps are the critical path.  Without them set B is not used (the states are binned in
+  // line), and the recompute sorts.  What a budget has no room or use for is given back.
+  size_t room = s->roll_budget == 0 ? SIZE_MAX
+                : overlap           ? s->roll_budget - ((size_t(nseg) + 2 * size_t(k - 1)) * S + store_bytes)
+                                    : s->roll_budget - std::min(s->roll_budget, (size_t(nseg) + size_t(k - 1)) * S);
+  if (bins && branch)
+    CKS(further_bins(s, s->binsB, &room));
+  else if (s->roll_budget != 0)
+    CKS(give_up_bins(s, s->binsB));
+  if (bins && overlap)
+    CKS(further_bins(s, s->bins2, &room));
+  else if (s->roll_budget != 0)
+    CKS(give_up_bins(s, s->bins2));
   if (overlap) {
-    CKS(ensure_ws2(s));
     if (int(s->seg2.size()) != k - 1) {
       std::vector<float4*> segs(k - 1, nullptr);  // the scene keeps them only once all exist
       for (int i = 0; i < k - 1; ++i) CKS(scene_alloc(s, &segs[i], S / sizeof(float4), s->roll_allocs));
@@ -1136,26 +1151,11 @@ mpm_status prepare_backward(mpm_scene* s, const float* gxT, const float* gvT, co
       CKS(dalloc(&s->sort_store, (store_bytes - ctrl_bytes) / sizeof(uint32_t), s->roll_allocs));
     if (keep_ctrl && !s->ctrl_store) CKS(scene_alloc(s, &s->ctrl_store, ctrl_bytes / sizeof(float), s->roll_allocs));
   }
-  // A scene with bins gives set B and workspace 2 bins of their own from what the budget leaves beside
-  // the states, while the context and (after the buffers above) the device have them.  Set B first: the
-  // reverse steps are the critical path.  Without them set B is not used (the states are binned in line), and the recompute
-  // sorts.  What a budget has no room or use for is given back.
-  size_t room = s->roll_budget == 0 ? SIZE_MAX
-                : overlap           ? s->roll_budget - ((size_t(nseg) + 2 * size_t(k - 1)) * S + store_bytes)
-                                    : s->roll_budget - std::min(s->roll_budget, (size_t(nseg) + size_t(k - 1)) * S);
   if (bins && branch) {
-    CKS(further_bins(s, s->binsB, &room));
     use_bins(s->bB, s->binsB, dim, s->b.tile_edge, s->hp.n_tiles, nullptr);
     branch = s->bB.bin_ctl != nullptr;
-  } else if (s->roll_budget != 0) {
-    CKS(give_up_bins(s, s->binsB));
   }
-  if (bins && overlap) {
-    CKS(further_bins(s, s->bins2, &room));
-    use_bins(s->b2, s->bins2, dim, s->b.tile_edge, s->hp.n_tiles, s->sorted2);
-  } else if (s->roll_budget != 0) {
-    CKS(give_up_bins(s, s->bins2));
-  }
+  if (bins && overlap) use_bins(s->b2, s->bins2, dim, s->b.tile_edge, s->hp.n_tiles, s->sorted2);
   if (s->graphs_ws2 != overlap || s->graphs_branch != branch) {
     drop_reverse_graphs(s);
     s->graphs_ws2 = overlap;
@@ -1765,15 +1765,18 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
     return st;
   };
   mpm_status st = MPM_OK;
-#define ALLOC(ptr, n)                              \
-  do {                                             \
-    st = dalloc(&(ptr), size_t(n), s->allocs);     \
-    if (st != MPM_OK) return fail(st);             \
-  } while (0)
+// the bins are what the scene can do without: until b names them they yield to an allocation that finds
+// no memory
 #define TRY(expr)                                  \
   do {                                             \
-    if ((st = (expr)) != MPM_OK) return fail(st);  \
+    st = (expr);                                   \
+    if (st == MPM_ERR_OOM && s->bins.mem) {        \
+      drop_bins(c, s->bins);                       \
+      st = (expr);                                 \
+    }                                              \
+    if (st != MPM_OK) return fail(st);             \
   } while (0)
+#define ALLOC(ptr, n) TRY(dalloc(&(ptr), size_t(n), s->allocs))
   ALLOC(s->state, size_t(PL) * s->npad);
   ALLOC(s->adj[0], size_t(PL) * s->npad);
   ALLOC(s->adj[1], size_t(PL) * s->npad);
@@ -1850,6 +1853,10 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   b.n_active = s->d_status + 1;
   ALLOC(b.block_sums, 2 * ((p.n_tiles + 2047) / 2048) + 2);
   ALLOC(b.work, 4);
+  if (s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES) {
+    st = take_bins(c, s->bins, bin_set_bytes(dim, edge, p.n_tiles));
+    if (st != MPM_OK) return fail(st);
+  }
   if (s->impl == MPM_IMPL_TILED) {
     ALLOC(b.partial, size_t(p.n_tiles) * NB);
     ALLOC(b.partial_b, size_t(p.n_tiles) * NB);
@@ -1961,15 +1968,12 @@ mpm_status mpm_scene_create(mpm_ctx* c, const mpm_scene_desc* d, mpm_scene** out
   TRY(upload_table(s, 0, t0));
   s->hsel[PH_STEP].table = s->tables[0].dev;
   TRY(upload_sel(s));
-  ALLOC(b.sorted, s->npad);
-  // bins last: they are what the scene can do without
-  if (s->impl == MPM_IMPL_TILED && p.n_tiles <= BIN_TILES)
-    TRY(take_bins(c, s->bins, bin_set_bytes(dim, edge, p.n_tiles)));
+  if (!s->bins.mem) ALLOC(b.sorted, s->npad);
   use_bins(b, s->bins, dim, edge, p.n_tiles, b.sorted);
   b.rec_flip = s->bins.mem ? 1 : 0;
-  TRY(tune_init(s));
-  TRY(enqueue_keys(s, PH_STEP, stream));
-  TRY(read_status(s));
+  if ((st = tune_init(s)) != MPM_OK) return fail(st);
+  if ((st = enqueue_keys(s, PH_STEP, stream)) != MPM_OK) return fail(st);
+  if ((st = read_status(s)) != MPM_OK) return fail(st);
 #undef ALLOC
 #undef TRY
   *out = s;

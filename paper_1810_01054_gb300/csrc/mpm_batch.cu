@@ -184,13 +184,21 @@ mpm_status grow(mpm_batch* B, SubBatch& sb, int n_scenes, int tiles, int particl
   CK(cudaMalloc(&sb.b.work, sizeof(uint32_t) * 4));
   CK(cudaMemsetAsync(sb.b.work, 0, sizeof(uint32_t) * 4, B->ctx->stream));
   CK(cudaMalloc(&sb.sorted, sizeof(uint32_t) * pc));
-  CK(cudaMalloc(&sb.b.gpartial, sizeof(float) * size_t(tl) * MAX_GROUPS));
+  // the bins are what the batch can do without: they yield to what follows
+  CKS(take_bins(B->ctx, sb.bins, bin_set_bytes(B->dim, B->edge, std::min(tl, BIN_TILES))));
+  auto get = [&](auto** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (sb.bins.mem && out_of_memory(e)) {
+      drop_bins(B->ctx, sb.bins);
+      e = cudaMalloc(p, bytes);
+    }
+    return e;
+  };
+  CK(get(&sb.b.gpartial, sizeof(float) * size_t(tl) * MAX_GROUPS));
   CK(cudaMemsetAsync(sb.b.tile_count, 0, sizeof(uint32_t) * tl, B->ctx->stream));
   CK(cudaMemsetAsync(sb.b.tile_fill, 0, sizeof(uint32_t) * tl, B->ctx->stream));
-  CK(cudaMalloc(&sb.partial, sizeof(float4) * size_t(tl) * block_nodes(B->dim, B->edge)));
-  CK(cudaMalloc(&sb.partial_b, sizeof(float4) * size_t(tl) * block_nodes(B->dim, B->edge)));
-  // bins last: they are what the batch can do without
-  CKS(take_bins(B->ctx, sb.bins, bin_set_bytes(B->dim, B->edge, std::min(tl, BIN_TILES))));
+  CK(get(&sb.partial, sizeof(float4) * size_t(tl) * block_nodes(B->dim, B->edge)));
+  CK(get(&sb.partial_b, sizeof(float4) * size_t(tl) * block_nodes(B->dim, B->edge)));
   sb.bin_tiles = sb.bins.mem ? std::min(tl, BIN_TILES) : 0;
   sb.cap_scenes = sc;  // only now: after a failed allocation the next call starts over
   sb.cap_tiles = tl;
